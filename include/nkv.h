@@ -21,7 +21,7 @@
  *     0-based.  All pointers in nkv_tensor and all array arguments are DEVICE
  *     pointers unless an argument says "host".  Strides are in elements; d is
  *     contiguous, stride_n must equal d, every row start is 16-byte aligned.
- *     d is 64 or 128, dtype bf16, fp16 or fp32 (fp16 keys run the FMA form of the key passes), 2 <= window <= 64 (with a window of one key the
+ *     d is 64 or 128, dtype bf16, fp16 or fp32, 2 <= window <= 64 (with a window of one key the
  *     current anchor is the key itself and that scale carries no information).
  *   - Every buffer is caller-owned.  No entry point except nkv_create,
  *     nkv_destroy and nkv_compress_host allocates, frees or synchronises; work
@@ -260,14 +260,13 @@ NKV_API int64_t nkv_launch_count(const nkv_handle* h);
  * first pass yields 1/||k||, the block sums of normalised keys and the current-memory anomaly a_c; the
  * second, which needs the anchors of the whole head, the anomalies a_s and a_e.
  *   NKV_KEY_PASS_FMA     both passes with fp32 FMAs on staged key tiles (any supported dtype and d).
- *   NKV_KEY_PASS_TENSOR  (bf16 keys) forms on the tensor cores what is a contraction: in the first pass
- *       (d = 128, W = 64, one CTA per head) k_hat_i . S_i and ||S_i||^2 as sums over a band of the keys'
- *       Gram matrix, and ||k_i||^2 as its diagonal; in the second pass (d = 64 or 128) the dots of the keys with the anchors, the fp32
- *       anchors split three ways into bf16.  A pass whose inputs do not allow the tensor form runs the
- *       FMA kernel.
- *   NKV_KEY_PASS_AUTO (default) takes the tensor form of the second pass when d = 128, and of the first
- *       pass when in addition the call's heads, dealt one per SM, keep at least 85 % of the SMs busy over
- *       the rounds that takes.
+ *   NKV_KEY_PASS_TENSOR  (bf16 and fp16 keys, W = 64, blocks of 128 keys or more) forms on the tensor cores what
+ *       is a contraction: in the first pass k_hat_i . S_i and ||S_i||^2 as sums over a band of the keys' Gram
+ *       matrix, and ||k_i||^2 as its diagonal; in the second pass the dots of the keys with the anchors, the
+ *       fp32 anchors split three ways into the keys' type.  A call whose inputs do not allow the tensor form runs
+ *       the FMA kernels.
+ *   NKV_KEY_PASS_AUTO (default) takes the tensor form of the first pass where its inputs allow it, and of the
+ *       second when in addition d = 128 or the FMA form does not take the block size.
  * The forms agree to fp32 rounding.
  */
 enum { NKV_KEY_PASS_AUTO = 0, NKV_KEY_PASS_FMA = 1, NKV_KEY_PASS_TENSOR = 2 };

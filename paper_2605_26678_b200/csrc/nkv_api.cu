@@ -187,46 +187,34 @@ template <typename Mark>
 int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreParams& sp, const Bufs& B, int* status,
              cudaStream_t st, Mark&& mark) {
     const int units = G * kv.H, N = kv.N, d = kv.d;
-    if (stream_path_supported(sp)) {
-        // pass A: norms, block sums and the current-memory anomaly; pass B: the two anchor anomalies
-        // the tensor-core form walks whole heads, one CTA each: by default it runs when the heads fill
-        // the SMs to at least 85 % over its waves (below that the FMA form, which splits heads, is faster)
-        const int waves = (units + h->sm_count - 1) / h->sm_count;
-        const bool fills = (double)units >= 0.85 * (double)waves * (double)h->sm_count;
-        const bool tensor_ok = h->key_pass != NKV_KEY_PASS_FMA && gram_pass_supported(kv, dtype, sp) &&
-                               (h->key_pass == NKV_KEY_PASS_TENSOR || fills);
-        if (tensor_ok)
-            CU(launch_gram_pass(kv, G, sp, B.mu_e, B.inv_norm, B.a_raw,
-                                B.mm, status, h->sm_count, st, &h->launches));
-        else
-            CU(launch_stream_a(kv, dtype, G, sp, B.mu_e, B.inv_norm,
-                               B.a_raw, B.mm, status, h->sm_count, st,
-                               &h->launches));
-        CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
-        CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s,
-                               B.inv_e, nullptr, st, &h->launches));
-        CU(mark());
-        // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
-        const bool dots_wanted = h->key_pass == NKV_KEY_PASS_TENSOR || (h->key_pass == NKV_KEY_PASS_AUTO && d == 128);
-        if (dots_wanted && anchor_dots_supported(kv, dtype, sp))
-            CU(launch_anchor_dots(kv, G, sp, B.mu_s, B.mu_e, B.inv_norm,
-                                  B.inv_s, B.inv_e, B.a_raw,
-                                  B.mm, status, h->sm_count, st, &h->launches));
-        else
-            CU(launch_stream_b(kv, dtype, G, sp, B.mu_s, B.mu_e,
-                               B.inv_norm, B.inv_s, B.inv_e,
-                               B.a_raw, B.mm, status, h->sm_count, st,
-                               &h->launches));
-    } else {
+    const bool tensor_a = h->key_pass != NKV_KEY_PASS_FMA && gram_pass_supported(kv, dtype, sp) &&
+                          anchor_dots_supported(kv, dtype, sp);
+    if (!tensor_a && !stream_path_supported(sp)) {
         CU(launch_anchor_sums(kv, dtype, G, sp, B.mu_e, B.inv_norm, st, &h->launches));
         CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
-        CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s,
-                               B.inv_e, B.mm, st, &h->launches));
+        CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, B.mm, st, &h->launches));
         CU(mark());
-        CU(launch_scan_scores(kv, dtype, G, sp, B.mu_s, B.mu_e,
-                              B.inv_norm, B.inv_s, B.inv_e,
-                              B.a_raw, B.mm, st, &h->launches));
+        CU(launch_scan_scores(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, st,
+                              &h->launches));
+        return NKV_OK;
     }
+    // pass A: norms, block sums and the current-memory anomaly; pass B: the two anchor anomalies
+    if (tensor_a)
+        CU(launch_gram_pass(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
+    else
+        CU(launch_stream_a(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
+    CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
+    CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, nullptr, st, &h->launches));
+    CU(mark());
+    // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
+    const bool tensor_b = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
+                          (h->key_pass == NKV_KEY_PASS_TENSOR || d == 128 || !stream_path_supported(sp));
+    if (tensor_b)
+        CU(launch_anchor_dots(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, status, h->sm_count,
+                              st, &h->launches));
+    else
+        CU(launch_stream_b(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, status, h->sm_count, st,
+                           &h->launches));
     return NKV_OK;
 }
 

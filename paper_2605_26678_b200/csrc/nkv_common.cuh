@@ -131,16 +131,16 @@ cudaError_t launch_stream_b(const TensorView& K, int dtype, int G, const ScorePa
                             const float* mu_e, const float* inv_norm, const float* inv_s, const float* inv_e,
                             float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
                             int64_t* launches);
-// first key pass on the tensor cores (bf16 keys, d = 128): same outputs as launch_stream_a
+// first key pass on the tensor cores (16-bit keys): same outputs as launch_stream_a
 bool gram_pass_supported(const TensorView& K, int dtype, const ScoreParams& sp);
 cudaError_t configure_gram_kernels();
-cudaError_t launch_gram_pass(const TensorView& K, int G, const ScoreParams& sp, float* block_sums, float* inv_norm,
+cudaError_t launch_gram_pass(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums, float* inv_norm,
                              float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
                              int64_t* launches);
-// second key pass on the tensor cores (bf16 keys, d = 128): same outputs as launch_stream_b
+// second key pass on the tensor cores (16-bit keys): same outputs as launch_stream_b
 bool anchor_dots_supported(const TensorView& K, int dtype, const ScoreParams& sp);
 cudaError_t configure_dots_kernels();
-cudaError_t launch_anchor_dots(const TensorView& K, int G, const ScoreParams& sp, const float* mu_s, const float* mu_e,
+cudaError_t launch_anchor_dots(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* mu_s, const float* mu_e,
                                const float* inv_norm, const float* inv_s, const float* inv_e, float* a_raw,
                                uint32_t* mm, int* status, int sm_count, cudaStream_t stream, int64_t* launches);
 cudaError_t configure_select_kernels();

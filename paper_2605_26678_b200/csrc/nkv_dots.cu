@@ -1,9 +1,11 @@
-// Second key pass on the tensor cores (bf16 keys, d = 64 or 128): a_s(i) = -cos(k_hat_i, mu_s) and
+// Second key pass on the tensor cores (bf16 or fp16 keys, d = 64 or 128): a_s(i) = -cos(k_hat_i, mu_s) and
 // a_e(i) = -cos(k_hat_i, mu_e(block of i)) with their per-head min/max (Section 2.3).
 //
 // The dots of 128 keys with the anchors are one skinny product [128 x d] x [d x 16] per tile.  The fp32
-// anchors enter as three bf16 columns each (hi + mid + lo carries all 24 mantissa bits; products of bf16
-// numbers are exact in fp32 and tcgen05.mma accumulates in fp32), so a tile's right-hand side is
+// anchors enter as three columns of the keys' type each (hi + mid + lo carries all 24 mantissa bits; products of
+// 16-bit numbers are exact in fp32 and tcgen05.mma accumulates in fp32; for fp16 the anchors, means of unit
+// vectors, are scaled by 2^10, which brings lo's quantum to 2^-34 of the anchors' scale), so a tile's right-hand
+// side is
 //     columns 0..2  mu_s        3..5  mu_e of the block the tile starts in        6..8  mu_e of the next block
 // (a tile of 128 keys touches at most two blocks because a block has at least 128 keys).  Key tiles are
 // staged by TMA (128-byte swizzle) several tiles ahead; the tensor core reads them from shared memory
@@ -93,11 +95,11 @@ __device__ void dots_producer(const CUtensorMap* tmap, unsigned char* tiles, Sme
     }
 }
 
-template <int D>
+template <typename T, int D>
 __device__ void dots_mma(unsigned char* tiles, unsigned char* rhs, Smem* s, uint32_t tmem_base, TileRange tr,
                          int* status) {
     using C = Cfg<D>;
-    constexpr uint32_t idesc = umma_idesc_bf16(kTile, 16);
+    constexpr uint32_t idesc = umma_idesc<T>(kTile, 16);
     const uint32_t tiles_addr = smem_addr(tiles), rhs_addr = smem_addr(rhs);
     long long n = 0;
     for (long long t = tr.first; t < tr.last; ++t, ++n) {
@@ -118,7 +120,7 @@ __device__ void dots_mma(unsigned char* tiles, unsigned char* rhs, Smem* s, uint
                                (uint32_t)(kk & 3) * 32u;
             const uint32_t b = rhs_addr + (uint32_t)slot * C::kRhsBytes + (uint32_t)(kk >> 2) * kRhsHalfBytes +
                                (uint32_t)(kk & 3) * 32u;
-            umma_bf16(tmem_base + (uint32_t)stage * 32u, umma_desc_sw128(a), umma_desc_sw128(b), idesc, kk > 0);
+            umma_f16(tmem_base + (uint32_t)stage * 32u, umma_desc_sw128(a), umma_desc_sw128(b), idesc, kk > 0);
         }
         umma_commit(&s->tfull[stage]);
         umma_commit(&s->kfree[slot]);
@@ -126,7 +128,14 @@ __device__ void dots_mma(unsigned char* tiles, unsigned char* rhs, Smem* s, uint
 }
 
 // Thread k writes column k of the nine right-hand-side rows of every tile (rows 9..15 stay zero).
-template <int D>
+template <typename T> constexpr float kAnchorScale = 1.f;
+template <> constexpr float kAnchorScale<__half> = 1024.f;
+template <typename T> __device__ __forceinline__ T narrow(float v);
+template <> __device__ __forceinline__ __nv_bfloat16 narrow<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
+template <> __device__ __forceinline__ __half narrow<__half>(float v) { return __float2half_rn(v); }
+template <typename T> __device__ __forceinline__ float widen(T v) { return (float)v; }
+
+template <typename T, int D>
 __device__ void dots_prep(unsigned char* rhs, Smem* s, ScoreParams sp, TileRange tr, const float* __restrict__ mu_s,
                           const float* __restrict__ mu_e, int* status) {
     using C = Cfg<D>;
@@ -153,15 +162,16 @@ __device__ void dots_prep(unsigned char* rhs, Smem* s, ScoreParams sp, TileRange
         unsigned char* base = rhs + (size_t)slot * C::kRhsBytes + (size_t)half * kRhsHalfBytes + (kk & 7) * 2;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const __nv_bfloat16 hi = __float2bfloat16_rn(v[a]);
-            const float r1 = v[a] - __bfloat162float(hi);
-            const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-            const __nv_bfloat16 part[3] = {hi, mid, lo};
+            const float x = v[a] * kAnchorScale<T>;
+            const T hi = narrow<T>(x);
+            const float r1 = x - widen(hi);
+            const T mid = narrow<T>(r1);
+            const T lo = narrow<T>(r1 - widen(mid));
+            const T part[3] = {hi, mid, lo};
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 const int row = 3 * a + j;   // row of the right-hand side, 8-row groups 1024 bytes apart
-                *reinterpret_cast<__nv_bfloat16*>(base + (row >> 3) * 1024 + (row & 7) * 128 +
+                *reinterpret_cast<T*>(base + (row >> 3) * 1024 + (row & 7) * 128 +
                                                   ((((kk >> 3) ^ (row & 7))) << 4)) = part[j];
             }
         }
@@ -172,6 +182,7 @@ __device__ void dots_prep(unsigned char* rhs, Smem* s, ScoreParams sp, TileRange
 }
 
 // Thread r reads row r of the accumulator: the key's dots with mu_s and with the two candidate mu_e.
+template <typename T>
 __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileRange tr, int N,
                               const float* __restrict__ inv_norm, const float* __restrict__ inv_s,
                               const float* __restrict__ inv_e, float* __restrict__ a_raw, uint32_t* __restrict__ mm,
@@ -235,8 +246,9 @@ __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileR
         if (lane == 0) mbar_arrive(&s->tempty[stage]);
         const float ds = d[0] + d[1] + d[2];
         const float de = cur.second ? d[6] + d[7] + d[8] : d[3] + d[4] + d[5];
-        const float a_s = -(ds * cur.inv_i) * rs + 0.f;
-        const float a_e = -(de * cur.inv_i) * cur.re + 0.f;
+        const float scaled = cur.inv_i * (1.f / kAnchorScale<T>);
+        const float a_s = -(ds * scaled) * rs + 0.f;
+        const float a_e = -(de * scaled) * cur.re + 0.f;
         if (cur.i < N) {
             a_raw[((int64_t)cur.u * 3 + 0) * N + cur.i] = a_s;
             a_raw[((int64_t)cur.u * 3 + 1) * N + cur.i] = a_e;
@@ -249,7 +261,7 @@ __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileR
     flush();
 }
 
-template <int D>
+template <typename T, int D>
 __global__ void __launch_bounds__(kThreads, 1)
 anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int units, int H, int N,
                    const float* __restrict__ mu_s, const float* __restrict__ mu_e, const float* __restrict__ inv_norm,
@@ -288,12 +300,12 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
         if (lane == 0) dots_producer<D>(&tmap, tiles, s, tr, H, status);
         __syncwarp();
     } else if (warp == kMmaWarp) {
-        if (lane == 0) dots_mma<D>(tiles, rhs, s, tmem_base, tr, status);
+        if (lane == 0) dots_mma<T, D>(tiles, rhs, s, tmem_base, tr, status);
         __syncwarp();
     } else if (warp >= kEpiWarp0) {
-        dots_epilogue(s, tmem_base, sp, tr, N, inv_norm, inv_s, inv_e, a_raw, mm, status);
+        dots_epilogue<T>(s, tmem_base, sp, tr, N, inv_norm, inv_s, inv_e, a_raw, mm, status);
     } else {
-        dots_prep<D>(rhs, s, sp, tr, mu_s, mu_e, status);
+        dots_prep<T, D>(rhs, s, sp, tr, mu_s, mu_e, status);
     }
 
     tc_fence_before();
@@ -304,39 +316,51 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
 }  // namespace
 
 cudaError_t configure_dots_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(anchor_dots_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes<64>());
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(anchor_dots_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_bytes<128>());
+    cudaError_t e;
+#define NKV_SET(T, D)                                                                                                    \
+    if ((e = cudaFuncSetAttribute(anchor_dots_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,                 \
+                                  (int)smem_bytes<D>())) != cudaSuccess)                                                  \
+        return e
+    NKV_SET(__nv_bfloat16, 64);
+    NKV_SET(__nv_bfloat16, 128);
+    NKV_SET(__half, 64);
+    NKV_SET(__half, 128);
+#undef NKV_SET
+    return cudaSuccess;
 }
 
-// bf16 keys of 64 or 128 columns, strides a tensor map accepts, and blocks of at least 128 keys (a tile
+// 16-bit keys of 64 or 128 columns, strides a tensor map accepts, and blocks of at least 128 keys (a tile
 // of 128 keys then touches at most two blocks).
 bool anchor_dots_supported(const TensorView& K, int dtype, const ScoreParams& sp) {
-    if (dtype != NKV_BF16 || (K.d != 64 && K.d != 128) || sp.block < kTile) return false;
+    if ((dtype != NKV_BF16 && dtype != NKV_F16) || (K.d != 64 && K.d != 128) || sp.block < kTile) return false;
     if (reinterpret_cast<uintptr_t>(K.ptr) % 16 != 0) return false;
     if (K.stride_h % 8 != 0 || K.stride_g % 8 != 0) return false;
     if (K.stride_h < (int64_t)K.N * K.d || K.stride_g < (int64_t)K.N * K.d) return false;
     CUtensorMap probe;   // the driver has the last word on what a tensor map can describe
-    return encode_key_map(K, 1, kTile, &probe) == cudaSuccess;
+    return encode_key_map(K, dtype, 1, kTile, &probe) == cudaSuccess;
 }
 
-cudaError_t launch_anchor_dots(const TensorView& K, int G, const ScoreParams& sp, const float* mu_s, const float* mu_e,
-                               const float* inv_norm, const float* inv_s, const float* inv_e, float* a_raw,
-                               uint32_t* mm, int* status, int sm_count, cudaStream_t stream, int64_t* launches) {
+cudaError_t launch_anchor_dots(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* mu_s,
+                               const float* mu_e, const float* inv_norm, const float* inv_s, const float* inv_e,
+                               float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
+                               int64_t* launches) {
     CUtensorMap tmap;
-    cudaError_t e = encode_key_map(K, G, kTile, &tmap);
+    cudaError_t e = encode_key_map(K, dtype, G, kTile, &tmap);
     if (e != cudaSuccess) return e;
     const int units = G * K.H;
     const long long total = (long long)units * ((K.N + kTile - 1) / kTile);
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
-    if (K.d == 128)
-        anchor_dots_kernel<128><<<grid, kThreads, smem_bytes<128>(), stream>>>(tmap, sp, units, K.H, K.N, mu_s, mu_e,
-                                                                               inv_norm, inv_s, inv_e, a_raw, mm, status);
-    else
-        anchor_dots_kernel<64><<<grid, kThreads, smem_bytes<64>(), stream>>>(tmap, sp, units, K.H, K.N, mu_s, mu_e,
-                                                                             inv_norm, inv_s, inv_e, a_raw, mm, status);
+#define NKV_DOTS(T, D)                                                                                                \
+    anchor_dots_kernel<T, D><<<grid, kThreads, smem_bytes<D>(), stream>>>(tmap, sp, units, K.H, K.N, mu_s, mu_e,     \
+                                                                          inv_norm, inv_s, inv_e, a_raw, mm, status)
+    if (dtype == NKV_BF16) {
+        if (K.d == 128) NKV_DOTS(__nv_bfloat16, 128);
+        else NKV_DOTS(__nv_bfloat16, 64);
+    } else {
+        if (K.d == 128) NKV_DOTS(__half, 128);
+        else NKV_DOTS(__half, 64);
+    }
+#undef NKV_DOTS
     ++*launches;
     return cudaGetLastError();
 }

@@ -8,8 +8,8 @@
 
 namespace nkv {
 
-// Tensor map of bf16 keys [G][H][N][128] for boxes of 64 columns x box_rows rows, 128-byte swizzle (host).
-cudaError_t encode_key_map(const TensorView& K, int G, int box_rows, CUtensorMap* out);
+// Tensor map of bf16 or fp16 keys [G][H][N][d] for boxes of 64 columns x box_rows rows, 128-byte swizzle (host).
+cudaError_t encode_key_map(const TensorView& K, int dtype, int G, int box_rows, CUtensorMap* out);
 
 namespace sm100 {
 
@@ -77,6 +77,11 @@ __device__ __forceinline__ void tma_load_4d(void* dst_smem, const CUtensorMap* m
         "[%6];" ::"r"(smem_addr(dst_smem)),
         "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_addr(bar))
         : "memory");
+}
+__device__ __forceinline__ uint64_t l2_evict_normal_policy() {
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+    return policy;
 }
 // The same with an L2 cache policy.  Keys are read once per pass and are far larger than L2: marking their lines
 // "evict first" leaves L2 to what is read again (anchors, weights, the scores written for the next kernel).
@@ -184,12 +189,15 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t addr) {
     d |= (uint64_t)2 << 61;                     // 128-byte swizzle
     return d;
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, tile M x N.
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor: bf16 x bf16 or fp16 x fp16 -> fp32, both operands K-major, tile M x N.
+template <typename T> constexpr uint32_t kOperandType = 1u;            // bf16
+template <> inline constexpr uint32_t kOperandType<__half> = 0u;
+template <typename T>
+__host__ __device__ constexpr uint32_t umma_idesc(int M, int N) {
+    return (1u << 4) | (kOperandType<T> << 7) | (kOperandType<T> << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           bool accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
@@ -225,12 +233,21 @@ __device__ __forceinline__ float hsum2(F2 x) {
     unpack2(x, a, b);
     return a + b;
 }
-// eight bf16 values of a 16-byte chunk as four fp32 pairs
-__device__ __forceinline__ void unpack_bf16x8(const uint4& q, F2* p) {
+// eight 16-bit values of a 16-byte chunk as four fp32 pairs
+template <typename T> __device__ __forceinline__ void unpack8(const uint4& q, F2* p);
+template <> __device__ __forceinline__ void unpack8<__nv_bfloat16>(const uint4& q, F2* p) {
     p[0] = pack2(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u));
     p[1] = pack2(__uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
     p[2] = pack2(__uint_as_float(q.z << 16), __uint_as_float(q.z & 0xffff0000u));
     p[3] = pack2(__uint_as_float(q.w << 16), __uint_as_float(q.w & 0xffff0000u));
+}
+template <> __device__ __forceinline__ void unpack8<__half>(const uint4& q, F2* p) {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
+        p[j] = pack2(f.x, f.y);
+    }
 }
 
 }  // namespace sm100

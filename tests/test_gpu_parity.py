@@ -464,3 +464,32 @@ def test_random_shapes_end_to_end(seed):
         swaps += rep.swapped_tokens
         heads += rep.heads
     assert swaps <= max(4, heads // 50)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,layers,N,d,dtype", [
+    (1, 1, 65, 128, "bf16"), (2, 1, 129, 64, "fp16"), (8, 40, 300, 128, "bf16"),   # many heads per SM, spans that cut them
+    (3, 1, 6000, 64, "bf16"), (3, 1, 6000, 128, "fp16"),       # blocks of 187 keys
+    (2, 1, 7937, 128, "bf16"), (2, 1, 8193, 64, "fp16"),       # a last block of one key
+    (1, 1, 40000, 128, "bf16")])                               # every SM starts inside the head
+def test_tensor_first_pass_edges(H, layers, N, d, dtype):
+    """The tensor-core key passes at the edges of tiles, blocks and the shares of the SMs, against the FMA kernels'
+    definition of the same quantities in the oracle (first and last head of the call)."""
+    K, _ = _cache(N, d, dtype, H=H, layers=layers)
+    p = nkv.nkv_default_params()
+    ws = nkv.alloc_workspace(K, p)
+    nkv.nkv_set_key_passes("tensor")
+    try:
+        got = nkv.nkv_key_scan(K, p, ws=ws)
+    finally:
+        nkv.nkv_set_key_passes("auto")
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    for g, h in {(0, 0), (layers - 1, H - 1)}:
+        ref = oracle.score_head(K[g, h].cpu())
+        inv_norm, mu_s, mu_e, a_raw, minmax = (x[g, h].cpu().numpy() for x in got)
+        pr.assert_close(inv_norm, ref.inv_norm, "inv_norm", 1e-5)
+        pr.assert_close(mu_s, ref.mu_s, "mu_s", 1e-5)
+        pr.assert_close(mu_e, ref.mu_e, "mu_e", 1e-5)
+        pr.assert_close(a_raw, ref.a_raw, "a_raw", 1e-5)
+        pr.assert_close(minmax[0::2], ref.lo, "lo", 1e-5)
+        pr.assert_close(minmax[1::2], ref.hi, "hi", 1e-5)
