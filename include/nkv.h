@@ -106,7 +106,8 @@ typedef struct nkv_handle nkv_handle;
  * min s, max s, mean of the min-max-normalised s, m (top/bottom count). */
 #define NKV_HEAD_STATS 16
 
-/* Stages whose device time nkv_compress records when timing is enabled. */
+/* Stages whose device time nkv_compress records when timing is enabled.  The head, budget and select stages run
+ * together; their time is recorded as the head stage's. */
 #define NKV_STAGE_ANCHORS 0
 #define NKV_STAGE_SCORE 1
 #define NKV_STAGE_HEAD 2
@@ -179,8 +180,7 @@ NKV_API int nkv_score(nkv_handle* h, const nkv_tensor* K, const float* mu_s, con
  *   thresholds_opt  out f32 [G,H] or NULL: the head's selection threshold: the head retains every token that
  *            scores above it and, in position order, as many of the tokens that score exactly it as its
  *            budget still allows (+inf while the sinks alone fill the head's budget)
- *   ws       at least 256 + 8*G*H bytes (rounded up to 256); with 8192*G*H + 42000*G bytes more, large calls
- *            spread the cross-head competition of a group over many thread blocks (same result)
+ *   ws       at least 256 + 8*G*H bytes (rounded up to 256)
  */
 NKV_API int nkv_budget(nkv_handle* h, const float* a_star, int64_t G, int64_t H, int64_t N, double r,
                const nkv_params* params, int32_t* budgets, float* thresholds_opt, void* ws, size_t ws_bytes,
@@ -308,8 +308,7 @@ NKV_API int nkv_debug_wait_probe(nkv_handle* h, int64_t polls, void* ws, size_t 
  * same kernel).  A host that runs inside a memory pool fixed at start-up, a
  * plugin that receives nothing but its inputs and outputs, or a step that runs
  * while the process may not grow its footprint has no scratch buffer to hand
- * to nkv_budget.  Here the scratch (status words and the per-head selection
- * thresholds, 256 + 8 * NKV_STATIC_MAX_UNITS bytes) is a fixed array inside
+ * to nkv_budget.  Here the scratch (status words, 256 bytes) is a fixed array inside
  * the library image; every GPU that loads the library holds it until the
  * process exits.  No handle and no workspace are needed, and the call makes no
  * cudaMalloc, cudaFree or other allocating call.
@@ -318,9 +317,8 @@ NKV_API int nkv_debug_wait_probe(nkv_handle* h, int64_t polls, void* ws, size_t 
  *   nothing is launched (use nkv_budget with your own workspace instead).
  * The first call made with a given device current looks up the array's device
  * address (once per device); make that first call before any stream capture.
- * All calls on a device share the one array, which still holds what the last
- * call left: the status words are cleared on the stream at the start of each
- * call, the threshold slots of the call's G * H heads are all rewritten.  Two
+ * All calls on a device share the one array, whose status words are cleared on
+ * the stream at the start of each call.  Two
  * calls whose work overlaps on the GPU (different streams) race on the array:
  * keep calls on one device ordered.  Device-side self-check results are not
  * readable through this entry point.

@@ -60,10 +60,13 @@ int64_t keep_count(int64_t N, double r) { return (int64_t)floor((1.0 - r) * (dou
 
 // Workspace carving shared by every entry point.
 struct Layout {
-    size_t status, inv_norm, mu_s, mu_e, inv_s, inv_e, mm, a_raw, a_star, thr, hstat, bscr, total;
+    size_t status, mm, inv_norm, mu_s, mu_e, inv_s, inv_e, a_raw, a_star, total;
 };
 
-Layout make_layout(int64_t G, int64_t units, int64_t N, int64_t d, int64_t nb) {
+// Rows of the per-token arrays start on 16-byte boundaries, so that ragged lengths keep the four-wide accesses.
+int64_t padded_row(int64_t N) { return (N + 3) & ~(int64_t)3; }
+
+Layout make_layout(int64_t units, int64_t N, int64_t d, int64_t nb) {
     Layout L;
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -71,21 +74,20 @@ Layout make_layout(int64_t G, int64_t units, int64_t N, int64_t d, int64_t nb) {
         o += align_up(bytes);
         return at;
     };
+    const size_t row = (size_t)padded_row(N) * 4;
     L.status = take(kStatusWords * sizeof(int));
-    L.inv_norm = take((size_t)units * N * 4);
+    L.mm = take((size_t)units * 6 * 4);      // cleared together with the status words in front of it
+    L.inv_norm = take((size_t)units * row);
     L.mu_s = take((size_t)units * d * 4);
     L.mu_e = take((size_t)units * nb * d * 4);
     L.inv_s = take((size_t)units * 4);
     L.inv_e = take((size_t)units * nb * 4);
-    L.mm = take((size_t)units * 6 * 4);
-    L.a_raw = take((size_t)units * 3 * N * 4);
-    L.a_star = take((size_t)units * N * 4);
-    L.thr = take((size_t)units * 2 * 4);
-    L.hstat = take(head_stat_bytes(units));
-    L.bscr = take(budget_scratch_bytes(G, units / G));   // the heads per group divide the units
+    L.a_raw = take((size_t)units * 3 * row);
+    L.a_star = take((size_t)units * row);
     L.total = o;
     return L;
 }
+size_t cleared_bytes(const Layout& L, int64_t units) { return L.mm + (size_t)units * 6 * 4; }
 
 int check_tensor(const nkv_tensor* t) {
     if (!t || !t->ptr) return NKV_ERR_INVALID_ARG;
@@ -134,6 +136,7 @@ int resolve_params(const nkv_params* p, int64_t N, ScoreParams* sp) {
     sp->beta = (float)p->beta;
     sp->tau = (float)p->tau;
     sp->kappa = (float)p->kappa;
+    sp->raw_row = sp->inv_row = padded_row(N);   // in the workspace
     return NKV_OK;
 }
 
@@ -158,30 +161,25 @@ int cuda_failed(cudaError_t e, const char* what, int line) {
         if (e__ != cudaSuccess) return cuda_failed(e__, #expr, __LINE__); \
     } while (0)
 
-// The workspace arrays of a run of groups that starts at group g0 (unit u0 = g0 * H).
+// The workspace arrays of the key passes.
 struct Bufs {
-    float *inv_norm, *mu_s, *mu_e, *inv_s, *inv_e, *a_raw, *hstat;
-    uint32_t *mm, *thr;
-    unsigned char* bscr;
+    float *inv_norm, *mu_s, *mu_e, *inv_s, *inv_e, *a_raw;
+    uint32_t* mm;
 };
-Bufs bufs_at(void* ws, const Layout& L, int64_t g0, int64_t H, int64_t N, int64_t d, int64_t nb) {
-    const int64_t u0 = g0 * H;
+Bufs bufs_at(void* ws, const Layout& L) {
     Bufs b;
-    b.inv_norm = at<float>(ws, L.inv_norm) + u0 * N;
-    b.mu_s = at<float>(ws, L.mu_s) + u0 * d;
-    b.mu_e = at<float>(ws, L.mu_e) + u0 * nb * d;
-    b.inv_s = at<float>(ws, L.inv_s) + u0;
-    b.inv_e = at<float>(ws, L.inv_e) + u0 * nb;
-    b.a_raw = at<float>(ws, L.a_raw) + u0 * 3 * N;
-    b.hstat = at<float>(ws, L.hstat) + head_stat_bytes(u0) / sizeof(float);
-    b.mm = at<uint32_t>(ws, L.mm) + u0 * 6;
-    b.thr = at<uint32_t>(ws, L.thr) + u0 * 2;
-    b.bscr = at<unsigned char>(ws, L.bscr) + (g0 ? budget_scratch_bytes(g0, H) : 0);   // every term is linear in G
+    b.inv_norm = at<float>(ws, L.inv_norm);
+    b.mu_s = at<float>(ws, L.mu_s);
+    b.mu_e = at<float>(ws, L.mu_e);
+    b.inv_s = at<float>(ws, L.inv_s);
+    b.inv_e = at<float>(ws, L.inv_e);
+    b.a_raw = at<float>(ws, L.a_raw);
+    b.mm = at<uint32_t>(ws, L.mm);
     return b;
 }
 
 // The two passes over the keys (Sections 2.1-2.3): afterwards the workspace holds 1/||k||, the anchors, the
-// three raw anomalies and their per-head min/max keys.  `mark` is called once between the passes (stage
+// three raw anomalies and their per-head min/max keys (which start out cleared).  `mark` is called once between the passes (stage
 // timing).
 template <typename Mark>
 int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreParams& sp, const Bufs& B, int* status,
@@ -192,7 +190,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
     if (!tensor_a && !stream_path_supported(sp)) {
         CU(launch_anchor_sums(kv, dtype, G, sp, B.mu_e, B.inv_norm, st, &h->launches));
         CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
-        CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, B.mm, st, &h->launches));
+        CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, st, &h->launches));
         CU(mark());
         CU(launch_scan_scores(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, st,
                               &h->launches));
@@ -204,7 +202,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
     else
         CU(launch_stream_a(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
     CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
-    CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, nullptr, st, &h->launches));
+    CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, st, &h->launches));
     CU(mark());
     // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
     const bool tensor_b = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
@@ -221,7 +219,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
 // ordered min/max keys -> floats (lo_s, hi_s, lo_e, hi_e, lo_c, hi_c per head)
 __global__ void minmax_floats_kernel(int n, const uint32_t* keys, float* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = ord_float(keys[i]);
+    if (i < n) out[i] = ord_float((i & 1) ? keys[i] : ~keys[i]);
 }
 
 }  // namespace
@@ -353,7 +351,7 @@ int nkv_workspace_bytes(const nkv_handle* h, int64_t G, int64_t H, int64_t N, in
     (void)dtype;
     if (!h || !out_bytes || G < 1 || H < 1 || N < 1 || d < 1 || !params_ok(params)) return NKV_ERR_INVALID_ARG;
     const int64_t b = block_size(N, params);
-    *out_bytes = make_layout(G, G * H, N, d, (N + b - 1) / b).total;
+    *out_bytes = make_layout(G * H, N, d, (N + b - 1) / b).total;
     return NKV_OK;
 }
 
@@ -368,6 +366,7 @@ int nkv_anchors(nkv_handle* h, const nkv_tensor* K, const nkv_params* params, fl
     cudaStream_t st = (cudaStream_t)stream;
     const TensorView kv = view_of(K);
     const int units = (int)(K->G * K->H);
+    sp.inv_row = K->N;
     CU(launch_anchor_sums(kv, K->dtype, (int)K->G, sp, mu_e, inv_norm, st, &h->launches));
     CU(launch_anchor_means(units, (int)K->N, (int)K->d, sp, mu_e, mu_s, st, &h->launches));
     if (mu_c_opt) CU(launch_window_means(kv, K->dtype, (int)K->G, sp, inv_norm, mu_c_opt, st, &h->launches));
@@ -384,18 +383,20 @@ int nkv_score(nkv_handle* h, const nkv_tensor* K, const float* mu_s, const float
     ScoreParams sp;
     if ((rc = resolve_params(params, K->N, &sp))) return rc;
     const int units = (int)(K->G * K->H);
-    const Layout L = make_layout(K->G, units, K->N, K->d, sp.nblocks);
+    const Layout L = make_layout(units, K->N, K->d, sp.nblocks);
     if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const TensorView kv = view_of(K);
+    sp.inv_row = K->N;
+    if (a_raw_opt) sp.raw_row = K->N;
     float* a_raw = a_raw_opt ? a_raw_opt : at<float>(ws, L.a_raw);
-    CU(cudaMemsetAsync(at<int>(ws, L.status), 0, kStatusWords * sizeof(int), st));
-    CU(launch_anchor_norms(units, (int)K->d, sp, mu_s, mu_e, at<float>(ws, L.inv_s), at<float>(ws, L.inv_e),
-                           at<uint32_t>(ws, L.mm), st, &h->launches));
+    CU(cudaMemsetAsync(ws, 0, cleared_bytes(L, units), st));
+    CU(launch_anchor_norms(units, (int)K->d, sp, mu_s, mu_e, at<float>(ws, L.inv_s), at<float>(ws, L.inv_e), st,
+                           &h->launches));
     CU(launch_scan_scores(kv, K->dtype, (int)K->G, sp, mu_s, mu_e, inv_norm, at<float>(ws, L.inv_s),
                           at<float>(ws, L.inv_e), a_raw, at<uint32_t>(ws, L.mm), st, &h->launches));
     CU(launch_head_scores(units, (int)K->N, sp, a_raw, at<uint32_t>(ws, L.mm), a_star, head_stats_opt,
-                          at<float>(ws, L.hstat), at<int>(ws, L.status), st, &h->launches));
+                          at<int>(ws, L.status), st, &h->launches));
     return NKV_OK;
 }
 
@@ -408,17 +409,12 @@ int nkv_budget(nkv_handle* h, const float* a_star, int64_t G, int64_t H, int64_t
     const int64_t k = keep_count(N, r);
     if (k < 1 || k > N) return NKV_ERR_INVALID_ARG;
     const int64_t n_safe = nkv_safeguard_count(N, r, params);
-    const size_t thr_off = align_up(kStatusWords * sizeof(int));
-    int rc = check_ws(ws, ws_bytes, thr_off + align_up((size_t)G * H * 8));
+    int rc = check_ws(ws, ws_bytes, align_up(kStatusWords * sizeof(int)) + align_up((size_t)G * H * 8));
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     CU(cudaMemsetAsync(ws, 0, kStatusWords * sizeof(int), st));
-    const size_t scr_off = thr_off + align_up((size_t)G * H * 8);
-    void* scratch = ws_bytes >= scr_off + budget_scratch_bytes(G, H) ? at<unsigned char>(ws, scr_off) : nullptr;
-    CU(launch_budget((int)G, (int)H, (int)N, (int)k, (int)n_safe, a_star, budgets, at<uint32_t>(ws, thr_off),
-                     at<int>(ws, 0), scratch, st, &h->launches));
-    if (thresholds_opt)
-        CU(launch_threshold_scores((int)(G * H), at<uint32_t>(ws, thr_off), thresholds_opt, st, &h->launches));
+    CU(launch_budget((int)G, (int)H, (int)N, (int)k, (int)n_safe, a_star, budgets, thresholds_opt, at<int>(ws, 0), st,
+                     &h->launches));
     return NKV_OK;
 }
 
@@ -432,8 +428,8 @@ int nkv_select(nkv_handle* h, const float* a_star, const int32_t* budgets, int64
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     CU(cudaMemsetAsync(ws, 0, kStatusWords * sizeof(int), st));
-    CU(launch_select((int)G, (int)H, (int)N, idx_capacity, a_star, budgets, nullptr, idx, head_offsets,
-                     at<int>(ws, 0), st, &h->launches));
+    CU(launch_select((int)G, (int)H, (int)N, idx_capacity, a_star, budgets, idx, head_offsets, at<int>(ws, 0), st,
+                     &h->launches));
     if (ranks_opt) {
         if (G * H > 65535) return NKV_ERR_UNSUPPORTED;
         CU(launch_ranks((int)(G * H), (int)N, a_star, ranks_opt, st, &h->launches));
@@ -486,12 +482,13 @@ int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double
     const int64_t n_safe = nkv_safeguard_count(K->N, r, params);
     const int G = (int)K->G, H = (int)K->H, N = (int)K->N, d = (int)K->d;
     const int units = G * H;
-    const Layout L = make_layout(G, units, N, d, sp.nblocks);
+    const Layout L = make_layout(units, N, d, sp.nblocks);
     if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const TensorView kv = view_of(K), vv = view_of(V);
     const int kb = K->dtype == NKV_F32 ? 4 : 2, vb = V->dtype == NKV_F32 ? 4 : 2;
     float* a_star = a_star_opt ? a_star_opt : at<float>(ws, L.a_star);
+    const int64_t star_row = a_star_opt ? N : padded_row(N);
     int* status = at<int>(ws, L.status);
     const bool timing = h->timing != 0;
     int stage = 0;
@@ -500,42 +497,18 @@ int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double
         return cudaEventRecord(h->ev[stage++], st);
     };
 
-    CU(cudaMemsetAsync(status, 0, kStatusWords * sizeof(int), st));
+    CU(cudaMemsetAsync(ws, 0, cleared_bytes(L, units), st));
     CU(mark());
-    // One run of groups: the key scan on `ks`, everything after it on `ss`.
-    auto run = [&](int g0, int gc, cudaStream_t ks, cudaStream_t ss, cudaEvent_t scanned) -> int {
-        const Bufs B = bufs_at(ws, L, g0, H, N, d, sp.nblocks);
-        TensorView kc = kv, vc = vv;
-        kc.ptr = static_cast<const unsigned char*>(kv.ptr) + (size_t)g0 * kv.stride_g * kb;
-        vc.ptr = static_cast<const unsigned char*>(vv.ptr) + (size_t)g0 * vv.stride_g * vb;
-        float* as = a_star + (size_t)g0 * H * N;
-        int32_t* bud = budgets + (size_t)g0 * H;
-        int32_t* ix = idx + (size_t)g0 * H * keep;
-        int32_t* ho = head_offsets + (size_t)g0 * (H + 1);
-        int rc2 = key_scan(h, kc, K->dtype, gc, sp, B, status, ks, mark);
-        if (rc2) return rc2;
-        CU(mark());
-        if (ss != ks) {
-            CU(cudaEventRecord(scanned, ks));
-            CU(cudaStreamWaitEvent(ss, scanned, 0));
-        }
-        CU(launch_head_scores(gc * H, N, sp, B.a_raw, B.mm, as, nullptr, B.hstat, status, ss, &h->launches));
-        CU(mark());
-        CU(launch_budget(gc, H, N, (int)keep, (int)n_safe, as, bud, B.thr, status, B.bscr, ss, &h->launches));
-        CU(mark());
-        CU(launch_select(gc, H, N, (int64_t)H * keep, as, bud, B.thr, ix, ho, status, ss, &h->launches));
-        CU(mark());
-        CU(launch_gather(kc, kb, vc, vb, gc, ix, ho, (int64_t)H * keep,
-                         static_cast<unsigned char*>(K_out) + (size_t)g0 * H * keep * kv.d * kb,
-                         static_cast<unsigned char*>(V_out) + (size_t)g0 * H * keep * vv.d * vb, h->sm_count, ss,
-                         &h->launches));
-        CU(mark());
-        return NKV_OK;
-    };
-    // Running a call as two halves on two streams (the score side of one half beside the second key pass and
-    // the compaction of the other) measured no faster: the first key pass leaves no registers for a second
-    // kernel on its SMs, and beside the second pass the score kernels get a quarter of their CTAs.
-    if ((rc = run(0, G, st, st, nullptr))) return rc;
+    const Bufs B = bufs_at(ws, L);
+    if ((rc = key_scan(h, kv, K->dtype, G, sp, B, status, st, mark))) return rc;
+    CU(mark());
+    CU(launch_score_to_select(G, H, N, sp, (int)keep, (int)n_safe, B.a_raw, B.mm, a_star, star_row, budgets, idx,
+                              (int64_t)H * keep, head_offsets, status, st, &h->launches));
+    CU(mark());
+    CU(mark());   // the budget and select stages are part of that call
+    CU(mark());
+    CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, K_out, V_out, h->sm_count, st, &h->launches));
+    CU(mark());
     if (timing) h->timing_valid = 1;
     return NKV_OK;
 }
@@ -556,7 +529,7 @@ int nkv_host_staging_bytes(const nkv_handle* h, int64_t H, int64_t N, int64_t d,
     slot += align_up(c * H * keep * 4);              // idx
     slot += align_up(c * (H + 1) * 4);               // head_offsets
     slot += align_up(c * H * 4);                     // budgets
-    slot += make_layout(c, c * H, N, d, (N + b - 1) / b).total;
+    slot += make_layout(c * H, N, d, (N + b - 1) / b).total;
     *out_bytes = 2 * slot;
     return NKV_OK;
 }
@@ -586,7 +559,7 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
     const size_t kv_bytes = align_up(c * H * N * d * eb), out_bytes = align_up(c * H * keep * d * eb);
     const size_t idx_bytes = align_up(c * H * keep * 4), off_bytes = align_up(c * (H + 1) * 4),
                  bud_bytes = align_up(c * H * 4);
-    const size_t ws_need = make_layout(c, c * H, N, d, (N + b - 1) / b).total;
+    const size_t ws_need = make_layout(c * H, N, d, (N + b - 1) / b).total;
 
     int result = NKV_OK;
     int chunk_index = 0;
@@ -686,18 +659,17 @@ int nkv_key_scan(nkv_handle* h, const nkv_tensor* K, const nkv_params* params, f
     ScoreParams sp;
     if ((rc = resolve_params(params, K->N, &sp))) return rc;
     const int G = (int)K->G, N = (int)K->N, d = (int)K->d, units = (int)(K->G * K->H);
-    const Layout L = make_layout(G, units, N, d, sp.nblocks);
+    const Layout L = make_layout(units, N, d, sp.nblocks);
     if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    CU(cudaMemsetAsync(at<int>(ws, L.status), 0, kStatusWords * sizeof(int), st));
+    CU(cudaMemsetAsync(ws, 0, cleared_bytes(L, units), st));
     auto no_mark = []() -> cudaError_t { return cudaSuccess; };
-    if ((rc = key_scan(h, view_of(K), K->dtype, G, sp, bufs_at(ws, L, 0, K->H, N, d, sp.nblocks), at<int>(ws, L.status), st,
-                       no_mark)))
-        return rc;
+    if ((rc = key_scan(h, view_of(K), K->dtype, G, sp, bufs_at(ws, L), at<int>(ws, L.status), st, no_mark))) return rc;
+    const size_t row = (size_t)padded_row(N) * 4, out_row = (size_t)N * 4;
     CU(cudaMemcpyAsync(mu_s, at<float>(ws, L.mu_s), (size_t)units * d * 4, cudaMemcpyDeviceToDevice, st));
     CU(cudaMemcpyAsync(mu_e, at<float>(ws, L.mu_e), (size_t)units * sp.nblocks * d * 4, cudaMemcpyDeviceToDevice, st));
-    CU(cudaMemcpyAsync(inv_norm, at<float>(ws, L.inv_norm), (size_t)units * N * 4, cudaMemcpyDeviceToDevice, st));
-    CU(cudaMemcpyAsync(a_raw, at<float>(ws, L.a_raw), (size_t)units * 3 * N * 4, cudaMemcpyDeviceToDevice, st));
+    CU(cudaMemcpy2DAsync(inv_norm, out_row, at<float>(ws, L.inv_norm), row, out_row, units, cudaMemcpyDeviceToDevice, st));
+    CU(cudaMemcpy2DAsync(a_raw, out_row, at<float>(ws, L.a_raw), row, out_row, (size_t)units * 3, cudaMemcpyDeviceToDevice, st));
     minmax_floats_kernel<<<(units * 6 + 255) / 256, 256, 0, st>>>(units * 6, at<uint32_t>(ws, L.mm), minmax);
     ++h->launches;
     CU(cudaGetLastError());

@@ -32,7 +32,11 @@ struct ScoreParams {
     int window, n_sink, block, nblocks, gate_mode, top_m;
     float log_prior[3];
     float beta, tau, kappa;
+    int64_t raw_row, inv_row;   // row strides (floats) of the raw anomalies and of 1/||k||
 };
+
+// Per-head minimum and maximum of each scale, [3][2] keys that start at 0 and grow by atomicMax: the complement of the
+// minimum's ordered key, the maximum's ordered key.
 
 // Order-preserving map float -> uint32 (larger float <=> larger key) and back.
 __host__ __device__ __forceinline__ uint32_t ord_key(float f) {
@@ -110,7 +114,6 @@ __device__ __forceinline__ void set_status(int* status, int code, int detail) {
 }
 
 // ---- launchers implemented in the .cu files (all enqueue on `stream`, return cudaError_t) ----
-cudaError_t launch_threshold_scores(int units, const uint32_t* thr, float* out, cudaStream_t stream, int64_t* launches);
 constexpr int kWaitProbeDetail = 799;   // status detail recorded by the wait probe
 cudaError_t launch_wait_probe(int* status, uint32_t limit, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_anchor_sums(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
@@ -120,8 +123,7 @@ cudaError_t launch_anchor_means(int units, int N, int d, const ScoreParams& sp, 
 cudaError_t launch_window_means(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* inv_norm,
                                 float* mu_c, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_anchor_norms(int units, int d, const ScoreParams& sp, const float* mu_s, const float* mu_e,
-                                float* inv_mu_s_norm, float* inv_mu_e_norm, uint32_t* minmax_keys_to_reset_or_null,
-                                cudaStream_t stream, int64_t* launches);
+                                float* inv_mu_s_norm, float* inv_mu_e_norm, cudaStream_t stream, int64_t* launches);
 // streaming key passes (block size a multiple of 8)
 bool stream_path_supported(const ScoreParams& sp);
 cudaError_t launch_stream_a(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
@@ -150,17 +152,18 @@ cudaError_t launch_scan_scores(const TensorView& K, int dtype, int G, const Scor
                                const float* mu_e, const float* inv_norm, const float* inv_mu_s_norm,
                                const float* inv_mu_e_norm, float* a_raw, uint32_t* minmax_keys,
                                cudaStream_t stream, int64_t* launches);
-size_t head_stat_bytes(int64_t units);   // scratch of launch_head_scores (`hstat`)
 cudaError_t launch_head_scores(int units, int N, const ScoreParams& sp, const float* a_raw,
-                               const uint32_t* minmax_keys, float* a_star, float* head_stats_opt, float* hstat,
-                               int* status, cudaStream_t stream, int64_t* launches);
-size_t budget_scratch_bytes(int64_t G, int64_t H);   // scratch of the parallel form of launch_budget
+                               const uint32_t* minmax_keys, float* a_star, float* head_stats_opt, int* status,
+                               cudaStream_t stream, int64_t* launches);
 cudaError_t launch_budget(int G, int H, int N, int keep, int n_safe, const float* a_star, int32_t* budgets,
-                          uint32_t* sel_thresholds, int* status, void* scratch_or_null, cudaStream_t stream,
-                          int64_t* launches);
+                          float* thresholds_opt, int* status, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_select(int G, int H, int N, int64_t idx_capacity, const float* a_star, const int32_t* budgets,
-                          const uint32_t* sel_thresholds_or_null, int32_t* idx, int32_t* head_offsets, int* status,
-                          cudaStream_t stream, int64_t* launches);
+                          int32_t* idx, int32_t* head_offsets, int* status, cudaStream_t stream, int64_t* launches);
+// the three in one or two launches; rows of a_star are star_row floats apart
+cudaError_t launch_score_to_select(int G, int H, int N, const ScoreParams& sp, int keep, int n_safe, const float* a_raw,
+                                   const uint32_t* minmax_keys, float* a_star, int64_t star_row, int32_t* budgets, int32_t* idx,
+                                   int64_t idx_capacity, int32_t* head_offsets, int* status, cudaStream_t stream,
+                                   int64_t* launches);
 cudaError_t launch_ranks(int units, int N, const float* a_star, int32_t* ranks, cudaStream_t stream,
                          int64_t* launches);
 cudaError_t launch_gather(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,

@@ -198,9 +198,9 @@ __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileR
         lo_e = warp_min(lo_e);
         hi_e = warp_max(hi_e);
         if (lane == 0 && lo_s <= hi_s) {
-            atomicMin(&mm[(int64_t)cur_u * 6 + 0], ord_key(lo_s));
+            atomicMax(&mm[(int64_t)cur_u * 6 + 0], ~ord_key(lo_s));
             atomicMax(&mm[(int64_t)cur_u * 6 + 1], ord_key(hi_s));
-            atomicMin(&mm[(int64_t)cur_u * 6 + 2], ord_key(lo_e));
+            atomicMax(&mm[(int64_t)cur_u * 6 + 2], ~ord_key(lo_e));
             atomicMax(&mm[(int64_t)cur_u * 6 + 3], ord_key(hi_e));
         }
         lo_s = lo_e = INFINITY;
@@ -220,7 +220,7 @@ __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileR
         x.i = i0 + r;
         x.second = x.i >= (blk0 + 1) * sp.block;   // the key lies in the block after the tile's first
         const int blk = min(blk0 + (x.second ? 1 : 0), sp.nblocks - 1);
-        x.inv_i = x.i < N ? inv_norm[(int64_t)x.u * N + x.i] : 0.f;
+        x.inv_i = x.i < N ? inv_norm[x.u * sp.inv_row + x.i] : 0.f;
         x.re = inv_e[(int64_t)x.u * sp.nblocks + blk];
         return x;
     };
@@ -250,8 +250,8 @@ __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileR
         const float a_s = -(ds * scaled) * rs + 0.f;
         const float a_e = -(de * scaled) * cur.re + 0.f;
         if (cur.i < N) {
-            a_raw[((int64_t)cur.u * 3 + 0) * N + cur.i] = a_s;
-            a_raw[((int64_t)cur.u * 3 + 1) * N + cur.i] = a_e;
+            a_raw[((int64_t)cur.u * 3 + 0) * sp.raw_row + cur.i] = a_s;
+            a_raw[((int64_t)cur.u * 3 + 1) * sp.raw_row + cur.i] = a_e;
             lo_s = fminf(lo_s, a_s);
             hi_s = fmaxf(hi_s, a_s);
             lo_e = fminf(lo_e, a_e);

@@ -3,9 +3,9 @@
 // Some hosts of this library may not create device memory at the point where they need budgets:
 // code running inside a memory pool whose size was fixed at start-up, a plugin that is handed
 // only its inputs and outputs, or a step that runs while the process is forbidden to grow its
-// footprint.  nkv_budget needs a small scratch area (status words and per-head selection
-// thresholds) that such a caller has no way to provide, so this variant keeps that scratch in a
-// fixed array that is part of the library image on every GPU that loads it.
+// footprint.  nkv_budget needs a small scratch area (status words) that such a caller has no way
+// to provide, so this variant keeps that scratch in a fixed array that is part of the library
+// image on every GPU that loads it.
 //
 // The array's name is only a host-side stand-in in host code; the device address is looked up
 // with cudaGetSymbolAddress, once per device, by the first call made with that device current.
@@ -17,10 +17,9 @@ namespace {
 
 constexpr int kStaticMaxUnits = NKV_STATIC_MAX_UNITS;
 constexpr size_t kStatusBytes = nkv::kStatusWords * sizeof(int);              // 256
-constexpr size_t kStaticBytes = kStatusBytes + (size_t)kStaticMaxUnits * 8;   // status words + (threshold, quota) pairs
 
 // Scratch shared by every nkv_budget_static call on a device; lives until the process exits.
-static __device__ __align__(256) unsigned char g_budget_scratch[kStaticBytes];
+static __device__ __align__(256) unsigned char g_budget_scratch[kStatusBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_lock;
@@ -58,14 +57,12 @@ extern "C" int nkv_budget_static(const float* a_star, int64_t G, int64_t H, int6
     int rc = scratch_for_current_device(&scratch);
     if (rc != NKV_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    // the scratch keeps the previous call's contents: the status words must start at zero, the
-    // threshold pairs of the G*H heads of this call are all rewritten by the kernel
+    // the scratch keeps the previous call's contents: the status words must start at zero
     if (cudaMemsetAsync(scratch, 0, kStatusBytes, st) != cudaSuccess) return NKV_ERR_CUDA;
     int64_t launches = 0;
     unsigned char* base = reinterpret_cast<unsigned char*>(scratch);
     if (nkv::launch_budget((int)G, (int)H, (int)N, (int)keep, (int)n_safe, a_star, budgets,
-                           reinterpret_cast<uint32_t*>(base + kStatusBytes), reinterpret_cast<int*>(base), nullptr, st,
-                           &launches) != cudaSuccess)
+                           nullptr, reinterpret_cast<int*>(base), st, &launches) != cudaSuccess)
         return NKV_ERR_CUDA;
     return NKV_OK;
 }

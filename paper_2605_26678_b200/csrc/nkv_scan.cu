@@ -3,7 +3,7 @@
 //   anchor_sums   (Section 2.1, 2.2)  1/||k_i|| per token and the sum of normalised
 //                                     keys of every episodic block
 //   anchor_means  (Section 2.2)       block means and the stable mean
-//   anchor_norms                      1/||mu_s||, 1/||mu_e[t]|| and min/max key reset
+//   anchor_norms                      1/||mu_s||, 1/||mu_e[t]||
 //   scan_scores   (Section 2.3)       a_s, a_e, a_c of every token from one staged
 //                                     read of the key tile, plus per-head min/max
 //   window_means  (Section 2.2)       explicit mu_c(i), for inspection only
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256) anchor_sums_kernel(TensorView K, ScorePar
         if (ok) {
 #pragma unroll
             for (int c = 0; c < M::kCols; ++c) acc[c] = fmaf(v[c], inv, acc[c]);
-            if (l == 0) inv_norm[(int64_t)u * K.N + r] = inv;
+            if (l == 0) inv_norm[u * sp.inv_row + r] = inv;
         }
     }
     store_cols<T, D>(&red[grp][0], l, acc);
@@ -146,10 +146,10 @@ __global__ void anchor_means_kernel(int N, int d, ScoreParams sp, float* __restr
     mu_s[(int64_t)u * d + c] = sum / (float)N;
 }
 
-// anchor_norms: reciprocal norms of the anchors; also resets the per-head min/max keys.
+// anchor_norms: reciprocal norms of the anchors.
 __global__ void __launch_bounds__(128) anchor_norms_kernel(int d, ScoreParams sp, const float* __restrict__ mu_s,
                                                            const float* __restrict__ mu_e, float* __restrict__ inv_s,
-                                                           float* __restrict__ inv_e, uint32_t* __restrict__ mm) {
+                                                           float* __restrict__ inv_e) {
     const int u = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll 4
     for (int t = w - 1; t < sp.nblocks; t += 4) {
@@ -163,7 +163,6 @@ __global__ void __launch_bounds__(128) anchor_norms_kernel(int d, ScoreParams sp
             else inv_e[(int64_t)u * sp.nblocks + t] = inv;
         }
     }
-    if (mm && threadIdx.x < 6) mm[(int64_t)u * 6 + threadIdx.x] = (threadIdx.x & 1) ? 0u : 0xffffffffu;  // [scale][min,max]
 }
 
 // ------------------------------------------------------------------------------------------
@@ -213,7 +212,7 @@ scan_scores_kernel(TensorView K, ScoreParams sp, const float* __restrict__ mu_s,
     }
     for (int sr = tid; sr < kRows; sr += 256) {
         const int gr = i0 - kMaxWindow + sr;
-        invs[sr] = (gr >= 0 && gr < N) ? inv_norm[(int64_t)u * N + gr] : 0.f;
+        invs[sr] = (gr >= 0 && gr < N) ? inv_norm[u * sp.inv_row + gr] : 0.f;
     }
     __syncthreads();
 
@@ -330,12 +329,11 @@ scan_scores_kernel(TensorView K, ScoreParams sp, const float* __restrict__ mu_s,
     if (tid < 6) {
         float v = red[tid];
         for (int w = 1; w < 8; ++w) v = (tid & 1) ? fmaxf(v, red[w * 6 + tid]) : fminf(v, red[w * 6 + tid]);
-        if (tid & 1) atomicMax(&mm[(int64_t)u * 6 + tid], ord_key(v));
-        else atomicMin(&mm[(int64_t)u * 6 + tid], ord_key(v));
+        atomicMax(&mm[(int64_t)u * 6 + tid], (tid & 1) ? ord_key(v) : ~ord_key(v));
     }
     for (int idx = tid; idx < 3 * kTile; idx += 256) {
         const int k = idx / kTile, j = idx - k * kTile;
-        if (i0 + j < N) a_raw[((int64_t)u * 3 + k) * N + i0 + j] = outbuf[idx];
+        if (i0 + j < N) a_raw[((int64_t)u * 3 + k) * sp.raw_row + i0 + j] = outbuf[idx];
     }
 }
 
@@ -349,7 +347,7 @@ __global__ void window_means_kernel(TensorView K, ScoreParams sp, const float* _
     const T* base = reinterpret_cast<const T*>(K.ptr) + (int64_t)g * K.stride_g + (int64_t)h * K.stride_h;
     const int lft = max(0, i - sp.window + 1);
     float s = 0.f;
-    for (int j = lft; j <= i; ++j) s = fmaf((float)base[(int64_t)j * K.d + c], inv_norm[(int64_t)u * K.N + j], s);
+    for (int j = lft; j <= i; ++j) s = fmaf((float)base[(int64_t)j * K.d + c], inv_norm[u * sp.inv_row + j], s);
     mu_c[((int64_t)u * K.N + i) * K.d + c] = s / (float)(i - lft + 1);
 }
 
@@ -401,9 +399,8 @@ cudaError_t launch_anchor_means(int units, int N, int d, const ScoreParams& sp, 
 }
 
 cudaError_t launch_anchor_norms(int units, int d, const ScoreParams& sp, const float* mu_s, const float* mu_e,
-                                float* inv_mu_s_norm, float* inv_mu_e_norm, uint32_t* minmax_keys,
-                                cudaStream_t stream, int64_t* launches) {
-    anchor_norms_kernel<<<units, 128, 0, stream>>>(d, sp, mu_s, mu_e, inv_mu_s_norm, inv_mu_e_norm, minmax_keys);
+                                float* inv_mu_s_norm, float* inv_mu_e_norm, cudaStream_t stream, int64_t* launches) {
+    anchor_norms_kernel<<<units, 128, 0, stream>>>(d, sp, mu_s, mu_e, inv_mu_s_norm, inv_mu_e_norm);
     ++*launches;
     return cudaGetLastError();
 }

@@ -192,7 +192,7 @@ __device__ __forceinline__ void cta_minmax_to_global(float lo, float hi, float* 
             hi = fmaxf(hi, red[w * 2 + 1]);
         }
         if (lo <= hi) {
-            atomicMin(mm_lo, ord_key(lo));
+            atomicMax(mm_lo, ~ord_key(lo));
             atomicMax(mm_hi, ord_key(hi));
         }
     }
@@ -435,8 +435,8 @@ stream_a_kernel(TensorView K, ScoreParams sp, int units, float* __restrict__ blo
         __syncthreads();
         for (int j = tid; j < TILE; j += C::kThreads) {
             if (i0 + j < N) {
-                a_raw[((int64_t)u * 3 + 2) * N + i0 + j] = outbuf[j];
-                inv_norm[(int64_t)u * N + i0 + j] = invs[kHalo + j];
+                a_raw[((int64_t)u * 3 + 2) * sp.raw_row + i0 + j] = outbuf[j];
+                inv_norm[u * sp.inv_row + i0 + j] = invs[kHalo + j];
             }
         }
         __syncthreads();   // the tile, pp, invs and outbuf may be overwritten from here on
@@ -528,7 +528,7 @@ stream_b_kernel(TensorView K, ScoreParams sp, int units, const float* __restrict
         const float re = inv_e[(int64_t)u * sp.nblocks + blk];
         // after the reduction lane l finishes token o_mine of the group
         const int o_mine = (L == 16) ? (l >> 1) : l;
-        const float inv_mine = (gi0 + o_mine < N) ? inv_norm[(int64_t)u * N + gi0 + o_mine] : 0.f;
+        const float inv_mine = (gi0 + o_mine < N) ? inv_norm[u * sp.inv_row + gi0 + o_mine] : 0.f;
 
         if (!mbar_wait(&full[buf], (uint32_t)((it >> 1) & 1), status, 402)) return;
         __syncthreads();
@@ -574,18 +574,10 @@ stream_b_kernel(TensorView K, ScoreParams sp, int units, const float* __restrict
         __syncthreads();
         for (int j = tid; j < 2 * TILE; j += C::kThreads) {
             const int k = j / TILE, jj = j - k * TILE;
-            if (i0 + jj < N) a_raw[((int64_t)u * 3 + k) * N + i0 + jj] = outbuf[j];
+            if (i0 + jj < N) a_raw[((int64_t)u * 3 + k) * sp.raw_row + i0 + jj] = outbuf[j];
         }
         __syncthreads();
     }
-}
-
-// reset of the per-head min/max keys (and, when blocks straddle tiles, of the block sums)
-__global__ void stream_init_kernel(int units, uint32_t* mm, float* block_sums, long long n_sums) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < (long long)units * 6) mm[i] = (i & 1) ? 0u : 0xffffffffu;
-    if (block_sums)
-        for (long long j = i; j < n_sums; j += (long long)gridDim.x * blockDim.x) block_sums[j] = 0.f;
 }
 
 // tile sizes per (type, head dim)
@@ -639,12 +631,10 @@ cudaError_t launch_stream_a(const TensorView& K, int dtype, int G, const ScorePa
 #define CALL(T, D) tile = Tiles<T, D>::A
     NKV_DISPATCH(dtype, K.d, CALL);
 #undef CALL
-    const bool straddle = (tile % sp.block) != 0;
-    const long long n_sums = (long long)units * sp.nblocks * K.d;
-    int init_grid = (units * 6 + 255) / 256;
-    if (straddle && init_grid < 1024) init_grid = 1024;
-    stream_init_kernel<<<init_grid, 256, 0, stream>>>(units, mm, straddle ? block_sums : nullptr, n_sums);
-    ++*launches;
+    if (tile % sp.block != 0) {   // blocks straddle tiles: their sums are added up
+        const cudaError_t e = cudaMemsetAsync(block_sums, 0, (size_t)units * sp.nblocks * K.d * sizeof(float), stream);
+        if (e != cudaSuccess) return e;
+    }
     const long long total = (long long)units * ((K.N + tile - 1) / tile);
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
 #define CALL(T, D)                                                                                         \

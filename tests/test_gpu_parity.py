@@ -493,3 +493,42 @@ def test_tensor_first_pass_edges(H, layers, N, d, dtype):
         pr.assert_close(a_raw, ref.a_raw, "a_raw", 1e-5)
         pr.assert_close(minmax[0::2], ref.lo, "lo", 1e-5)
         pr.assert_close(minmax[1::2], ref.hi, "hi", 1e-5)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,H,N,r,ties", [
+    (40, 8, 611, 0.75, "none"), (20, 12, 900, 0.5, "none"), (1, 64, 303, 0.5, "many"), (200, 2, 260, 0.9, "none"),
+    (1, 1, 5, 0.5, "none"), (3, 8, 40000, 0.75, "dense"), (1, 16, 20000, 0.9, "all"), (1, 7, 26001, 0.6, "none")])
+def test_budget_and_select_in_every_layout(G, H, N, r, ties):
+    """One, two, four and eight CTAs per group, several heads per CTA, scores in shared memory and not, bins that
+    overflow their lists: budgets and positions bit for bit."""
+    s = _random_scores(G, H, N, seed=N + G, ties=ties)
+    a_star = torch.from_numpy(s).to(DEV)
+    ws = torch.zeros(256 + 256 * ((8 * G * H + 255) // 256), dtype=torch.uint8, device=DEV)
+    budgets = nkv.nkv_budget(a_star, r, ws=ws)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    idx, offs, _ = nkv.nkv_select(a_star, budgets, H * nkv.nkv_keep_per_head(N, r))
+    torch.cuda.synchronize()
+    for g in {0, G // 2, G - 1}:
+        ref = oracle.budget_select(s[g], r)
+        assert np.array_equal(budgets[g].cpu().numpy(), ref.budgets)
+        assert np.array_equal(offs[g].cpu().numpy(), ref.offsets)
+        assert np.array_equal(idx[g].cpu().numpy(), ref.idx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("layers,H,N,d", [(40, 8, 701, 64), (20, 12, 1100, 64), (2, 8, 30011, 64), (37, 4, 5000, 64)])
+def test_score_to_select_in_every_layout(layers, H, N, d):
+    """The score side of the fused call in one launch and in two, one head per CTA and several."""
+    K, V = _cache(N, d, "bf16", H=H, layers=layers)
+    p = nkv.nkv_default_params()
+    ws = nkv.alloc_workspace(K, p)
+    res = nkv.nkv_compress(K, V, 0.75, p, ws=ws, want_a_star=True)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    plain = nkv.nkv_compress(K, V, 0.75, p, ws=ws)     # scores in the padded rows of the workspace
+    torch.cuda.synchronize()
+    assert torch.equal(plain.idx, res.idx) and torch.equal(plain.budgets, res.budgets)
+    rep = pr.SwapReport()
+    for g in {0, layers - 1}:
+        pr.check_group_against_oracle(K, V, res, g, 0.75, p, rep)
+    assert rep.swapped_tokens <= max(2, rep.heads)
