@@ -189,8 +189,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
                           anchor_dots_supported(kv, dtype, sp);
     if (!tensor_a && !stream_path_supported(sp)) {
         CU(launch_anchor_sums(kv, dtype, G, sp, B.mu_e, B.inv_norm, st, &h->launches));
-        CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
-        CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, st, &h->launches));
+        CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, B.inv_e, B.inv_s, st, &h->launches));
         CU(mark());
         CU(launch_scan_scores(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, st,
                               &h->launches));
@@ -201,8 +200,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
         CU(launch_gram_pass(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
     else
         CU(launch_stream_a(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
-    CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, st, &h->launches));
-    CU(launch_anchor_norms(units, d, sp, B.mu_s, B.mu_e, B.inv_s, B.inv_e, st, &h->launches));
+    CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, B.inv_e, B.inv_s, st, &h->launches));
     CU(mark());
     // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
     const bool tensor_b = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
@@ -368,7 +366,7 @@ int nkv_anchors(nkv_handle* h, const nkv_tensor* K, const nkv_params* params, fl
     const int units = (int)(K->G * K->H);
     sp.inv_row = K->N;
     CU(launch_anchor_sums(kv, K->dtype, (int)K->G, sp, mu_e, inv_norm, st, &h->launches));
-    CU(launch_anchor_means(units, (int)K->N, (int)K->d, sp, mu_e, mu_s, st, &h->launches));
+    CU(launch_anchor_means(units, (int)K->N, (int)K->d, sp, mu_e, mu_s, nullptr, nullptr, st, &h->launches));
     if (mu_c_opt) CU(launch_window_means(kv, K->dtype, (int)K->G, sp, inv_norm, mu_c_opt, st, &h->launches));
     return NKV_OK;
 }

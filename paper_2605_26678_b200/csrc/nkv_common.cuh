@@ -119,7 +119,8 @@ cudaError_t launch_wait_probe(int* status, uint32_t limit, cudaStream_t stream, 
 cudaError_t launch_anchor_sums(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
                                float* inv_norm, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_anchor_means(int units, int N, int d, const ScoreParams& sp, float* mu_e_inout, float* mu_s,
-                                cudaStream_t stream, int64_t* launches);
+                                float* inv_mu_e_norm_or_null, float* inv_mu_s_norm_or_null, cudaStream_t stream,
+                                int64_t* launches);
 cudaError_t launch_window_means(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* inv_norm,
                                 float* mu_c, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_anchor_norms(int units, int d, const ScoreParams& sp, const float* mu_s, const float* mu_e,
