@@ -498,7 +498,7 @@ def test_tensor_first_pass_edges(H, layers, N, d, dtype):
 @pytest.mark.gpu
 @pytest.mark.parametrize("G,H,N,r,ties", [
     (40, 8, 611, 0.75, "none"), (20, 12, 900, 0.5, "none"), (1, 64, 303, 0.5, "many"), (200, 2, 260, 0.9, "none"),
-    (1, 1, 5, 0.5, "none"), (3, 8, 40000, 0.75, "dense"), (1, 16, 20000, 0.9, "all"), (1, 7, 26001, 0.6, "none")])
+    (150, 64, 120, 0.5, "none"), (150, 16, 130, 0.75, "many"), (1, 1, 5, 0.5, "none"), (3, 8, 40000, 0.75, "dense"), (1, 16, 20000, 0.9, "all"), (1, 7, 26001, 0.6, "none")])
 def test_budget_and_select_in_every_layout(G, H, N, r, ties):
     """One, two, four and eight CTAs per group, several heads per CTA, scores in shared memory and not, bins that
     overflow their lists: budgets and positions bit for bit."""
