@@ -231,8 +231,9 @@ NKV_API int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V
  * nkv_compress.  The call stages `groups_per_chunk` groups at a time through
  * the caller-provided device staging area `dev` (at least
  * nkv_host_staging_bytes() bytes, 256-byte aligned), overlapping the copies of
- * one chunk with the kernels of the previous one on two internal streams, and
- * returns after everything has arrived on the host (it synchronises).
+ * some groups with the kernels of others on internal streams, and returns after
+ * everything has arrived on the host (it synchronises).  Of a pinned V only the
+ * retained rows cross the bus, unless most of them are retained.
  */
 NKV_API int nkv_host_staging_bytes(const nkv_handle* h, int64_t H, int64_t N, int64_t d, int32_t dtype, double r,
                            const nkv_params* params, int64_t groups_per_chunk, size_t* out_bytes);

@@ -9,6 +9,8 @@
 
 using namespace nkv;
 
+constexpr int kHostSlots = 4;   // staging slots of nkv_compress_host, a stream each
+
 struct nkv_handle {
     int device;
     int sm_count;
@@ -18,8 +20,7 @@ struct nkv_handle {
     int timing_valid;
     int key_pass;     // NKV_KEY_PASS_*: which kernels make the two key passes
     cudaEvent_t ev[NKV_NUM_STAGES + 1];
-    cudaStream_t copy_streams[2];
-    cudaEvent_t slot_done[2];
+    cudaStream_t copy_streams[kHostSlots];
     int* chunk_status;   // pinned host copy of every chunk's status words (nkv_compress_host)
     int inject_status;   // tests: status code planted in chunk `inject_chunk` of nkv_compress_host
     int inject_chunk;
@@ -215,6 +216,62 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
     return NKV_OK;
 }
 
+// Staging of nkv_compress_host: the groups of a chunk are halved where possible, so that twice as many slots keep the
+// copy engines busy in both directions while kernels run.
+constexpr int kHostGatherCtas = 16;
+constexpr double kHostRowsShare = 0.6;
+struct HostSlot {
+    size_t K, V, K_out, V_out, idx, offsets, budgets, ws, total;
+};
+struct HostPlan {
+    int64_t groups;   // per slot
+    int slots;
+    HostSlot slot;
+};
+HostSlot host_slot(int64_t c, int64_t H, int64_t N, int64_t d, int dtype, int64_t keep, const nkv_params* params) {
+    const size_t eb = dtype == NKV_F32 ? 4 : 2;
+    const int64_t b = block_size(N, params);
+    HostSlot s;
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o += align_up(bytes);
+        return at;
+    };
+    s.K = take((size_t)c * H * N * d * eb);
+    s.V = take((size_t)c * H * N * d * eb);
+    s.K_out = take((size_t)c * H * keep * d * eb);
+    s.V_out = take((size_t)c * H * keep * d * eb);
+    s.idx = take((size_t)c * H * keep * 4);
+    s.offsets = take((size_t)c * (H + 1) * 4);
+    s.budgets = take((size_t)c * H * 4);
+    s.ws = o;
+    s.total = o + make_layout(c * H, N, d, (N + b - 1) / b).total;
+    return s;
+}
+HostPlan host_plan(int64_t H, int64_t N, int64_t d, int dtype, int64_t keep, const nkv_params* params, int64_t groups_per_chunk) {
+    HostPlan p;
+    p.slots = groups_per_chunk >= 2 ? kHostSlots : 2;
+    p.groups = groups_per_chunk >= 2 ? groups_per_chunk / 2 : 1;
+    p.slot = host_slot(p.groups, H, N, d, dtype, keep, params);
+    return p;
+}
+
+// The address at which the current device reads [p, p + bytes) of host memory in place; null when it cannot.
+const void* device_address(const void* p, size_t bytes) {
+    cudaPointerAttributes first, last;
+    if (cudaPointerGetAttributes(&first, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&last, static_cast<const unsigned char*>(p) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer || !last.devicePointer)
+        return nullptr;
+    if (static_cast<unsigned char*>(last.devicePointer) - static_cast<unsigned char*>(first.devicePointer) != (ptrdiff_t)(bytes - 1))
+        return nullptr;
+    return first.devicePointer;
+}
+
 // ordered min/max keys -> floats (lo_s, hi_s, lo_e, hi_e, lo_c, hi_c per head)
 __global__ void minmax_floats_kernel(int n, const uint32_t* keys, float* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -322,9 +379,8 @@ int nkv_create(nkv_handle** out, int device) {
         delete h;
         return NKV_ERR_CUDA;
     }
-    for (int i = 0; i < 2; ++i) {
-        if (cudaStreamCreateWithFlags(&h->copy_streams[i], cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->slot_done[i], cudaEventDisableTiming) != cudaSuccess) {
+    for (int i = 0; i < kHostSlots; ++i) {
+        if (cudaStreamCreateWithFlags(&h->copy_streams[i], cudaStreamNonBlocking) != cudaSuccess) {
             delete h;
             return NKV_ERR_CUDA;
         }
@@ -336,10 +392,7 @@ int nkv_create(nkv_handle** out, int device) {
 int nkv_destroy(nkv_handle* h) {
     if (!h) return NKV_ERR_INVALID_ARG;
     for (int i = 0; i <= NKV_NUM_STAGES; ++i) cudaEventDestroy(h->ev[i]);
-    for (int i = 0; i < 2; ++i) {
-        cudaStreamDestroy(h->copy_streams[i]);
-        cudaEventDestroy(h->slot_done[i]);
-    }
+    for (int i = 0; i < kHostSlots; ++i) cudaStreamDestroy(h->copy_streams[i]);
     cudaFreeHost(h->chunk_status);
     delete h;
     return NKV_OK;
@@ -451,7 +504,7 @@ int nkv_compact(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, const i
     if (mode == NKV_OUT_OF_PLACE) {
         if (!K_out || !V_out || ((uintptr_t)K_out) % 16 || ((uintptr_t)V_out) % 16) return NKV_ERR_INVALID_ARG;
         CU(launch_gather(view_of(K), kb, view_of(V), vb, (int)K->G, idx, head_offsets, idx_capacity, K_out, V_out,
-                         h->sm_count, st, &h->launches));
+                         h->sm_count, 0, st, &h->launches));
     } else if (mode == NKV_IN_PLACE) {
         if (K_out || V_out) return NKV_ERR_INVALID_ARG;
         CU(launch_gather_in_place(view_of(K), kb, view_of(V), vb, (int)K->G, idx, head_offsets, idx_capacity, st,
@@ -462,9 +515,10 @@ int nkv_compact(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, const i
     return NKV_OK;
 }
 
-int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double r, const nkv_params* params,
-                 void* K_out, void* V_out, int32_t* idx, int32_t* head_offsets, int32_t* budgets,
-                 float* a_star_opt, void* ws, size_t ws_bytes, void* stream) {
+// `host_v`: V lies in host memory that the device can read; its retained rows are fetched over the bus from there.
+static int compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double r, const nkv_params* params, void* K_out,
+                    void* V_out, int32_t* idx, int32_t* head_offsets, int32_t* budgets, float* a_star_opt, void* ws,
+                    size_t ws_bytes, cudaStream_t st, bool host_v) {
     if (!h || !K_out || !V_out || !idx || !head_offsets || !budgets) return NKV_ERR_INVALID_ARG;
     int rc = check_tensor(K);
     if (rc) return rc;
@@ -483,7 +537,6 @@ int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double
     const int units = G * H;
     const Layout L = make_layout(units, N, d, sp.nblocks);
     if ((rc = check_ws(ws, ws_bytes, L.total))) return rc;
-    cudaStream_t st = (cudaStream_t)stream;
     const TensorView kv = view_of(K), vv = view_of(V);
     const int kb = K->dtype == NKV_F32 ? 4 : 2, vb = V->dtype == NKV_F32 ? 4 : 2;
     float* a_star = a_star_opt ? a_star_opt : at<float>(ws, L.a_star);
@@ -506,10 +559,22 @@ int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double
     CU(mark());
     CU(mark());   // the budget and select stages are part of that call
     CU(mark());
-    CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, K_out, V_out, h->sm_count, st, &h->launches));
+    CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, K_out, host_v ? nullptr : V_out, h->sm_count, 0, st,
+                     &h->launches));
+    // a few CTAs keep more reads on the bus than it takes to fill it, and leave the SMs to the kernels of other chunks
+    if (host_v)
+        CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, nullptr, V_out, h->sm_count, kHostGatherCtas, st,
+                         &h->launches));
     CU(mark());
     if (timing) h->timing_valid = 1;
     return NKV_OK;
+}
+
+int nkv_compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, double r, const nkv_params* params,
+                 void* K_out, void* V_out, int32_t* idx, int32_t* head_offsets, int32_t* budgets,
+                 float* a_star_opt, void* ws, size_t ws_bytes, void* stream) {
+    return compress(h, K, V, r, params, K_out, V_out, idx, head_offsets, budgets, a_star_opt, ws, ws_bytes, (cudaStream_t)stream,
+                    false);
 }
 
 int nkv_host_staging_bytes(const nkv_handle* h, int64_t H, int64_t N, int64_t d, int32_t dtype, double r,
@@ -519,17 +584,8 @@ int nkv_host_staging_bytes(const nkv_handle* h, int64_t H, int64_t N, int64_t d,
     if (!(r >= 0.0 && r < 1.0)) return NKV_ERR_INVALID_ARG;
     const int64_t keep = keep_count(N, r);
     if (keep < 1) return NKV_ERR_INVALID_ARG;
-    const size_t eb = dtype == NKV_F32 ? 4 : 2;
-    const int64_t b = block_size(N, params);
-    const size_t c = (size_t)groups_per_chunk;
-    size_t slot = 0;
-    slot += 2 * align_up(c * H * N * d * eb);        // K, V
-    slot += 2 * align_up(c * H * keep * d * eb);     // K_out, V_out
-    slot += align_up(c * H * keep * 4);              // idx
-    slot += align_up(c * (H + 1) * 4);               // head_offsets
-    slot += align_up(c * H * 4);                     // budgets
-    slot += make_layout(c * H, N, d, (N + b - 1) / b).total;
-    *out_bytes = 2 * slot;
+    const HostPlan p = host_plan(H, N, d, dtype, keep, params, groups_per_chunk);
+    *out_bytes = p.slots * p.slot.total;
     return NKV_OK;
 }
 
@@ -552,48 +608,44 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
     const int64_t G = Kh->G, H = Kh->H, N = Kh->N, d = Kh->d;
     const int64_t keep = keep_count(N, r);
     const size_t eb = Kh->dtype == NKV_F32 ? 4 : 2;
-    const int64_t b = block_size(N, params);
-    const size_t c = (size_t)groups_per_chunk;
-    const size_t slot_bytes = need / 2;
-    const size_t kv_bytes = align_up(c * H * N * d * eb), out_bytes = align_up(c * H * keep * d * eb);
-    const size_t idx_bytes = align_up(c * H * keep * 4), off_bytes = align_up(c * (H + 1) * 4),
-                 bud_bytes = align_up(c * H * 4);
-    const size_t ws_need = make_layout(c * H, N, d, (N + b - 1) / b).total;
+    const HostPlan p = host_plan(H, N, d, Kh->dtype, keep, params, groups_per_chunk);
+    const size_t grp_in = (size_t)H * N * d * eb, grp_out = (size_t)H * keep * d * eb;
+    // Only the retained rows of V are needed on the device.  Where the device can read V in place (pinned memory) the
+    // gather kernel fetches them from there, which spares the bus the others.  16 x 8 heads of 8192 x 64 bf16 keys: with
+    // a quarter of the rows kept 5.34 -> 3.52 ms, with half 5.67 -> 4.92, with three quarters 6.06 -> 6.60, where one
+    // copy is the better way; the two meet at about 0.6 of the rows.
+    const void* v_mapped = (double)keep <= kHostRowsShare * (double)N ? device_address(Vh->ptr, (size_t)G * grp_in) : nullptr;
 
     int result = NKV_OK;
-    int chunk_index = 0;
-    for (int64_t g0 = 0; g0 < G && result == NKV_OK; g0 += groups_per_chunk, ++chunk_index) {
-        const int slot = chunk_index & 1;
-        cudaStream_t st = h->copy_streams[slot];
-        const int64_t gc = (G - g0 < groups_per_chunk) ? (G - g0) : groups_per_chunk;
-        unsigned char* base = reinterpret_cast<unsigned char*>(dev) + slot * slot_bytes;
-        unsigned char* dK = base;
-        unsigned char* dV = dK + kv_bytes;
-        unsigned char* dKo = dV + kv_bytes;
-        unsigned char* dVo = dKo + out_bytes;
-        int32_t* dIdx = reinterpret_cast<int32_t*>(dVo + out_bytes);
-        int32_t* dOff = reinterpret_cast<int32_t*>(reinterpret_cast<unsigned char*>(dIdx) + idx_bytes);
-        int32_t* dBud = reinterpret_cast<int32_t*>(reinterpret_cast<unsigned char*>(dOff) + off_bytes);
-        void* dWs = reinterpret_cast<unsigned char*>(dBud) + bud_bytes;
-        const size_t grp_in = (size_t)H * N * d * eb, grp_out = (size_t)H * keep * d * eb;
-        // the slot's previous chunk finished all its copies before this stream reaches here (same stream)
+    int step = 0;
+    for (int64_t g0 = 0; g0 < G && result == NKV_OK; g0 += p.groups, ++step) {
+        cudaStream_t st = h->copy_streams[step % p.slots];
+        const int64_t gc = (G - g0 < p.groups) ? (G - g0) : p.groups;
+        unsigned char* base = reinterpret_cast<unsigned char*>(dev) + (size_t)(step % p.slots) * p.slot.total;
+        unsigned char *dK = base + p.slot.K, *dV = base + p.slot.V, *dKo = base + p.slot.K_out, *dVo = base + p.slot.V_out;
+        int32_t* dIdx = reinterpret_cast<int32_t*>(base + p.slot.idx);
+        int32_t* dOff = reinterpret_cast<int32_t*>(base + p.slot.offsets);
+        int32_t* dBud = reinterpret_cast<int32_t*>(base + p.slot.budgets);
+        void* dWs = base + p.slot.ws;
+        // the slot's previous groups finished all their copies before this stream reaches here (same stream)
         if (cudaMemcpyAsync(dK, (const unsigned char*)Kh->ptr + g0 * grp_in, gc * grp_in, cudaMemcpyHostToDevice, st) !=
                 cudaSuccess ||
-            cudaMemcpyAsync(dV, (const unsigned char*)Vh->ptr + g0 * grp_in, gc * grp_in, cudaMemcpyHostToDevice, st) !=
-                cudaSuccess) {
+            (!v_mapped && cudaMemcpyAsync(dV, (const unsigned char*)Vh->ptr + g0 * grp_in, gc * grp_in, cudaMemcpyHostToDevice,
+                                          st) != cudaSuccess)) {
             result = NKV_ERR_CUDA;
             break;
         }
         nkv_tensor dk = *Kh, dv = *Vh;
         dk.ptr = dK;
-        dv.ptr = dV;
+        dv.ptr = v_mapped ? const_cast<unsigned char*>((const unsigned char*)v_mapped) + g0 * grp_in : dV;
         dk.G = dv.G = gc;
-        rc = nkv_compress(h, &dk, &dv, r, params, dKo, dVo, dIdx, dOff, dBud, nullptr, dWs, ws_need, st);
+        rc = compress(h, &dk, &dv, r, params, dKo, dVo, dIdx, dOff, dBud, nullptr, dWs, p.slot.total - p.slot.ws, st,
+                      v_mapped != nullptr);
         if (rc) {
             result = rc;
             break;
         }
-        if (h->inject_status && chunk_index == h->inject_chunk &&
+        if (h->inject_status && g0 / groups_per_chunk == h->inject_chunk &&
             cudaMemcpyAsync(dWs, &h->inject_status, sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess) {
             result = NKV_ERR_CUDA;
             break;
@@ -607,13 +659,14 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
             cudaMemcpyAsync(head_offsets_host + g0 * (H + 1), dOff, gc * (H + 1) * 4, cudaMemcpyDeviceToHost, st) !=
                 cudaSuccess ||
             cudaMemcpyAsync(budgets_host + g0 * H, dBud, gc * H * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            (chunk_index < kMaxHostChunks &&
-             cudaMemcpyAsync(h->chunk_status + chunk_index * 4, dWs, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess)) {
+            (step < kMaxHostChunks &&
+             cudaMemcpyAsync(h->chunk_status + step * 4, dWs, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess)) {
             result = NKV_ERR_CUDA;
             break;
         }
     }
-    for (int i = 0; i < 2; ++i)
+    const int chunk_index = step;
+    for (int i = 0; i < kHostSlots; ++i)
         if (cudaStreamSynchronize(h->copy_streams[i]) != cudaSuccess) result = result ? result : NKV_ERR_CUDA;
     // every chunk's device status words were copied out before its slot was reused: report the first failure
     for (int c2 = 0; c2 < chunk_index && c2 < kMaxHostChunks && result == NKV_OK; ++c2)

@@ -152,11 +152,11 @@ GatherArgs make_args(const TensorView& K, int kb, const TensorView& V, int vb, i
 
 cudaError_t launch_gather(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,
                           const int32_t* idx, const int32_t* head_offsets, int64_t idx_capacity, void* K_out,
-                          void* V_out, int sm_count, cudaStream_t stream, int64_t* launches) {
+                          void* V_out, int sm_count, int ctas_or_0, cudaStream_t stream, int64_t* launches) {
     GatherArgs A = make_args(K, k_elem_bytes, V, v_elem_bytes, G, idx_capacity, K_out, V_out);
     const int64_t nbatch = (A.total_rows + kGatherRows - 1) / kGatherRows;
     if (nbatch == 0) return cudaSuccess;
-    int64_t grid = (int64_t)sm_count * 8;
+    int64_t grid = ctas_or_0 ? ctas_or_0 : (int64_t)sm_count * 8;
     if (grid > nbatch) grid = nbatch;
     gather_kernel<<<(unsigned)grid, 256, 0, stream>>>(A, idx, head_offsets);
     ++*launches;

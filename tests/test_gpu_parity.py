@@ -532,3 +532,22 @@ def test_score_to_select_in_every_layout(layers, H, N, d):
     for g in {0, layers - 1}:
         pr.check_group_against_oracle(K, V, res, g, 0.75, p, rep)
     assert rep.swapped_tokens <= max(2, rep.heads)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("layers,chunk,r,pinned", [(5, 1, 0.75, True), (7, 3, 0.75, True), (4, 4, 0.25, True), (3, 2, 0.75, False)])
+def test_host_entry_point_with_rows_fetched_in_place_and_copied(layers, chunk, r, pinned):
+    """Retained rows of V read from pinned memory, and V copied whole (most rows retained, or memory that the device
+    cannot read); chunks that do and do not divide the groups."""
+    K, V = _cache(700, 64, "bf16", H=3, layers=layers)
+    dev = nkv.nkv_compress(K, V, r)
+    torch.cuda.synchronize()
+    hold = (lambda t: t.pin_memory()) if pinned else (lambda t: t)
+    Kh, Vh = hold(K.cpu()), hold(V.cpu())
+    out = nkv.Compressed(*[hold(torch.empty(t.shape, dtype=t.dtype)) for t in
+                           (dev.k_out, dev.v_out, dev.idx, dev.head_offsets, dev.budgets)], None)
+    staging = torch.empty(nkv.nkv_host_staging_bytes(3, 700, 64, nkv.NKV_BF16, r, chunk), dtype=torch.uint8, device=DEV)
+    nkv.nkv_compress_host(Kh, Vh, r, out, staging, chunk)
+    for a, b in ((out.k_out, dev.k_out), (out.v_out, dev.v_out), (out.idx, dev.idx), (out.head_offsets, dev.head_offsets),
+                 (out.budgets, dev.budgets)):
+        assert torch.equal(a, b.cpu())
