@@ -180,6 +180,21 @@ Bufs bufs_at(void* ws, const Layout& L) {
     return b;
 }
 
+// The second pass over the keys: a_s and a_e of every token from the anchors.
+int anchor_scores(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreParams& sp, const float* mu_s, const float* mu_e,
+                  const float* inv_norm, const Bufs& B, float* a_raw, int* status, cudaStream_t st) {
+    // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
+    const bool tensor = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
+                        (h->key_pass == NKV_KEY_PASS_TENSOR || kv.d == 128 || !stream_path_supported(sp));
+    if (tensor)
+        CU(launch_anchor_dots(kv, dtype, G, sp, mu_s, mu_e, inv_norm, B.inv_s, B.inv_e, a_raw, B.mm, status, h->sm_count, st,
+                              &h->launches));
+    else
+        CU(launch_stream_b(kv, dtype, G, sp, mu_s, mu_e, inv_norm, B.inv_s, B.inv_e, a_raw, B.mm, status, h->sm_count, st,
+                           &h->launches));
+    return NKV_OK;
+}
+
 // The two passes over the keys (Sections 2.1-2.3): afterwards the workspace holds 1/||k||, the anchors, the
 // three raw anomalies and their per-head min/max keys (which start out cleared).  `mark` is called once between the passes (stage
 // timing).
@@ -199,21 +214,12 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
     }
     // pass A: norms, block sums and the current-memory anomaly; pass B: the two anchor anomalies
     if (tensor_a)
-        CU(launch_gram_pass(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
+        CU(launch_gram_pass(kv, dtype, G, sp, nullptr, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
     else
         CU(launch_stream_a(kv, dtype, G, sp, B.mu_e, B.inv_norm, B.a_raw, B.mm, status, h->sm_count, st, &h->launches));
     CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, B.inv_e, B.inv_s, st, &h->launches));
     CU(mark());
-    // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
-    const bool tensor_b = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
-                          (h->key_pass == NKV_KEY_PASS_TENSOR || d == 128 || !stream_path_supported(sp));
-    if (tensor_b)
-        CU(launch_anchor_dots(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, status, h->sm_count,
-                              st, &h->launches));
-    else
-        CU(launch_stream_b(kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B.inv_s, B.inv_e, B.a_raw, B.mm, status, h->sm_count, st,
-                           &h->launches));
-    return NKV_OK;
+    return anchor_scores(h, kv, dtype, G, sp, B.mu_s, B.mu_e, B.inv_norm, B, B.a_raw, status, st);
 }
 
 // Staging of nkv_compress_host: the groups of a chunk are halved where possible, so that twice as many slots keep the
@@ -443,10 +449,18 @@ int nkv_score(nkv_handle* h, const nkv_tensor* K, const float* mu_s, const float
     if (a_raw_opt) sp.raw_row = K->N;
     float* a_raw = a_raw_opt ? a_raw_opt : at<float>(ws, L.a_raw);
     CU(cudaMemsetAsync(ws, 0, cleared_bytes(L, units), st));
-    CU(launch_anchor_norms(units, (int)K->d, sp, mu_s, mu_e, at<float>(ws, L.inv_s), at<float>(ws, L.inv_e), st,
-                           &h->launches));
-    CU(launch_scan_scores(kv, K->dtype, (int)K->G, sp, mu_s, mu_e, inv_norm, at<float>(ws, L.inv_s),
-                          at<float>(ws, L.inv_e), a_raw, at<uint32_t>(ws, L.mm), st, &h->launches));
+    const Bufs B = bufs_at(ws, L);
+    const int G = (int)K->G;
+    CU(launch_anchor_norms(units, (int)K->d, sp, mu_s, mu_e, B.inv_s, B.inv_e, st, &h->launches));
+    // two passes on the tensor cores against one that keeps a window sum per lane group: 58 + 56 us against 257 at
+    // 28 x 8 heads of 4133 x 128 bf16 keys
+    if (h->key_pass != NKV_KEY_PASS_FMA && gram_pass_supported(kv, K->dtype, sp) && anchor_dots_supported(kv, K->dtype, sp)) {
+        CU(launch_gram_pass(kv, K->dtype, G, sp, inv_norm, nullptr, nullptr, a_raw, B.mm, at<int>(ws, L.status), h->sm_count, st,
+                            &h->launches));
+        if ((rc = anchor_scores(h, kv, K->dtype, G, sp, mu_s, mu_e, inv_norm, B, a_raw, at<int>(ws, L.status), st))) return rc;
+    } else {
+        CU(launch_scan_scores(kv, K->dtype, G, sp, mu_s, mu_e, inv_norm, B.inv_s, B.inv_e, a_raw, B.mm, st, &h->launches));
+    }
     CU(launch_head_scores(units, (int)K->N, sp, a_raw, at<uint32_t>(ws, L.mm), a_star, head_stats_opt,
                           at<int>(ws, L.status), st, &h->launches));
     return NKV_OK;

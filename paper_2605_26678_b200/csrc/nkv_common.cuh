@@ -137,8 +137,9 @@ cudaError_t launch_stream_b(const TensorView& K, int dtype, int G, const ScorePa
 // first key pass on the tensor cores (16-bit keys): same outputs as launch_stream_a
 bool gram_pass_supported(const TensorView& K, int dtype, const ScoreParams& sp);
 cudaError_t configure_gram_kernels();
-cudaError_t launch_gram_pass(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums, float* inv_norm,
-                             float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
+// (`given`: the norms are the caller's, block_sums and inv_norm are null)
+cudaError_t launch_gram_pass(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* given,
+                             float* block_sums, float* inv_norm, float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
                              int64_t* launches);
 // second key pass on the tensor cores (16-bit keys): same outputs as launch_stream_b
 bool anchor_dots_supported(const TensorView& K, int dtype, const ScoreParams& sp);

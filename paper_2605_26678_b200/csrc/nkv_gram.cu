@@ -263,7 +263,7 @@ __device__ void mma_role(unsigned char* ring, Smem<D>* s, uint32_t tmem_base, Wa
 // Sums of normalised keys per episodic block.  Lane group grp (8 columns per lane) takes rows
 // [grp * R, grp * R + R) of every tile and keeps its running sum in registers until the block ends; then the groups'
 // parts are added up over the warp and in shared memory.
-template <typename T, int D>
+template <typename T, int D, bool kGiven>
 __device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int block, int N, float* __restrict__ block_sums,
                           int* status) {
     using C = Cfg<D>;
@@ -302,7 +302,7 @@ __device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int 
             while (true) {
                 const int cut = min(end - R0, hi);
                 const int a = lo - r0, b = cut - r0;        // the same in rows of this group
-                if (a < R && b > 0) {
+                if (!kGiven && a < R && b > 0) {
                     float v[R];
 #pragma unroll
                     for (int i = 0; i < R; ++i) v[i] = w[i];
@@ -338,7 +338,7 @@ __device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int 
                     *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
                 }
                 if (bar_or(kBarSums, kSumsThreads, false)) return;
-                if (t < D) {
+                if (!kGiven && t < D) {
                     float sum = 0.f;
 #pragma unroll
                     for (int q = 0; q < kSumsThreads / 32; ++q) sum += s->red[flushes & 1][q][t];
@@ -398,8 +398,9 @@ __device__ __forceinline__ void chunk_sums(const float (*v)[16], const float* wc
     }
 }
 
-template <int D>
-__device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, int N, int* status) {
+template <int D, bool kGiven>
+__device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, int N, const float* __restrict__ given, int64_t inv_row,
+                          int* status) {
     const int warp = threadIdx.x >> 5, t = threadIdx.x & 31;
     const int q = warp & 3, which = warp >> 2;   // lane quarter; the group takes tiles n with n % 2 == which
     const int b0 = 2 * (t & 3), r0 = (t >> 2) + 1;
@@ -415,6 +416,14 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
         for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
             if ((int)(n & 1) != which) continue;
             const int slot = (int)(n & (kWRing - 1)), prev = (int)((n - 1) & (kWRing - 1)), cb = (int)(n & (kCfRing - 1));
+            float have[4];   // the norms of the quarter's rows, where the caller brings them
+            if constexpr (kGiven) {
+#pragma unroll
+                for (int J = 0; J < 4; ++J) {
+                    const int i = sp.base + kTile * tau + 32 * q + 8 * J + (t >> 2);
+                    have[J] = i < N ? given[sp.u * inv_row + i] : 0.f;
+                }
+            }
             if (!warp_wait(&s->tfull[which], (n >> 1) & 1u, status, 706)) return;
             tc_fence_after();
             float z[2][16], y[2][16];
@@ -428,7 +437,8 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
                     const float* c = z[J >> 1];
                     const float G = oe ? c[4 * J + 2 * (J & 1) + 1] : c[4 * J + 2 * (J & 1)];
                     const int row = 32 * q + 8 * J + (t >> 2);
-                    const float inv = R0 + row < N ? inv_sqrt(fmaxf(G, kEps * kEps)) : 0.f;   // 1 / max(||k||, eps)
+                    // 1 / max(||k||, eps)
+                    const float inv = kGiven ? have[J] : R0 + row < N ? inv_sqrt(fmaxf(G, kEps * kEps)) : 0.f;
                     s->w[slot][row] = inv;
                     s->g[slot][row] = inv * inv * G;
                 }
@@ -521,7 +531,7 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x, a.y += b.y, a.z += b.z, a.w += b.w; }
 
-template <int D>
+template <int D, bool kGiven>
 __device__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __restrict__ inv_norm, int64_t inv_row,
                           float* __restrict__ a_raw, int64_t raw_row, uint32_t* __restrict__ mm, int* status) {
     const int which = (threadIdx.x >> 5) - kScanWarp0, l = threadIdx.x & 31;
@@ -580,10 +590,10 @@ __device__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __rest
             for (int e = 0; e < 4; ++e) ac[e] = quotient_by_root(-cc[e], fmaxf(base + x[e], kEps * kEps)) + 0.f;
             const int i = sp.base + kTile * tau + r;
             float* out_a = a_raw + ((int64_t)sp.u * 3 + 2) * raw_row + i;
-            float* out_w = inv_norm + sp.u * inv_row + i;
+            float* out_w = kGiven ? out_a : inv_norm + sp.u * inv_row + i;
             if (i >= sp.row0 && i + 4 <= sp.row1 && ((reinterpret_cast<uintptr_t>(out_a) | reinterpret_cast<uintptr_t>(out_w)) & 15) == 0) {
                 *reinterpret_cast<float4*>(out_a) = make_float4(ac[0], ac[1], ac[2], ac[3]);
-                *reinterpret_cast<float4*>(out_w) = wi;
+                if (!kGiven) *reinterpret_cast<float4*>(out_w) = wi;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) lo = fminf(lo, ac[e]), hi = fmaxf(hi, ac[e]);
             } else {
@@ -591,7 +601,7 @@ __device__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __rest
                 for (int e = 0; e < 4; ++e)
                     if (i + e >= sp.row0 && i + e < sp.row1) {
                         out_a[e] = ac[e];
-                        out_w[e] = ww[e];
+                        if (!kGiven) out_w[e] = ww[e];
                         lo = fminf(lo, ac[e]), hi = fmaxf(hi, ac[e]);
                     }
             }
@@ -606,10 +616,10 @@ __device__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __rest
     }
 }
 
-template <typename T, int D>
+template <typename T, int D, bool kGiven>
 __global__ void __launch_bounds__(kThreads, 1)
 gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblocks, int units, int H, int N, bool keep_in_l2,
-                 float* __restrict__ block_sums, float* __restrict__ inv_norm, int64_t inv_row, float* __restrict__ a_raw,
+                 const float* __restrict__ given, float* __restrict__ block_sums, float* __restrict__ inv_norm, int64_t inv_row, float* __restrict__ a_raw,
                  int64_t raw_row, uint32_t* __restrict__ mm, int* status) {
     using C = Cfg<D>;
     extern __shared__ unsigned char smem_raw[];
@@ -655,11 +665,11 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
         if (lane == 0) mma_role<T, D>(ring, s, tmem_base, walk, block, N, status);
         __syncwarp();
     } else if (warp >= kScanWarp0) {
-        scan_role<D>(s, walk, block, N, inv_norm, inv_row, a_raw, raw_row, mm, status);
+        scan_role<D, kGiven>(s, walk, block, N, inv_norm, inv_row, a_raw, raw_row, mm, status);
     } else if (warp >= kSumsWarp0) {
-        sums_role<T, D>(ring, s, walk, block, N, block_sums, status);
+        sums_role<T, D, kGiven>(ring, s, walk, block, N, block_sums, status);
     } else {
-        band_role<D>(s, tmem_base, walk, block, N, status);
+        band_role<D, kGiven>(s, tmem_base, walk, block, N, given, inv_row, status);
     }
 
     tc_fence_before();
@@ -686,12 +696,13 @@ EncodeTiledFn tensor_map_encoder() {
 
 template <typename T, int D>
 cudaError_t launch_typed(const CUtensorMap& tmap, const TensorView& K, int units, const ScoreParams& sp, bool keep_in_l2,
-                         float* block_sums, float* inv_norm, float* a_raw, uint32_t* mm, int* status, int sm_count,
+                         const float* given, float* block_sums, float* inv_norm, float* a_raw, uint32_t* mm, int* status, int sm_count,
                          cudaStream_t stream) {
     const long long total = (long long)units * sp.nblocks;
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
-    gram_pass_kernel<T, D><<<grid, kThreads, smem_bytes<D>(), stream>>>(tmap, sp.block, sp.nblocks, units, K.H, K.N, keep_in_l2,
-                                                                        block_sums, inv_norm, sp.inv_row, a_raw, sp.raw_row, mm, status);
+    auto kernel = given ? gram_pass_kernel<T, D, true> : gram_pass_kernel<T, D, false>;
+    kernel<<<grid, kThreads, smem_bytes<D>(), stream>>>(tmap, sp.block, sp.nblocks, units, K.H, K.N, keep_in_l2,
+                                                                        given, block_sums, inv_norm, sp.inv_row, a_raw, sp.raw_row, mm, status);
     return cudaGetLastError();
 }
 
@@ -715,7 +726,9 @@ cudaError_t encode_key_map(const TensorView& K, int dtype, int G, int box_rows, 
 cudaError_t configure_gram_kernels() {
     cudaError_t e;
 #define NKV_SET(T, D)                                                                                                    \
-    if ((e = cudaFuncSetAttribute(gram_pass_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,                   \
+    if ((e = cudaFuncSetAttribute(gram_pass_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
+                                  (int)smem_bytes<D>())) != cudaSuccess ||                                               \
+        (e = cudaFuncSetAttribute(gram_pass_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,             \
                                   (int)smem_bytes<D>())) != cudaSuccess)                                                  \
         return e
     NKV_SET(__nv_bfloat16, 64);
@@ -737,8 +750,10 @@ bool gram_pass_supported(const TensorView& K, int dtype, const ScoreParams& sp) 
     return encode_key_map(K, dtype, 1, kHalo, &probe) == cudaSuccess;
 }
 
-cudaError_t launch_gram_pass(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums, float* inv_norm,
-                             float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
+// With `given` the norms are the caller's (rows of sp.inv_row) and only a_c and its extremes are written: block_sums and
+// inv_norm are null.
+cudaError_t launch_gram_pass(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* given,
+                             float* block_sums, float* inv_norm, float* a_raw, uint32_t* mm, int* status, int sm_count, cudaStream_t stream,
                              int64_t* launches) {
     const int units = G * K.H;
     CUtensorMap tmap;
@@ -746,7 +761,7 @@ cudaError_t launch_gram_pass(const TensorView& K, int dtype, int G, const ScoreP
     if (e != cudaSuccess) return e;
     // keys that fit L2 (126 MB) beside the scores stay there for the second pass
     const bool keep = (int64_t)units * K.N * K.d * 2 <= ((int64_t)48 << 20);
-#define NKV_ARGS tmap, K, units, sp, keep, block_sums, inv_norm, a_raw, mm, status, sm_count, stream
+#define NKV_ARGS tmap, K, units, sp, keep, given, block_sums, inv_norm, a_raw, mm, status, sm_count, stream
     if (dtype == NKV_BF16) e = K.d == 128 ? launch_typed<__nv_bfloat16, 128>(NKV_ARGS) : launch_typed<__nv_bfloat16, 64>(NKV_ARGS);
     else e = K.d == 128 ? launch_typed<__half, 128>(NKV_ARGS) : launch_typed<__half, 64>(NKV_ARGS);
 #undef NKV_ARGS
