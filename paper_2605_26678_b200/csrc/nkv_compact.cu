@@ -26,6 +26,7 @@ struct GatherArgs {
 __global__ void __launch_bounds__(256) gather_kernel(GatherArgs A, const int32_t* __restrict__ idx,
                                                      const int32_t* __restrict__ head_offsets) {
     __shared__ int64_t src_off[2][kGatherRows];
+    pdl_wait();
     const int64_t nbatch = (A.total_rows + kGatherRows - 1) / kGatherRows;
     const int cpr0 = A.row_bytes[0] >> 4, cpr1 = A.dst[1] ? (A.row_bytes[1] >> 4) : 0;   // 16-byte chunks per row
     const int total0 = A.dst[0] ? kGatherRows * cpr0 : 0, total = total0 + kGatherRows * cpr1;
@@ -158,9 +159,8 @@ cudaError_t launch_gather(const TensorView& K, int k_elem_bytes, const TensorVie
     if (nbatch == 0) return cudaSuccess;
     int64_t grid = ctas_or_0 ? ctas_or_0 : (int64_t)sm_count * 8;
     if (grid > nbatch) grid = nbatch;
-    gather_kernel<<<(unsigned)grid, 256, 0, stream>>>(A, idx, head_offsets);
     ++*launches;
-    return cudaGetLastError();
+    return launch_chained(gather_kernel, (unsigned)grid, 256, 0, stream, 1, A, idx, head_offsets);
 }
 
 cudaError_t launch_gather_in_place(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,

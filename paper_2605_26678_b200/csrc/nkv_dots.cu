@@ -295,6 +295,7 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = s->tmem_base;
+    pdl_wait();
 
     if (warp == kProducerWarp) {
         if (lane == 0) dots_producer<D>(&tmap, tiles, s, tr, H, status);
@@ -350,9 +351,9 @@ cudaError_t launch_anchor_dots(const TensorView& K, int dtype, int G, const Scor
     const int units = G * K.H;
     const long long total = (long long)units * ((K.N + kTile - 1) / kTile);
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
-#define NKV_DOTS(T, D)                                                                                                \
-    anchor_dots_kernel<T, D><<<grid, kThreads, smem_bytes<D>(), stream>>>(tmap, sp, units, K.H, K.N, mu_s, mu_e,     \
-                                                                          inv_norm, inv_s, inv_e, a_raw, mm, status)
+#define NKV_DOTS(T, D)                                                                                                    \
+    e = launch_chained(anchor_dots_kernel<T, D>, grid, kThreads, smem_bytes<D>(), stream, 1, tmap, sp, units, K.H, K.N,  \
+                       mu_s, mu_e, inv_norm, inv_s, inv_e, a_raw, mm, status)
     if (dtype == NKV_BF16) {
         if (K.d == 128) NKV_DOTS(__nv_bfloat16, 128);
         else NKV_DOTS(__nv_bfloat16, 64);
@@ -362,7 +363,7 @@ cudaError_t launch_anchor_dots(const TensorView& K, int dtype, int G, const Scor
     }
 #undef NKV_DOTS
     ++*launches;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace nkv

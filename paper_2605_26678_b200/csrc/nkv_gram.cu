@@ -656,6 +656,7 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = s->tmem_base;
+    pdl_wait();
     const Walk walk = my_walk(units, nblocks);
 
     if (warp == kProducerWarp) {
@@ -701,9 +702,8 @@ cudaError_t launch_typed(const CUtensorMap& tmap, const TensorView& K, int units
     const long long total = (long long)units * sp.nblocks;
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
     auto kernel = given ? gram_pass_kernel<T, D, true> : gram_pass_kernel<T, D, false>;
-    kernel<<<grid, kThreads, smem_bytes<D>(), stream>>>(tmap, sp.block, sp.nblocks, units, K.H, K.N, keep_in_l2,
-                                                                        given, block_sums, inv_norm, sp.inv_row, a_raw, sp.raw_row, mm, status);
-    return cudaGetLastError();
+    return launch_chained(kernel, grid, kThreads, smem_bytes<D>(), stream, 1, tmap, sp.block, sp.nblocks, units, K.H, K.N, keep_in_l2, given,
+                          block_sums, inv_norm, sp.inv_row, a_raw, sp.raw_row, mm, status);
 }
 
 }  // namespace

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(kMeanWarps * 32) anchor_means_kernel(int N, Sc
                                                                        float* __restrict__ mu_s, float* __restrict__ inv_e,
                                                                        float* __restrict__ inv_s) {
     constexpr int P = D / 32;   // columns per lane: lane, lane + 32, ...
+    pdl_wait();
     __shared__ float part[kMeanWarps][D];
     const int u = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = sp.nblocks;
     float* rows = mu_e + (int64_t)u * nb * D;
@@ -430,14 +431,9 @@ cudaError_t launch_anchor_sums(const TensorView& K, int dtype, int G, const Scor
 cudaError_t launch_anchor_means(int units, int N, int d, const ScoreParams& sp, float* mu_e_inout, float* mu_s,
                                 float* inv_mu_e_norm_or_null, float* inv_mu_s_norm_or_null, cudaStream_t stream,
                                 int64_t* launches) {
-    if (d == 128)
-        anchor_means_kernel<128><<<units, kMeanWarps * 32, 0, stream>>>(N, sp, mu_e_inout, mu_s, inv_mu_e_norm_or_null,
-                                                                        inv_mu_s_norm_or_null);
-    else
-        anchor_means_kernel<64><<<units, kMeanWarps * 32, 0, stream>>>(N, sp, mu_e_inout, mu_s, inv_mu_e_norm_or_null,
-                                                                       inv_mu_s_norm_or_null);
     ++*launches;
-    return cudaGetLastError();
+    return launch_chained(d == 128 ? anchor_means_kernel<128> : anchor_means_kernel<64>, (unsigned)units, kMeanWarps * 32, 0, stream, 1, N,
+                          sp, mu_e_inout, mu_s, inv_mu_e_norm_or_null, inv_mu_s_norm_or_null);
 }
 
 cudaError_t launch_anchor_norms(int units, int d, const ScoreParams& sp, const float* mu_s, const float* mu_e,

@@ -264,6 +264,7 @@ stream_a_kernel(TensorView K, ScoreParams sp, int units, float* __restrict__ blo
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();
 
     auto issue = [&](long long t, int buf) {   // thread 0 only
         const int u = (int)(t / tiles_per_unit);
@@ -480,6 +481,7 @@ stream_b_kernel(TensorView K, ScoreParams sp, int units, const float* __restrict
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();
 
     auto issue = [&](long long t, int buf) {
         const int u = (int)(t / tiles_per_unit);
@@ -637,14 +639,14 @@ cudaError_t launch_stream_a(const TensorView& K, int dtype, int G, const ScorePa
     }
     const long long total = (long long)units * ((K.N + tile - 1) / tile);
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
-#define CALL(T, D)                                                                                         \
-    stream_a_kernel<T, D, Tiles<T, D>::A><<<grid, ACfg<T, D, Tiles<T, D>::A>::kThreads,                       \
-                                            ACfg<T, D, Tiles<T, D>::A>::kSmem, stream>>>(                    \
-        K, sp, units, block_sums, inv_norm, a_raw, mm, status)
+#define CALL(T, D)                                                                                                     \
+    e = launch_chained(stream_a_kernel<T, D, Tiles<T, D>::A>, grid, ACfg<T, D, Tiles<T, D>::A>::kThreads,                   \
+                       ACfg<T, D, Tiles<T, D>::A>::kSmem, stream, 1, K, sp, units, block_sums, inv_norm, a_raw, mm, status)
+    cudaError_t e;
     NKV_DISPATCH(dtype, K.d, CALL);
 #undef CALL
     ++*launches;
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_stream_b(const TensorView& K, int dtype, int G, const ScoreParams& sp, const float* mu_s,
@@ -658,14 +660,14 @@ cudaError_t launch_stream_b(const TensorView& K, int dtype, int G, const ScorePa
 #undef CALL
     const long long total = (long long)units * ((K.N + tile - 1) / tile);
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
-#define CALL(T, D)                                                                                         \
-    stream_b_kernel<T, D, Tiles<T, D>::B><<<grid, BCfg<T, D, Tiles<T, D>::B>::kThreads,                       \
-                                            BCfg<T, D, Tiles<T, D>::B>::kSmem, stream>>>(                    \
-        K, sp, units, mu_s, mu_e, inv_norm, inv_s, inv_e, a_raw, mm, status)
+#define CALL(T, D)                                                                                                     \
+    e = launch_chained(stream_b_kernel<T, D, Tiles<T, D>::B>, grid, BCfg<T, D, Tiles<T, D>::B>::kThreads,                   \
+                       BCfg<T, D, Tiles<T, D>::B>::kSmem, stream, 1, K, sp, units, mu_s, mu_e, inv_norm, inv_s, inv_e, a_raw, mm, status)
+    cudaError_t e;
     NKV_DISPATCH(dtype, K.d, CALL);
 #undef CALL
     ++*launches;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace nkv
