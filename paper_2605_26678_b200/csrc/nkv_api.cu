@@ -61,7 +61,7 @@ int64_t keep_count(int64_t N, double r) { return (int64_t)floor((1.0 - r) * (dou
 
 // Workspace carving shared by every entry point.
 struct Layout {
-    size_t status, mm, inv_norm, mu_s, mu_e, inv_s, inv_e, a_raw, a_star, thr, total;
+    size_t status, mm, inv_norm, mu_s, mu_e, inv_s, inv_e, a_raw, a_star, hist, total;
 };
 
 // Rows of the per-token arrays start on 16-byte boundaries, so that ragged lengths keep the four-wide accesses.
@@ -85,7 +85,7 @@ Layout make_layout(int64_t units, int64_t N, int64_t d, int64_t nb) {
     L.inv_e = take((size_t)units * nb * 4);
     L.a_raw = take((size_t)units * 3 * row);
     L.a_star = take((size_t)units * row);
-    L.thr = take((size_t)units * 2 * 4);
+    L.hist = take(score_hist_bytes(units));
     L.total = o;
     return L;
 }
@@ -568,7 +568,7 @@ static int compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, dou
     const Bufs B = bufs_at(ws, L);
     if ((rc = key_scan(h, kv, K->dtype, G, sp, B, status, st, mark))) return rc;
     CU(mark());
-    CU(launch_score_to_select(G, H, N, sp, (int)keep, (int)n_safe, B.a_raw, B.mm, a_star, star_row, at<uint32_t>(ws, L.thr), budgets, idx,
+    CU(launch_score_to_select(G, H, N, sp, (int)keep, (int)n_safe, B.a_raw, B.mm, a_star, star_row, at<int>(ws, L.hist), budgets, idx,
                               (int64_t)H * keep, head_offsets, status, st, &h->launches));
     CU(mark());
     CU(mark());   // the budget and select stages are part of that call
