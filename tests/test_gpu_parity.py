@@ -535,6 +535,27 @@ def test_score_to_select_in_every_layout(layers, H, N, d):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("safeguard", [0.0, 0.9, 1.0])
+@pytest.mark.parametrize("layers,H,N", [(3, 8, 701), (2, 3, 30011), (30, 12, 900)])
+def test_safeguard_that_no_head_and_some_head_needs(layers, H, N, safeguard):
+    """Heads that compete once, and twice because one came out short of its safeguard; scores of one launch and of two."""
+    K, V = _cache(N, 64, "bf16", H=H, layers=layers)
+    p = nkv.nkv_default_params()
+    p.safeguard = safeguard
+    ws = nkv.alloc_workspace(K, p)
+    res = nkv.nkv_compress(K, V, 0.75, p, ws=ws, want_a_star=True)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    n_safe = nkv.nkv_safeguard_count(N, 0.75, p)
+    assert int(res.budgets.min()) >= n_safe
+    for g in {0, layers - 1}:
+        own = oracle.budget_select(res.a_star[g].cpu().numpy(), 0.75, pr.oracle_params(p))
+        assert np.array_equal(own.budgets, res.budgets[g].cpu().numpy())
+        assert np.array_equal(own.idx, res.idx[g].cpu().numpy())
+        if safeguard == 0.9:
+            assert (own.budgets == n_safe).any()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("layers,chunk,r,pinned", [(5, 1, 0.75, True), (7, 3, 0.75, True), (4, 4, 0.25, True), (3, 2, 0.75, False)])
 def test_host_entry_point_with_rows_fetched_in_place_and_copied(layers, chunk, r, pinned):
     """Retained rows of V read from pinned memory, and V copied whole (most rows retained, or memory that the device
