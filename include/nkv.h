@@ -266,8 +266,8 @@ NKV_API int64_t nkv_launch_count(const nkv_handle* h);
  *       matrix, and ||k_i||^2 as its diagonal; in the second pass the dots of the keys with the anchors, the
  *       fp32 anchors split three ways into the keys' type.  A call whose inputs do not allow the tensor form runs
  *       the FMA kernels.
- *   NKV_KEY_PASS_AUTO (default) takes the tensor form of the first pass where its inputs allow it, and of the
- *       second when in addition d = 128 or the FMA form does not take the block size.
+ *   NKV_KEY_PASS_AUTO (default) takes the tensor form where the inputs allow it and the call has enough keys for it to be
+ *       the faster one, or the FMA form does not take the block size.
  * The forms agree to fp32 rounding.
  */
 enum { NKV_KEY_PASS_AUTO = 0, NKV_KEY_PASS_FMA = 1, NKV_KEY_PASS_TENSOR = 2 };

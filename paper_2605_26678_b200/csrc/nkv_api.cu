@@ -180,12 +180,23 @@ Bufs bufs_at(void* ws, const Layout& L) {
     return b;
 }
 
+// Whether the tensor form of a key pass is the better one where both are there.  It is bound by the read of the keys (the
+// first pass: by half the FMA form's instructions), but its roles take 1 to 2 us longer to get going.  Whole calls with both
+// passes in the FMA form / the second / none, H = 8, r = 0.75, bf16, us:
+//     d = 64    17 MB of keys 52 / 54 / 56   33 MB 69 / 70 / 69   67 MB 106 / 100 / 99 (64 x 8192), 99 / 102 / 102 (128 x 4096)
+//     d = 128   17 MB 53 / 54 / 54           33 MB 66 / 62 / 62   67 MB 98 / 84 / 84
+// With keys that are not in L2, 33 MB of 16 x 8 x 2048 x 64: 85.5 / - / 85.8, and 84.9 with only the first in tensor form.
+constexpr int kFirstPassKb = 192, kSecondPassKb64 = 256, kSecondPassKb128 = 192;   // of keys per SM
+bool tensor_pays(const nkv_handle* h, const TensorView& kv, int G, const ScoreParams& sp, int kb) {
+    const int64_t bytes = (int64_t)G * kv.H * kv.N * kv.d * 2;
+    return h->key_pass == NKV_KEY_PASS_TENSOR || !stream_path_supported(sp) || bytes >= (int64_t)h->sm_count * kb * 1024;
+}
+
 // The second pass over the keys: a_s and a_e of every token from the anchors.
 int anchor_scores(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreParams& sp, const float* mu_s, const float* mu_e,
                   const float* inv_norm, const Bufs& B, float* a_raw, int* status, cudaStream_t st) {
-    // d = 64 tiles are too small to pay for the per-tile hand-overs: the FMA form is faster there
     const bool tensor = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
-                        (h->key_pass == NKV_KEY_PASS_TENSOR || kv.d == 128 || !stream_path_supported(sp));
+                        tensor_pays(h, kv, G, sp, kv.d == 64 ? kSecondPassKb64 : kSecondPassKb128);
     if (tensor)
         CU(launch_anchor_dots(kv, dtype, G, sp, mu_s, mu_e, inv_norm, B.inv_s, B.inv_e, a_raw, B.mm, status, h->sm_count, st,
                               &h->launches));
@@ -203,7 +214,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
              cudaStream_t st, Mark&& mark) {
     const int units = G * kv.H, N = kv.N, d = kv.d;
     const bool tensor_a = h->key_pass != NKV_KEY_PASS_FMA && gram_pass_supported(kv, dtype, sp) &&
-                          anchor_dots_supported(kv, dtype, sp);
+                          anchor_dots_supported(kv, dtype, sp) && tensor_pays(h, kv, G, sp, kFirstPassKb);
     if (!tensor_a && !stream_path_supported(sp)) {
         CU(launch_anchor_sums(kv, dtype, G, sp, B.mu_e, B.inv_norm, st, &h->launches));
         CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, B.inv_e, B.inv_s, st, &h->launches));

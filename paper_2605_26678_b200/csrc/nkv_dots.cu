@@ -7,11 +7,18 @@
 // vectors, are scaled by 2^10, which brings lo's quantum to 2^-34 of the anchors' scale), so a tile's right-hand
 // side is
 //     columns 0..2  mu_s        3..5  mu_e of the block the tile starts in        6..8  mu_e of the next block
-// (a tile of 128 keys touches at most two blocks because a block has at least 128 keys).  Key tiles are
-// staged by TMA (128-byte swizzle) several tiles ahead; the tensor core reads them from shared memory
-// directly, so the SM issues a few dozen instructions per tile and the pass runs at the speed of the
-// copy.  Warp roles: TMA producer, MMA issuer, four warps that build the right-hand sides, four warps
-// that turn the accumulator into scores.  Every wait is bounded.
+// (a tile of 128 keys touches at most two blocks because a block has at least 128 keys).  Key tiles are staged by TMA
+// (128-byte swizzle); the tensor core reads them from shared memory directly.  Warp roles: TMA producer, two MMA
+// issuers, four warps that build the right-hand sides, four warps that turn the accumulator into scores.  Every wait is
+// bounded.
+//
+// Bound: the read of the keys; no role may then need more than the 1300 cycles in which a tile of 32 KB arrives.  What
+// that took: places in the tensors are counted, not divided out (tile), right-hand sides are built per block and not per
+// tile, the rows' norms and the anchors come by asynchronous copies several tiles ahead, and two threads issue the
+// products in turn (one needs 1050 cycles per tile of 128 columns, 790 per tile of 64).  128 KB of keys in flight per SM:
+// a bare read of 604 MB in 32 KB pieces takes 101 us with 96 KB in flight per SM, 107 with 160 or 192.
+// 16 x 8 heads of 32768 x 64 bf16 keys: 141 -> 98 us (and 141 in the FMA form of nkv_stream.cu); 36 x 8 x 8192 x 128:
+// 109 -> 106; 36 x 8 x 131072 x 128: 1910 -> 1475 (6.7 TB/s).
 #include "nkv_sm100.cuh"
 
 namespace nkv {
@@ -26,108 +33,181 @@ constexpr int kRhsHalfBytes = 16 * 128;           // 16 right-hand-side rows of 
 constexpr int kStages = 4;                        // accumulators of 32 columns (16 used)
 constexpr uint32_t kTmemCols = 128;
 constexpr int kPrepWarp0 = 0, kEpiWarp0 = 4, kProducerWarp = 8, kMmaWarp = 9;
-constexpr int kThreads = 10 * 32;
-constexpr int kMaxSlots = 10;
+constexpr int kMmaWarps = 2;                      // they take the tiles in turn
+constexpr int kThreads = (9 + kMmaWarps) * 32;
+constexpr int kMaxSlots = 8;
+constexpr int kRhs = 4;                           // right-hand sides kept at once
+constexpr int kAhead = 8;                         // tiles (blocks) whose per-row inputs (anchors) are on their way
 
 // Sizes for head dimension D (64 or 128): a key row is D / 64 swizzled halves of 128 bytes.
 template <int D>
 struct Cfg {
     static constexpr int kHalves = D / 64;
-    static constexpr int kSlots = 640 / D;                       // key tiles staged at once (160 KB)
+    static constexpr int kSlots = 512 / D;                       // key tiles staged at once (128 KB)
     static constexpr int kTileBytes = kHalves * kTileHalfBytes;
     static constexpr int kRhsBytes = kHalves * kRhsHalfBytes;
     static constexpr int kPrepWarps = D / 32;                    // one thread per column
+    static constexpr size_t kRhsAt = (size_t)kSlots * kTileBytes;             // offsets of the parts behind the tiles
+    static constexpr size_t kRowsAt = kRhsAt + (size_t)kRhs * kRhsBytes;      // [kAhead][2][kTile] floats
+    static constexpr size_t kMuAt = kRowsAt + (size_t)kAhead * 2 * kTile * 4; // [kAhead][D] floats
+    static constexpr size_t kSmemAt = kMuAt + (size_t)kAhead * D * 4;
     static_assert(kSlots <= kMaxSlots, "barrier arrays too small");
+    // an issuer has then itself waited for the round before the one that it waits for, so parities are unambiguous
+    static_assert(kSlots % kMmaWarps == 0 && kStages % kMmaWarps == 0, "a slot or stage belongs to one issuer");
 };
 
 struct Smem {
     uint64_t full[kMaxSlots];   // key tile landed
-    uint64_t rready[kMaxSlots]; // right-hand side written (one arrival per building warp)
-    uint64_t kfree[kMaxSlots];  // tile and right-hand side consumed by the MMAs
+    uint64_t kfree[kMaxSlots];  // tile consumed by the MMAs
+    uint64_t rready[kRhs];      // right-hand side written (one arrival per building warp)
+    uint64_t rfree[kRhs];       // consumed by the MMAs of all its tiles
     uint64_t tfull[kStages];    // accumulator written
     uint64_t tempty[kStages];   // accumulator read (one arrival per reading warp)
-    uint64_t drain;             // products issued before a give-up have completed
+    uint64_t drain[kMmaWarps];  // products issued before a give-up have completed
     uint32_t tmem_base;
 };
 template <int D>
 constexpr size_t smem_bytes() {
-    return 1024 + (size_t)Cfg<D>::kSlots * (Cfg<D>::kTileBytes + Cfg<D>::kRhsBytes) + sizeof(Smem);
+    return 1024 + Cfg<D>::kSmemAt + sizeof(Smem);
 }
 
+// A CTA's tiles: `count` of them from tile `first` on, counted through the heads.
 struct TileRange {
-    long long first, last;      // this CTA's tiles [first, last)
-    int tiles_per_unit;
+    long long first;
+    int count, tiles_per_unit;
 };
 __device__ __forceinline__ TileRange my_tiles(int units, int N) {
     TileRange r;
     r.tiles_per_unit = (N + kTile - 1) / kTile;
     const long long total = (long long)units * r.tiles_per_unit;
     r.first = total * blockIdx.x / gridDim.x;
-    r.last = total * (blockIdx.x + 1) / gridDim.x;
+    r.count = (int)(total * (blockIdx.x + 1) / gridDim.x - r.first);
     return r;
 }
+// Where a role is: head, first key of the tile, the block it lies in and that block's end.  Every role steps through the
+// tiles on its own; the steps are additions (a division per tile and role cost as much as the rest of its work).
+struct Place {
+    int u, i0, blk, blk_end;
+    __device__ __forceinline__ Place(TileRange tr, int block) {
+        u = (int)(tr.first / tr.tiles_per_unit);
+        i0 = (int)(tr.first - (long long)u * tr.tiles_per_unit) * kTile;
+        blk = i0 / block;
+        blk_end = (blk + 1) * block;
+    }
+    __device__ __forceinline__ bool next(int N, int block) {   // true: another head or block
+        i0 += kTile;
+        if (i0 >= N) {
+            ++u;
+            i0 = blk = 0;
+            blk_end = block;
+            return true;
+        }
+        if (i0 < blk_end) return false;   // a block has at least kTile keys, so it is the next one otherwise
+        ++blk;
+        blk_end += block;
+        return true;
+    }
+};
+// Position in a ring and the parity of the round.
+template <int kSize>
+struct Ring {
+    int at = 0;
+    uint32_t round = 0;
+    __device__ __forceinline__ void next() {
+        if (++at == kSize) {
+            at = 0;
+            round ^= 1u;
+        }
+    }
+};
+
+// Four bytes into shared memory behind the thread's back.  (Loads into registers that are due several tiles later share a
+// handful of scoreboards with newer ones and get waited for too early: 12 tiles ahead was slower than one.)
+__device__ __forceinline__ void copy4(float* dst_smem, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst_smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
 
 // ---------------------------------------------------------------------------- roles
 template <int D>
-__device__ void dots_producer(const CUtensorMap* tmap, unsigned char* tiles, Smem* s, TileRange tr, int H, int* status) {
+__device__ void dots_producer(const CUtensorMap* tmap, unsigned char* tiles, Smem* s, TileRange tr, int H, int N, int* status) {
     using C = Cfg<D>;
-    long long n = 0;
     const uint64_t policy = l2_evict_first_policy();   // keys are read once per pass
-    for (long long t = tr.first; t < tr.last; ++t, ++n) {
-        const int slot = (int)(n % C::kSlots);
-        const long long fill = n / C::kSlots;
-        if (fill > 0 && !mbar_wait(&s->kfree[slot], (uint32_t)((fill - 1) & 1), status, 711)) {
+    Ring<C::kSlots> slot;
+    int u = (int)(tr.first / tr.tiles_per_unit), i0 = (int)(tr.first - (long long)u * tr.tiles_per_unit) * kTile;
+    int g = u / H, h = u - g * H;
+    for (int n = 0; n < tr.count; ++n, slot.next()) {
+        if (n >= C::kSlots && !mbar_wait(&s->kfree[slot.at], slot.round ^ 1u, status, 711)) {
             // giving up: the copies already armed still land in this CTA's shared memory, so stay (bounded)
             // until they have
-            for (long long m = n > C::kSlots ? n - C::kSlots : 0; m < n; ++m)
+            for (int m = n - C::kSlots; m < n; ++m)
                 for (uint32_t spin = 0; spin < (1u << 16) && !mbar_try_wait(&s->full[m % C::kSlots], (uint32_t)((m / C::kSlots) & 1)); ++spin)
                     __nanosleep(256);
             return;
         }
-        const int u = (int)(t / tr.tiles_per_unit);
-        const int i0 = (int)(t - (long long)u * tr.tiles_per_unit) * kTile;
-        const int g = u / H, h = u - g * H;
-        unsigned char* dst = tiles + (size_t)slot * C::kTileBytes;
-        mbar_expect_tx(&s->full[slot], C::kTileBytes);
+        unsigned char* dst = tiles + (size_t)slot.at * C::kTileBytes;
+        mbar_expect_tx(&s->full[slot.at], C::kTileBytes);
 #pragma unroll
         for (int half = 0; half < C::kHalves; ++half)
-            tma_load_4d(dst + half * kTileHalfBytes, tmap, 64 * half, i0, h, g, &s->full[slot], policy);
+            tma_load_4d(dst + half * kTileHalfBytes, tmap, 64 * half, i0, h, g, &s->full[slot.at], policy);
+        i0 += kTile;
+        if (i0 >= N) {
+            i0 = 0;
+            if (++h == H) {
+                h = 0;
+                ++g;
+            }
+        }
     }
 }
 
 template <typename T, int D>
-__device__ void dots_mma(unsigned char* tiles, unsigned char* rhs, Smem* s, uint32_t tmem_base, TileRange tr,
+__device__ void dots_mma(int which, unsigned char* tiles, unsigned char* rhs, Smem* s, uint32_t tmem_base, TileRange tr, int N, int block,
                          int* status) {
     using C = Cfg<D>;
     constexpr uint32_t idesc = umma_idesc<T>(kTile, 16);
-    const uint32_t tiles_addr = smem_addr(tiles), rhs_addr = smem_addr(rhs);
-    long long n = 0;
-    for (long long t = tr.first; t < tr.last; ++t, ++n) {
-        const int slot = (int)(n % C::kSlots), stage = (int)(n % kStages);
-        const uint32_t fpar = (uint32_t)((n / C::kSlots) & 1), upar = (uint32_t)((n / kStages) & 1);
-        if (!mbar_wait(&s->full[slot], fpar, status, 712) || !mbar_wait(&s->rready[slot], fpar, status, 713) ||
-            !mbar_wait(&s->tempty[stage], upar ^ 1u, status, 714)) {
+    const uint64_t tiles_desc = umma_desc_sw128(smem_addr(tiles)), rhs_desc = umma_desc_sw128(smem_addr(rhs));
+    Ring<C::kSlots> slot;
+    Ring<kStages> stage;
+    Ring<kRhs> r;
+    Place at(tr, block);
+    bool fresh = true, used = false;   // another right-hand side; products of this thread have read it
+    for (int n = 0; n < tr.count; ++n, slot.next(), stage.next()) {
+        const bool mine = n % kMmaWarps == which;
+        // (a thread without a tile of the block waits too: its arrival below must not count for an earlier round)
+        if ((fresh && !mbar_wait(&s->rready[r.at], r.round, status, 713)) ||
+            (mine && (!mbar_wait(&s->tempty[stage.at], stage.round ^ 1u, status, 714) ||
+                      !mbar_wait(&s->full[slot.at], slot.round, status, 712)))) {
             // products already issued keep reading shared memory and writing tensor memory: wait (bounded)
             // for them before the CTA frees both
-            umma_commit(&s->drain);
-            for (uint32_t spin = 0; spin < (1u << 16) && !mbar_try_wait(&s->drain, 0); ++spin) __nanosleep(256);
+            umma_commit(&s->drain[which]);
+            for (uint32_t spin = 0; spin < (1u << 16) && !mbar_try_wait(&s->drain[which], 0); ++spin) __nanosleep(256);
             return;
         }
-        tc_fence_after();
+        if (mine) {
+            tc_fence_after();
+            const uint64_t a = tiles_desc + (uint32_t)(slot.at * C::kTileBytes >> 4), b = rhs_desc + (uint32_t)(r.at * C::kRhsBytes >> 4);
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t a = tiles_addr + (uint32_t)slot * C::kTileBytes + (uint32_t)(kk >> 2) * kTileHalfBytes +
-                               (uint32_t)(kk & 3) * 32u;
-            const uint32_t b = rhs_addr + (uint32_t)slot * C::kRhsBytes + (uint32_t)(kk >> 2) * kRhsHalfBytes +
-                               (uint32_t)(kk & 3) * 32u;
-            umma_f16(tmem_base + (uint32_t)stage * 32u, umma_desc_sw128(a), umma_desc_sw128(b), idesc, kk > 0);
+            for (int kk = 0; kk < D / 16; ++kk)
+                umma_f16(tmem_base + (uint32_t)stage.at * 32u, a + (uint32_t)((kk >> 2) * kTileHalfBytes + (kk & 3) * 32 >> 4),
+                         b + (uint32_t)((kk >> 2) * kRhsHalfBytes + (kk & 3) * 32 >> 4), idesc, kk > 0);
+            umma_commit(&s->tfull[stage.at]);
+            umma_commit(&s->kfree[slot.at]);
+            used = true;
         }
-        umma_commit(&s->tfull[stage]);
-        umma_commit(&s->kfree[slot]);
+        fresh = at.next(N, block);
+        if (fresh && n + 1 < tr.count) {
+            if (used) umma_commit(&s->rfree[r.at]);
+            else mbar_arrive(&s->rfree[r.at]);
+            used = false;
+            r.next();
+        }
     }
 }
 
-// Thread k writes column k of the nine right-hand-side rows of every tile (rows 9..15 stay zero).
+// Thread k writes column k of the nine right-hand-side rows of every block (rows 9..15 stay zero).
 template <typename T> constexpr float kAnchorScale = 1.f;
 template <> constexpr float kAnchorScale<__half> = 1024.f;
 template <typename T> __device__ __forceinline__ T narrow(float v);
@@ -136,30 +216,41 @@ template <> __device__ __forceinline__ __half narrow<__half>(float v) { return _
 template <typename T> __device__ __forceinline__ float widen(T v) { return (float)v; }
 
 template <typename T, int D>
-__device__ void dots_prep(unsigned char* rhs, Smem* s, ScoreParams sp, TileRange tr, const float* __restrict__ mu_s,
-                          const float* __restrict__ mu_e, int* status) {
+__device__ void dots_prep(unsigned char* rhs, float* mu, Smem* s, ScoreParams sp, TileRange tr, int units, int N,
+                          const float* __restrict__ mu_s, const float* __restrict__ mu_e, int* status) {
     using C = Cfg<D>;
     const int k = threadIdx.x - kPrepWarp0 * 32, lane = k & 31;
     if (k >= D) return;   // d = 64 needs two of the four warps
     const int half = k >> 6, kk = k & 63;
-    float v[3] = {0.f, 0.f, 0.f};
-    int cur_u = -1, cur_blk = -1;
-    long long n = 0;
-    for (long long t = tr.first; t < tr.last; ++t, ++n) {
-        const int slot = (int)(n % C::kSlots);
-        const long long fill = n / C::kSlots;
-        if (fill > 0 && !mbar_wait(&s->kfree[slot], (uint32_t)((fill - 1) & 1), status, 715)) return;
-        const int u = (int)(t / tr.tiles_per_unit);
-        const int i0 = (int)(t - (long long)u * tr.tiles_per_unit) * kTile;
-        const int blk0 = i0 / sp.block;
-        if (u != cur_u || blk0 != cur_blk) {   // the anchors change every few tiles only
-            if (u != cur_u) v[0] = mu_s[(int64_t)u * D + k];
-            v[1] = mu_e[((int64_t)u * sp.nblocks + blk0) * D + k];
-            v[2] = blk0 + 1 < sp.nblocks ? mu_e[((int64_t)u * sp.nblocks + blk0 + 1) * D + k] : 0.f;
-            cur_u = u;
-            cur_blk = blk0;
+    Place at(tr, sp.block);
+    // The anchors of a head's blocks follow one another, and the next head's come behind them: element k of row j of that
+    // sequence waits in mu[j % kAhead][k], fetched kAhead - 1 rows ahead.  A thread reads what it has copied itself.
+    const int64_t rows = (int64_t)units * sp.nblocks;
+    int64_t row = (int64_t)at.u * sp.nblocks + at.blk, fetched = row;
+    auto fetch_to = [&](int64_t end) {
+        for (; fetched < end; ++fetched) {
+            if (fetched < rows) copy4(mu + (int)(fetched % kAhead) * D + k, mu_e + fetched * D + k);
+            copies_commit();
         }
-        unsigned char* base = rhs + (size_t)slot * C::kRhsBytes + (size_t)half * kRhsHalfBytes + (kk & 7) * 2;
+    };
+    int cur_u = -1;
+    float v[3] = {0.f, 0.f, 0.f}, s_next = mu_s[(int64_t)at.u * D + k];
+    Ring<kRhs> r;
+    bool fresh = true, wrapped = false;
+    for (int n = 0; n < tr.count; ++n, fresh = at.next(N, sp.block)) {
+        if (!fresh) continue;
+        row = (int64_t)at.u * sp.nblocks + at.blk;
+        fetch_to(row + kAhead);
+        copies_wait<kAhead - 2>();   // rows `row` and `row` + 1 are here
+        if (at.u != cur_u) {
+            cur_u = at.u;
+            v[0] = s_next;
+            if (cur_u + 1 < units) s_next = mu_s[(int64_t)(cur_u + 1) * D + k];
+        }
+        v[1] = mu[(int)(row % kAhead) * D + k];
+        v[2] = at.blk + 1 < sp.nblocks ? mu[(int)((row + 1) % kAhead) * D + k] : 0.f;
+        if (wrapped && !mbar_wait(&s->rfree[r.at], r.round ^ 1u, status, 715)) break;
+        unsigned char* base = rhs + (size_t)r.at * C::kRhsBytes + (size_t)half * kRhsHalfBytes + (kk & 7) * 2;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const float x = v[a] * kAnchorScale<T>;
@@ -170,20 +261,22 @@ __device__ void dots_prep(unsigned char* rhs, Smem* s, ScoreParams sp, TileRange
             const T part[3] = {hi, mid, lo};
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const int row = 3 * a + j;   // row of the right-hand side, 8-row groups 1024 bytes apart
-                *reinterpret_cast<T*>(base + (row >> 3) * 1024 + (row & 7) * 128 +
-                                                  ((((kk >> 3) ^ (row & 7))) << 4)) = part[j];
+                const int line = 3 * a + j;   // row of the right-hand side, 8-row groups 1024 bytes apart
+                *reinterpret_cast<T*>(base + (line >> 3) * 1024 + (line & 7) * 128 + ((((kk >> 3) ^ (line & 7))) << 4)) = part[j];
             }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads these writes
         __syncwarp();
-        if (lane == 0) mbar_arrive(&s->rready[slot]);
+        if (lane == 0) mbar_arrive(&s->rready[r.at]);
+        r.next();
+        wrapped = wrapped || r.at == 0;
     }
+    copies_wait<0>();
 }
 
 // Thread r reads row r of the accumulator: the key's dots with mu_s and with the two candidate mu_e.
 template <typename T>
-__device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileRange tr, int N,
+__device__ void dots_epilogue(Smem* s, float* rows, uint32_t tmem_base, ScoreParams sp, TileRange tr, int units, int N,
                               const float* __restrict__ inv_norm, const float* __restrict__ inv_s,
                               const float* __restrict__ inv_e, float* __restrict__ a_raw, uint32_t* __restrict__ mm,
                               int* status) {
@@ -206,58 +299,58 @@ __device__ void dots_epilogue(Smem* s, uint32_t tmem_base, ScoreParams sp, TileR
         lo_s = lo_e = INFINITY;
         hi_s = hi_e = -INFINITY;
     };
-    // per-tile inputs of this thread's row, fetched one tile ahead of their use
-    struct RowIn {
-        int u, i;
-        bool second;
-        float inv_i, re;
-    };
-    auto fetch = [&](long long t) {
-        RowIn x;
-        x.u = (int)(t / tr.tiles_per_unit);
-        const int i0 = (int)(t - (long long)x.u * tr.tiles_per_unit) * kTile;
-        const int blk0 = i0 / sp.block;
-        x.i = i0 + r;
-        x.second = x.i >= (blk0 + 1) * sp.block;   // the key lies in the block after the tile's first
-        const int blk = min(blk0 + (x.second ? 1 : 0), sp.nblocks - 1);
-        x.inv_i = x.i < N ? inv_norm[x.u * sp.inv_row + x.i] : 0.f;
-        x.re = inv_e[(int64_t)x.u * sp.nblocks + blk];
-        return x;
-    };
-    long long n = 0;
-    RowIn nxt = {};
-    if (tr.first < tr.last) nxt = fetch(tr.first);
-    for (long long t = tr.first; t < tr.last; ++t, ++n) {
-        const int stage = (int)(n % kStages);
-        const RowIn cur = nxt;
-        if (t + 1 < tr.last) nxt = fetch(t + 1);
-        if (cur.u != cur_u) {
-            flush();
-            cur_u = cur.u;
-            rs = inv_s[cur.u];
+    // 1 / ||k|| and 1 / ||mu_e|| of this thread's row, copied kAhead tiles ahead: with the key copies of a whole ring queued
+    // in front of them such loads take microseconds
+    Place to(tr, sp.block), at = to;
+    auto fetch = [&](int n) {
+        if (n < tr.count) {
+            float* dst = rows + (n % kAhead) * 2 * kTile + r;
+            const int i = min(to.i0 + r, N - 1);
+            copy4(dst, inv_norm + to.u * sp.inv_row + i);
+            copy4(dst + kTile, inv_e + (int64_t)to.u * sp.nblocks + to.blk + (i >= to.blk_end ? 1 : 0));
+            to.next(N, sp.block);
         }
-        if (!mbar_wait(&s->tfull[stage], (uint32_t)((n / kStages) & 1), status, 716)) return;
+        copies_commit();
+    };
+    for (int k = 0; k < kAhead; ++k) fetch(k);
+    Ring<kStages> stage;
+    float rs_next = tr.count > 0 ? inv_s[at.u] : 0.f;
+    for (int n = 0; n < tr.count; ++n, stage.next(), at.next(N, sp.block)) {
+        if (at.u != cur_u) {
+            flush();
+            cur_u = at.u;
+            rs = rs_next;
+            if (cur_u + 1 < units) rs_next = inv_s[cur_u + 1];
+        }
+        copies_wait<kAhead - 1>();
+        const float inv_i = rows[(n % kAhead) * 2 * kTile + r], re = rows[((n % kAhead) * 2 + 1) * kTile + r];
+        fetch(n + kAhead);
+        const int i = at.i0 + r;
+        const bool second = i >= at.blk_end;   // the key lies in the block after the tile's first
+        if (!mbar_wait(&s->tfull[stage.at], stage.round, status, 716)) break;
         tc_fence_after();
         float d[16];
-        tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)stage * 32u, d);
+        tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)stage.at * 32u, d);
         tmem_wait_ld(d);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&s->tempty[stage]);
+        if (lane == 0) mbar_arrive(&s->tempty[stage.at]);
         const float ds = d[0] + d[1] + d[2];
-        const float de = cur.second ? d[6] + d[7] + d[8] : d[3] + d[4] + d[5];
-        const float scaled = cur.inv_i * (1.f / kAnchorScale<T>);
+        const float de = second ? d[6] + d[7] + d[8] : d[3] + d[4] + d[5];
+        const float scaled = inv_i * (1.f / kAnchorScale<T>);
         const float a_s = -(ds * scaled) * rs + 0.f;
-        const float a_e = -(de * scaled) * cur.re + 0.f;
-        if (cur.i < N) {
-            a_raw[((int64_t)cur.u * 3 + 0) * sp.raw_row + cur.i] = a_s;
-            a_raw[((int64_t)cur.u * 3 + 1) * sp.raw_row + cur.i] = a_e;
+        const float a_e = -(de * scaled) * re + 0.f;
+        if (i < N) {
+            float* out = a_raw + (int64_t)cur_u * 3 * sp.raw_row + i;
+            out[0] = a_s;
+            out[sp.raw_row] = a_e;
             lo_s = fminf(lo_s, a_s);
             hi_s = fmaxf(hi_s, a_s);
             lo_e = fminf(lo_e, a_e);
             hi_e = fmaxf(hi_e, a_e);
         }
     }
+    copies_wait<0>();
     flush();
 }
 
@@ -270,25 +363,30 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
     using C = Cfg<D>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* tiles = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-    unsigned char* rhs = tiles + (size_t)C::kSlots * C::kTileBytes;
-    Smem* s = reinterpret_cast<Smem*>(rhs + (size_t)C::kSlots * C::kRhsBytes);
+    unsigned char* rhs = tiles + C::kRhsAt;
+    float* rows = reinterpret_cast<float*>(tiles + C::kRowsAt);
+    float* mu = reinterpret_cast<float*>(tiles + C::kMuAt);
+    Smem* s = reinterpret_cast<Smem*>(tiles + C::kSmemAt);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const TileRange tr = my_tiles(units, N);
 
     if (tid == 0) {
         for (int i = 0; i < C::kSlots; ++i) {
             mbar_init(&s->full[i], 1);
-            mbar_init(&s->rready[i], C::kPrepWarps);
             mbar_init(&s->kfree[i], 1);
+        }
+        for (int i = 0; i < kRhs; ++i) {
+            mbar_init(&s->rready[i], C::kPrepWarps);
+            mbar_init(&s->rfree[i], kMmaWarps);
         }
         for (int i = 0; i < kStages; ++i) {
             mbar_init(&s->tfull[i], 1);
             mbar_init(&s->tempty[i], 4);
         }
-        mbar_init(&s->drain, 1);
+        for (int i = 0; i < kMmaWarps; ++i) mbar_init(&s->drain[i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i < C::kSlots * C::kRhsBytes / 16; i += kThreads) reinterpret_cast<uint4*>(rhs)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < kRhs * C::kRhsBytes / 16; i += kThreads) reinterpret_cast<uint4*>(rhs)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (warp == kMmaWarp) tmem_alloc(&s->tmem_base, kTmemCols);
     tc_fence_before();
@@ -298,15 +396,15 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
     pdl_wait();
 
     if (warp == kProducerWarp) {
-        if (lane == 0) dots_producer<D>(&tmap, tiles, s, tr, H, status);
+        if (lane == 0) dots_producer<D>(&tmap, tiles, s, tr, H, N, status);
         __syncwarp();
-    } else if (warp == kMmaWarp) {
-        if (lane == 0) dots_mma<T, D>(tiles, rhs, s, tmem_base, tr, status);
+    } else if (warp >= kMmaWarp) {
+        if (lane == 0) dots_mma<T, D>(warp - kMmaWarp, tiles, rhs, s, tmem_base, tr, N, sp.block, status);
         __syncwarp();
     } else if (warp >= kEpiWarp0) {
-        dots_epilogue<T>(s, tmem_base, sp, tr, N, inv_norm, inv_s, inv_e, a_raw, mm, status);
+        dots_epilogue<T>(s, rows, tmem_base, sp, tr, units, N, inv_norm, inv_s, inv_e, a_raw, mm, status);
     } else {
-        dots_prep<T, D>(rhs, s, sp, tr, mu_s, mu_e, status);
+        dots_prep<T, D>(rhs, mu, s, sp, tr, units, N, mu_s, mu_e, status);
     }
 
     tc_fence_before();
