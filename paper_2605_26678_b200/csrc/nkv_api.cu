@@ -185,8 +185,8 @@ Bufs bufs_at(void* ws, const Layout& L) {
 // passes in the FMA form / the second / none, H = 8, r = 0.75, bf16, us:
 //     d = 64    17 MB of keys 52 / 54 / 56   33 MB 69 / 70 / 69   67 MB 106 / 100 / 99 (64 x 8192), 99 / 102 / 102 (128 x 4096)
 //     d = 128   17 MB 53 / 54 / 54           33 MB 66 / 62 / 62   67 MB 98 / 84 / 84
-// With keys that are not in L2, 33 MB of 16 x 8 x 2048 x 64: 85.5 / - / 85.8, and 84.9 with only the first in tensor form.
-constexpr int kFirstPassKb = 192, kSecondPassKb64 = 256, kSecondPassKb128 = 192;   // of keys per SM
+// With keys that are not in L2, 41 MB of 16 x 8 x 2500 x 64 at r = 0.5: 84.7 with the second pass in FMA form, 85.5 with none.
+constexpr int kFirstPassKb = 192, kSecondPassKb64 = 320, kSecondPassKb128 = 192;   // of keys per SM
 bool tensor_pays(const nkv_handle* h, const TensorView& kv, int G, const ScoreParams& sp, int kb) {
     const int64_t bytes = (int64_t)G * kv.H * kv.N * kv.d * 2;
     return h->key_pass == NKV_KEY_PASS_TENSOR || !stream_path_supported(sp) || bytes >= (int64_t)h->sm_count * kb * 1024;
