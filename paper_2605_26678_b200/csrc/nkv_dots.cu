@@ -8,17 +8,17 @@
 // side is
 //     columns 0..2  mu_s        3..5  mu_e of the block the tile starts in        6..8  mu_e of the next block
 // (a tile of 128 keys touches at most two blocks because a block has at least 128 keys).  Key tiles are staged by TMA
-// (128-byte swizzle); the tensor core reads them from shared memory directly.  Warp roles: TMA producer, two MMA
-// issuers, four warps that build the right-hand sides, four warps that turn the accumulator into scores.  Every wait is
-// bounded.
+// (128-byte swizzle); the tensor core reads them from shared memory directly.  Warp roles: TMA producer, MMA issuer, four
+// warps that build the right-hand sides, four warps that turn the accumulator into scores.  Every wait is bounded.
 //
 // Bound: the read of the keys; no role may then need more than the 1300 cycles in which a tile of 32 KB arrives.  What
-// that took: places in the tensors are counted, not divided out (tile), right-hand sides are built per block and not per
-// tile, the rows' norms and the anchors come by asynchronous copies several tiles ahead, and two threads issue the
-// products in turn (one needs 1050 cycles per tile of 128 columns, 790 per tile of 64).  128 KB of keys in flight per SM:
-// a bare read of 604 MB in 32 KB pieces takes 101 us with 96 KB in flight per SM, 107 with 160 or 192.
-// 16 x 8 heads of 32768 x 64 bf16 keys: 141 -> 98 us (and 141 in the FMA form of nkv_stream.cu); 36 x 8 x 8192 x 128:
-// 109 -> 106; 36 x 8 x 131072 x 128: 1910 -> 1475 (6.7 TB/s).
+// that took: places in the tensors are counted, not divided out (per tile), right-hand sides are built per block and not
+// per tile, the rows' norms and the anchors come by asynchronous copies several tiles ahead, and the products are issued
+// by a warp in step (umma_f16; one thread by itself needed 1050 cycles per tile of 128 columns, 790 per tile of 64).
+// 96 KB of keys in flight per SM: a bare read of 604 MB in 32 KB pieces takes 101 us with 96, 107 with 160 or 192, and this
+// pass 105, 107 and 112 us with 96, 128 and 160 KB; 64 KB is too little (119).
+// 16 x 8 heads of 32768 x 64 bf16 keys: 141 -> 95 us (and 141 in the FMA form of nkv_stream.cu); 36 x 8 x 8192 x 128:
+// 109 -> 105; 36 x 8 x 131072 x 128: 1900 -> 1470 (6.7 TB/s).
 #include "nkv_sm100.cuh"
 
 namespace nkv {
@@ -33,8 +33,7 @@ constexpr int kRhsHalfBytes = 16 * 128;           // 16 right-hand-side rows of 
 constexpr int kStages = 4;                        // accumulators of 32 columns (16 used)
 constexpr uint32_t kTmemCols = 128;
 constexpr int kPrepWarp0 = 0, kEpiWarp0 = 4, kProducerWarp = 8, kMmaWarp = 9;
-constexpr int kMmaWarps = 2;                      // they take the tiles in turn
-constexpr int kThreads = (9 + kMmaWarps) * 32;
+constexpr int kThreads = 10 * 32;
 constexpr int kMaxSlots = 8;
 constexpr int kRhs = 4;                           // right-hand sides kept at once
 constexpr int kAhead = 8;                         // tiles (blocks) whose per-row inputs (anchors) are on their way
@@ -43,7 +42,7 @@ constexpr int kAhead = 8;                         // tiles (blocks) whose per-ro
 template <int D>
 struct Cfg {
     static constexpr int kHalves = D / 64;
-    static constexpr int kSlots = 512 / D;                       // key tiles staged at once (128 KB)
+    static constexpr int kSlots = 384 / D;                       // key tiles staged at once (96 KB)
     static constexpr int kTileBytes = kHalves * kTileHalfBytes;
     static constexpr int kRhsBytes = kHalves * kRhsHalfBytes;
     static constexpr int kPrepWarps = D / 32;                    // one thread per column
@@ -52,8 +51,6 @@ struct Cfg {
     static constexpr size_t kMuAt = kRowsAt + (size_t)kAhead * 2 * kTile * 4; // [kAhead][D] floats
     static constexpr size_t kSmemAt = kMuAt + (size_t)kAhead * D * 4;
     static_assert(kSlots <= kMaxSlots, "barrier arrays too small");
-    // an issuer has then itself waited for the round before the one that it waits for, so parities are unambiguous
-    static_assert(kSlots % kMmaWarps == 0 && kStages % kMmaWarps == 0, "a slot or stage belongs to one issuer");
 };
 
 struct Smem {
@@ -63,7 +60,7 @@ struct Smem {
     uint64_t rfree[kRhs];       // consumed by the MMAs of all its tiles
     uint64_t tfull[kStages];    // accumulator written
     uint64_t tempty[kStages];   // accumulator read (one arrival per reading warp)
-    uint64_t drain[kMmaWarps];  // products issued before a give-up have completed
+    uint64_t drain;             // products issued before a give-up have completed
     uint32_t tmem_base;
 };
 template <int D>
@@ -164,7 +161,7 @@ __device__ void dots_producer(const CUtensorMap* tmap, unsigned char* tiles, Sme
 }
 
 template <typename T, int D>
-__device__ void dots_mma(int which, unsigned char* tiles, unsigned char* rhs, Smem* s, uint32_t tmem_base, TileRange tr, int N, int block,
+__device__ void dots_mma(unsigned char* tiles, unsigned char* rhs, Smem* s, uint32_t tmem_base, TileRange tr, int N, int block,
                          int* status) {
     using C = Cfg<D>;
     constexpr uint32_t idesc = umma_idesc<T>(kTile, 16);
@@ -173,35 +170,22 @@ __device__ void dots_mma(int which, unsigned char* tiles, unsigned char* rhs, Sm
     Ring<kStages> stage;
     Ring<kRhs> r;
     Place at(tr, block);
-    bool fresh = true, used = false;   // another right-hand side; products of this thread have read it
+    bool fresh = true;   // another right-hand side
     for (int n = 0; n < tr.count; ++n, slot.next(), stage.next()) {
-        const bool mine = n % kMmaWarps == which;
-        // (a thread without a tile of the block waits too: its arrival below must not count for an earlier round)
-        if ((fresh && !mbar_wait(&s->rready[r.at], r.round, status, 713)) ||
-            (mine && (!mbar_wait(&s->tempty[stage.at], stage.round ^ 1u, status, 714) ||
-                      !mbar_wait(&s->full[slot.at], slot.round, status, 712)))) {
-            // products already issued keep reading shared memory and writing tensor memory: wait (bounded)
-            // for them before the CTA frees both
-            umma_commit(&s->drain[which]);
-            for (uint32_t spin = 0; spin < (1u << 16) && !mbar_try_wait(&s->drain[which], 0); ++spin) __nanosleep(256);
-            return;
-        }
-        if (mine) {
-            tc_fence_after();
-            const uint64_t a = tiles_desc + (uint32_t)(slot.at * C::kTileBytes >> 4), b = rhs_desc + (uint32_t)(r.at * C::kRhsBytes >> 4);
+        if ((fresh && !warp_wait(&s->rready[r.at], r.round, status, 713)) ||
+            !warp_wait(&s->tempty[stage.at], stage.round ^ 1u, status, 714) || !warp_wait(&s->full[slot.at], slot.round, status, 712))
+            return umma_drain(&s->drain);
+        tc_fence_after();
+        const uint64_t a = tiles_desc + (uint32_t)(slot.at * C::kTileBytes >> 4), b = rhs_desc + (uint32_t)(r.at * C::kRhsBytes >> 4);
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)
-                umma_f16(tmem_base + (uint32_t)stage.at * 32u, a + (uint32_t)((kk >> 2) * kTileHalfBytes + (kk & 3) * 32 >> 4),
-                         b + (uint32_t)((kk >> 2) * kRhsHalfBytes + (kk & 3) * 32 >> 4), idesc, kk > 0);
-            umma_commit(&s->tfull[stage.at]);
-            umma_commit(&s->kfree[slot.at]);
-            used = true;
-        }
+        for (int kk = 0; kk < D / 16; ++kk)
+            umma_f16(tmem_base + (uint32_t)stage.at * 32u, a + (uint32_t)((kk >> 2) * kTileHalfBytes + (kk & 3) * 32 >> 4),
+                     b + (uint32_t)((kk >> 2) * kRhsHalfBytes + (kk & 3) * 32 >> 4), idesc, kk > 0);
+        umma_commit(&s->tfull[stage.at]);
+        umma_commit(&s->kfree[slot.at]);
         fresh = at.next(N, block);
         if (fresh && n + 1 < tr.count) {
-            if (used) umma_commit(&s->rfree[r.at]);
-            else mbar_arrive(&s->rfree[r.at]);
-            used = false;
+            umma_commit(&s->rfree[r.at]);
             r.next();
         }
     }
@@ -377,13 +361,13 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
         }
         for (int i = 0; i < kRhs; ++i) {
             mbar_init(&s->rready[i], C::kPrepWarps);
-            mbar_init(&s->rfree[i], kMmaWarps);
+            mbar_init(&s->rfree[i], 1);
         }
         for (int i = 0; i < kStages; ++i) {
             mbar_init(&s->tfull[i], 1);
             mbar_init(&s->tempty[i], 4);
         }
-        for (int i = 0; i < kMmaWarps; ++i) mbar_init(&s->drain[i], 1);
+        mbar_init(&s->drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < kRhs * C::kRhsBytes / 16; i += kThreads) reinterpret_cast<uint4*>(rhs)[i] = make_uint4(0, 0, 0, 0);
@@ -398,8 +382,8 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
     if (warp == kProducerWarp) {
         if (lane == 0) dots_producer<D>(&tmap, tiles, s, tr, H, N, status);
         __syncwarp();
-    } else if (warp >= kMmaWarp) {
-        if (lane == 0) dots_mma<T, D>(warp - kMmaWarp, tiles, rhs, s, tmem_base, tr, N, sp.block, status);
+    } else if (warp == kMmaWarp) {
+        dots_mma<T, D>(tiles, rhs, s, tmem_base, tr, N, sp.block, status);
         __syncwarp();
     } else if (warp >= kEpiWarp0) {
         dots_epilogue<T>(s, rows, tmem_base, sp, tr, units, N, inv_norm, inv_s, inv_e, a_raw, mm, status);

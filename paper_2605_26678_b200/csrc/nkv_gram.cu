@@ -32,7 +32,7 @@
 //
 // The CTA is a pipeline of warp groups:
 //     producer (1 thread)    TMA loads of the stages
-//     mma      (1 thread)    the Gram rectangle of the tile
+//     mma      (1 warp)      the Gram rectangle of the tile
 //     band     (2 x 4 warps) the two groups take alternate tiles: norms from the diagonal, then row and column
 //                            sums of the band and the row's part of the next exact restart value
 //     sums     (8 warps)     block sums of normalised keys, kept in registers over the block
@@ -148,11 +148,6 @@ __device__ __forceinline__ float quotient_by_root(float a, float T) {
     return fmaf(y, fmaf(-q0, r, a), q0);
 }
 
-// A whole warp waits; false for all of its lanes when any of them gave up.
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* status, int where) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, where));
-}
-
 // Transposed reduction of V per-lane partial values over a group of L lanes (L, V powers of two, V <= L):
 // afterwards lane l holds in v[0] the complete sum of value l / (L/V).
 template <int V, int L>
@@ -220,16 +215,7 @@ __device__ void producer_role(const CUtensorMap* tmap, unsigned char* ring, Smem
     }
 }
 
-// Products already issued keep reading shared memory and writing tensor memory: a role that gives up
-// waits (bounded) for them before the CTA frees both.
-template <int D>
-__device__ __forceinline__ void drain_products(Smem<D>* s) {
-    umma_commit(&s->drain);
-#pragma unroll 1
-    for (uint32_t spin = 0; spin < (1u << 16) && !mbar_try_wait(&s->drain, 0); ++spin) __nanosleep(256);
-}
-
-// MMA issuer (one thread).  A = the tile's 128 rows, B = those rows and the 64 in front of them.
+// MMA issuer (one warp).  A = the tile's 128 rows, B = those rows and the 64 in front of them.
 template <typename T, int D>
 __device__ void mma_role(unsigned char* ring, Smem<D>* s, uint32_t tmem_base, Walk walk, int block, int N, int* status) {
     using C = Cfg<D>;
@@ -242,8 +228,8 @@ __device__ void mma_role(unsigned char* ring, Smem<D>* s, uint32_t tmem_base, Wa
 #pragma unroll 1
         for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
             const int st = (int)(n % C::kStages), acc = (int)(n & 1);
-            if (!mbar_wait(&s->full[st], (n / C::kStages) & 1u, status, 702)) return drain_products(s);
-            if (!mbar_wait(&s->tempty[acc], ((n >> 1) & 1u) ^ 1u, status, 703)) return drain_products(s);
+            if (!warp_wait(&s->full[st], (n / C::kStages) & 1u, status, 702)) return umma_drain(&s->drain);
+            if (!warp_wait(&s->tempty[acc], ((n >> 1) & 1u) ^ 1u, status, 703)) return umma_drain(&s->drain);
             tc_fence_after();
             // the address field of a descriptor counts 16-byte units: a K step moves it by a constant
             const uint64_t bdesc = umma_desc_sw128(ring_addr + (uint32_t)st * kStageHalfBytes);
@@ -531,8 +517,10 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x, a.y += b.y, a.z += b.z, a.w += b.w; }
 
+// (Out of line: five roles share the instruction caches, and with this one inlined the pass took 158 instead of 154 us at
+// 36 x 8 heads of 8192 x 128 keys.)
 template <int D, bool kGiven>
-__device__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __restrict__ inv_norm, int64_t inv_row,
+__device__ __noinline__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __restrict__ inv_norm, int64_t inv_row,
                           float* __restrict__ a_raw, int64_t raw_row, uint32_t* __restrict__ mm, int* status) {
     const int which = (threadIdx.x >> 5) - kScanWarp0, l = threadIdx.x & 31;
     const int r = 4 * l, q = l >> 3, c = r - 32 * q;
@@ -663,7 +651,7 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
         if (lane == 0) producer_role<D>(&tmap, ring, s, walk, block, N, H, keep_in_l2, status);
         __syncwarp();
     } else if (warp == kMmaWarp) {
-        if (lane == 0) mma_role<T, D>(ring, s, tmem_base, walk, block, N, status);
+        mma_role<T, D>(ring, s, tmem_base, walk, block, N, status);
         __syncwarp();
     } else if (warp >= kScanWarp0) {
         scan_role<D, kGiven>(s, walk, block, N, inv_norm, inv_row, a_raw, raw_row, mm, status);

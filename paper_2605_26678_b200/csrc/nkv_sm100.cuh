@@ -53,6 +53,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     return mbar_wait_poll(bar, parity, status, where);
 }
 
+// A whole warp waits; false for all of its lanes when any of them gave up.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* status, int where) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, where));
+}
+
 // Named barrier over `count` threads that also ORs a predicate over them.
 __device__ __forceinline__ bool bar_or(int id, int count, bool pred) {
     uint32_t r;
@@ -196,19 +201,32 @@ template <typename T>
 __host__ __device__ constexpr uint32_t umma_idesc(int M, int N) {
     return (1u << 4) | (kOperandType<T> << 7) | (kOperandType<T> << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread.
+// D[tmem] (+)= A[smem] * B[smem]^T.  Products and commits are issued by a whole warp in step, of which one elected lane
+// (always the same) counts: the operands then stay in uniform registers.  From a thread that has left its warp behind a
+// product took 61 cycles to issue, on an idle SM, and up to 270 beside busy warps; so it takes 6 for a batch of eight, and
+// the tensor core sets the pace (97 cycles for M = 128, N = 192, K = 16; 33 for N = 16).
 __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           bool accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
         : "memory");
 }
-// The barrier gets one arrival once every MMA issued so far by this thread has completed.
+// The barrier gets one arrival once every MMA issued so far by this warp has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_addr(bar))
+        : "memory");
+}
+// Products already issued keep reading shared memory and writing tensor memory: a warp that gives up waits (bounded)
+// for them before the CTA frees both.
+static __device__ __noinline__ void umma_drain(uint64_t* bar) {
+    __syncwarp();
+    umma_commit(bar);
+    for (uint32_t spin = 0; spin < (1u << 16) && !mbar_try_wait(bar, 0); ++spin) __nanosleep(256);
+    __syncwarp();
 }
 
 // ---------------------------------------------------------------------------- packed fp32 pairs
