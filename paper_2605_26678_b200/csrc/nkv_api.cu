@@ -235,7 +235,7 @@ int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreP
 
 // Staging of nkv_compress_host: the groups of a chunk are halved where possible, so that twice as many slots keep the
 // copy engines busy in both directions while kernels run.
-constexpr int kHostGatherCtas = 16;
+constexpr int kHostGatherCtas = 32;
 constexpr double kHostRowsShare = 0.6;
 struct HostSlot {
     size_t K, V, K_out, V_out, idx, offsets, budgets, ws, total;
@@ -529,7 +529,7 @@ int nkv_compact(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, const i
     if (mode == NKV_OUT_OF_PLACE) {
         if (!K_out || !V_out || ((uintptr_t)K_out) % 16 || ((uintptr_t)V_out) % 16) return NKV_ERR_INVALID_ARG;
         CU(launch_gather(view_of(K), kb, view_of(V), vb, (int)K->G, idx, head_offsets, idx_capacity, K_out, V_out,
-                         h->sm_count, 0, st, &h->launches));
+                         0, st, &h->launches));
     } else if (mode == NKV_IN_PLACE) {
         if (K_out || V_out) return NKV_ERR_INVALID_ARG;
         CU(launch_gather_in_place(view_of(K), kb, view_of(V), vb, (int)K->G, idx, head_offsets, idx_capacity, st,
@@ -584,11 +584,11 @@ static int compress(nkv_handle* h, const nkv_tensor* K, const nkv_tensor* V, dou
     CU(mark());
     CU(mark());   // the budget and select stages are part of that call
     CU(mark());
-    CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, K_out, host_v ? nullptr : V_out, h->sm_count, 0, st,
+    CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, K_out, host_v ? nullptr : V_out, 0, st,
                      &h->launches));
     // a few CTAs keep more reads on the bus than it takes to fill it, and leave the SMs to the kernels of other chunks
     if (host_v)
-        CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, nullptr, V_out, h->sm_count, kHostGatherCtas, st,
+        CU(launch_gather(kv, kb, vv, vb, G, idx, head_offsets, (int64_t)H * keep, nullptr, V_out, kHostGatherCtas, st,
                          &h->launches));
     CU(mark());
     if (timing) h->timing_valid = 1;

@@ -198,7 +198,7 @@ cudaError_t launch_ranks(int units, int N, const float* a_star, int32_t* ranks, 
                          int64_t* launches);
 cudaError_t launch_gather(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,
                           const int32_t* idx, const int32_t* head_offsets, int64_t idx_capacity, void* K_out,
-                          void* V_out, int sm_count, int ctas_or_0, cudaStream_t stream, int64_t* launches);
+                          void* V_out, int ctas_or_0, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_gather_in_place(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,
                                    const int32_t* idx, const int32_t* head_offsets, int64_t idx_capacity,
                                    cudaStream_t stream, int64_t* launches);

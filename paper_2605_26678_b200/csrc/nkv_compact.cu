@@ -10,7 +10,8 @@ namespace nkv {
 namespace {
 
 constexpr int kRowsPerBatch = 32;   // in-place kernel
-constexpr int kGatherRows = 128;    // out-of-place kernel: rows per batch (64: 8 % slower at 9.7 GB of rows)
+constexpr int kGatherThreads = 128; // out-of-place kernel
+constexpr int kGatherRows = 64;     // rows per batch
 constexpr int kGatherInFlight = 8;  // 16-byte loads each thread issues before its first store
 
 struct GatherArgs {
@@ -23,7 +24,11 @@ struct GatherArgs {
     int64_t total_rows;  // G * cap
 };
 
-__global__ void __launch_bounds__(256) gather_kernel(GatherArgs A, const int32_t* __restrict__ idx,
+// Bound: DRAM, half of it reads and half writes.  Every CTA moves one batch, a thread's share of which is one or two rounds
+// of kGatherInFlight loads: the block scheduler then evens out what the SMs get.  144 x 8 heads, a quarter of 32768 x 128
+// bf16 rows of K and V each (9.7 GB of traffic): 1630 us with 8 CTAs of 256 threads per SM that stride over the batches,
+// 1540 with a CTA of 256 threads for every batch of 128 rows, 1495 (6.5 TB/s) like this; 36 x 8 x 16384 fp16: 422, 377, 377.
+__global__ void __launch_bounds__(kGatherThreads) gather_kernel(GatherArgs A, const int32_t* __restrict__ idx,
                                                      const int32_t* __restrict__ head_offsets) {
     __shared__ int64_t src_off[2][kGatherRows];
     pdl_wait();
@@ -56,12 +61,12 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherArgs A, const int32_t
         __syncthreads();
         // the chunks of the batch's K rows, then of its V rows, form one list; every thread keeps
         // kGatherInFlight loads in flight before it stores
-        for (int c0 = threadIdx.x; c0 < total; c0 += 256 * kGatherInFlight) {
+        for (int c0 = threadIdx.x; c0 < total; c0 += kGatherThreads * kGatherInFlight) {
             uint4 q[kGatherInFlight];
             uint4* dst[kGatherInFlight];
 #pragma unroll
             for (int e = 0; e < kGatherInFlight; ++e) {
-                const int c = c0 + e * 256;
+                const int c = c0 + e * kGatherThreads;
                 dst[e] = nullptr;
                 if (c < total) {
                     const int t = c >= total0 ? 1 : 0;
@@ -153,14 +158,14 @@ GatherArgs make_args(const TensorView& K, int kb, const TensorView& V, int vb, i
 
 cudaError_t launch_gather(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,
                           const int32_t* idx, const int32_t* head_offsets, int64_t idx_capacity, void* K_out,
-                          void* V_out, int sm_count, int ctas_or_0, cudaStream_t stream, int64_t* launches) {
+                          void* V_out, int ctas_or_0, cudaStream_t stream, int64_t* launches) {
     GatherArgs A = make_args(K, k_elem_bytes, V, v_elem_bytes, G, idx_capacity, K_out, V_out);
     const int64_t nbatch = (A.total_rows + kGatherRows - 1) / kGatherRows;
     if (nbatch == 0) return cudaSuccess;
-    int64_t grid = ctas_or_0 ? ctas_or_0 : (int64_t)sm_count * 8;
-    if (grid > nbatch) grid = nbatch;
+    int64_t grid = ctas_or_0 && ctas_or_0 < nbatch ? ctas_or_0 : nbatch;
+    if (grid > 0x7fffffff) grid = 0x7fffffff;
     ++*launches;
-    return launch_chained(gather_kernel, (unsigned)grid, 256, 0, stream, 1, A, idx, head_offsets);
+    return launch_chained(gather_kernel, (unsigned)grid, kGatherThreads, 0, stream, 1, A, idx, head_offsets);
 }
 
 cudaError_t launch_gather_in_place(const TensorView& K, int k_elem_bytes, const TensorView& V, int v_elem_bytes, int G,
