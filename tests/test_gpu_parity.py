@@ -556,6 +556,27 @@ def test_safeguard_that_no_head_and_some_head_needs(layers, H, N, safeguard):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("repeat", [False, True])
+@pytest.mark.parametrize("layers,H,N", [(1, 8, 16384), (1, 3, 33333), (4, 8, 16701), (8, 8, 25100), (1, 1, 14400)])
+def test_score_phase_with_a_head_shared_by_several_ctas(layers, H, N, repeat):
+    """Two, four and eight CTAs per head; keys that repeat crowd the bins of the tails."""
+    K, V = _cache(N, 64, "bf16", H=H, layers=layers)
+    if repeat:
+        K = K[:, :, torch.arange(N, device=DEV) % 7].contiguous()
+    p = nkv.nkv_default_params()
+    ws = nkv.alloc_workspace(K, p)
+    res = nkv.nkv_compress(K, V, 0.75, p, ws=ws, want_a_star=True)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    for g in {0, layers - 1}:
+        if not repeat:   # equal keys: the tails' members are a matter of rounding
+            ref = oracle.compress_group(K[g].cpu(), V[g].cpu(), 0.75, pr.oracle_params(p))
+            pr.assert_close(res.a_star[g].cpu().numpy(), ref.a_star, "a_star")
+        own = oracle.budget_select(res.a_star[g].cpu().numpy(), 0.75, pr.oracle_params(p))
+        assert np.array_equal(own.budgets, res.budgets[g].cpu().numpy())
+        assert np.array_equal(own.idx, res.idx[g].cpu().numpy())
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("layers,chunk,r,pinned", [(5, 1, 0.75, True), (7, 3, 0.75, True), (4, 4, 0.25, True), (3, 2, 0.75, False)])
 def test_host_entry_point_with_rows_fetched_in_place_and_copied(layers, chunk, r, pinned):
     """Retained rows of V read from pinned memory, and V copied whole (most rows retained, or memory that the device
