@@ -42,8 +42,8 @@ DEFAULT_RATIO = 0.75
 # reports no traffic.
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_bytes_per_key.txt")
 STAGE_KERNEL = {"anchors": ("gram_pass_kernel", "nkv_gram.cu"), "score": ("anchor_dots_kernel", "nkv_dots.cu"),
-                "compact": ("gather_kernel", "nkv_compact.cu"), "head": ("scale_stats_kernel", "nkv_select.cu"),
-                "budget": ("budget_kernel", "nkv_select.cu"), "select": ("select_kernel", "nkv_select.cu")}
+                "compact": ("gather_kernel", "nkv_compact.cu"), "head": ("group_kernel", "nkv_select.cu"),
+                "budget": ("group_kernel", "nkv_select.cu"), "select": ("group_kernel", "nkv_select.cu")}
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 

@@ -27,8 +27,8 @@
 // the tile that restarts every tile from an exact value (the sum of the 64 x 64 Gram block that ends at
 // the previous tile's last row, which is in that tile's D).  f is read with a lag of 64 rows, when every row of its
 // column has been seen.  Only the block sums of normalised keys need the key values themselves and stay on the FMA
-// pipes.  (As a second product, K[tile]^T x (1/||k|| split three ways into bf16), a K step took 280 cycles with the
-// tile as the transposed A operand and 290 (d = 64) to 400 (d = 128) with it as the MN-major B operand.)
+// pipes.  (As a second product, K[tile]^T x (1/||k|| split three ways into bf16), it was slower: 280 cycles per K step
+// with the tile as the transposed A operand, 290 to 400 with it as the MN-major B operand, all issued by one thread.)
 //
 // The CTA is a pipeline of warp groups:
 //     producer (1 thread)    TMA loads of the stages
