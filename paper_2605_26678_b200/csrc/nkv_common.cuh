@@ -38,19 +38,15 @@ struct ScoreParams {
 // Per-head minimum and maximum of each scale, [3][2] keys that start at 0 and grow by atomicMax: the complement of the
 // minimum's ordered key, the maximum's ordered key.
 
-// Order-preserving map float -> uint32 (larger float <=> larger key) and back.
-__host__ __device__ __forceinline__ uint32_t ord_key(float f) {
-#ifdef __CUDA_ARCH__
-    uint32_t b = __float_as_uint(f);
-#else
-    uint32_t b;
-    memcpy(&b, &f, 4);
-#endif
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+// Order-preserving map float -> uint32 (larger float <=> larger key; NaN above +inf, or below -inf with its sign set) and
+// back.  In this form it stays integer arithmetic: `bits | 0x80000000` was turned into a floating-point negation, which
+// makes 0x7fffffff of every NaN.
+__device__ __forceinline__ uint32_t ord_key(float f) {
+    const uint32_t b = __float_as_uint(f);
+    return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
 }
 __device__ __forceinline__ float ord_float(uint32_t k) {
-    uint32_t b = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
-    return __uint_as_float(b);
+    return __uint_as_float(k ^ (~(uint32_t)((int32_t)k >> 31) | 0x80000000u));
 }
 
 // 16-byte chunk -> fp32 values.  bf16 and fp16: 8 values, fp32: 4 values.

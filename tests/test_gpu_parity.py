@@ -593,3 +593,65 @@ def test_host_entry_point_with_rows_fetched_in_place_and_copied(layers, chunk, r
     for a, b in ((out.k_out, dev.k_out), (out.v_out, dev.v_out), (out.idx, dev.idx), (out.head_offsets, dev.head_offsets),
                  (out.budgets, dev.budgets)):
         assert torch.equal(a, b.cpu())
+
+
+def _keys(s):
+    """Ordered keys of fp32 scores: larger score, larger key; NaN by its bits, above +inf or (sign set) below -inf."""
+    b = np.ascontiguousarray(s, np.float32).view(np.uint32)
+    return np.where(b & 0x80000000, ~b, b | 0x80000000).astype(np.int64)
+
+
+def _select_by_key(s, r, n_safe):
+    """Budgets and positions of one group [H, N] in the order (key descending, head, position), safeguard first."""
+    H, N = s.shape
+    keep = H * nkv.nkv_keep_per_head(N, r)
+    key = _keys(s)
+    taken = np.zeros((H, N), bool)
+    for h in range(H):
+        taken[h, np.lexsort((np.arange(N), -key[h]))[:n_safe]] = True
+    head, pos = np.divmod(np.arange(H * N), N)
+    order = np.lexsort((pos, head, -key.ravel()))
+    order = order[~taken.ravel()[order]]
+    taken.ravel()[order[:keep - H * n_safe]] = True
+    return taken.sum(1), np.concatenate([np.flatnonzero(t) for t in taken])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,H,N,r,share", [(2, 3, 700, 0.5, 0.01), (1, 8, 5000, 0.75, 0.1), (1, 2, 6000, 0.9, 0.5),
+                                           (1, 4, 30000, 0.5, 0.4), (3, 1, 9000, 0.5, 1.0)])
+def test_scores_that_are_not_finite_are_ordered_by_their_bits(G, H, N, r, share):
+    """NaN of either sign, infinities and signed zeros among a caller's scores: every budgeted position is written."""
+    rng = np.random.default_rng(N)
+    s = _random_scores(G, H, N, seed=N, ties="none")
+    odd = np.array([0x7fc00000, 0x7fffffff, 0xffc00000, 0xffffffff, 0x7f800000, 0xff800000, 0x80000000, 0, 0x7f7fffff], np.uint32)
+    mask = rng.random(s.shape) < share
+    s[mask] = rng.choice(odd, mask.sum()).view(np.float32)
+    a_star = torch.from_numpy(s).to(DEV)
+    ws = torch.zeros(1 << 16, dtype=torch.uint8, device=DEV)
+    budgets = nkv.nkv_budget(a_star, r, ws=ws)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    idx, offs, _ = nkv.nkv_select(a_star, budgets, H * nkv.nkv_keep_per_head(N, r), ws=ws)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    for g in range(G):
+        want_b, want_idx = _select_by_key(s[g], r, nkv.nkv_safeguard_count(N, r))
+        assert np.array_equal(budgets[g].cpu().numpy(), want_b)
+        assert np.array_equal(idx[g].cpu().numpy(), want_idx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,layers,d,r", [(700, 1, 64, 0.5), (5000, 3, 128, 0.75), (12000, 2, 64, 0.5), (30000, 1, 128, 0.75),
+                                          (8192, 19, 128, 0.5)])
+def test_a_key_that_is_not_finite_leaves_no_position_unwritten(N, layers, d, r):
+    """One infinite key makes the scores of its head NaN: the positions are those of the scores' order all the same."""
+    K, V = _cache(N, d, "bf16", H=4, layers=layers)
+    K[layers - 1, 2, N // 2, 5] = float("inf")
+    ws = nkv.alloc_workspace(K)
+    out = nkv.alloc_outputs(K, V, r, want_a_star=True)
+    out.idx.fill_(-7)
+    res = nkv.nkv_compress(K, V, r, ws=ws, out=out)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    assert bool(torch.isnan(res.a_star[layers - 1, 2, 4:]).all())
+    for g in {0, layers - 1}:
+        want_b, want_idx = _select_by_key(res.a_star[g].cpu().numpy(), r, nkv.nkv_safeguard_count(N, r))
+        assert np.array_equal(res.budgets[g].cpu().numpy(), want_b)
+        assert np.array_equal(res.idx[g].cpu().numpy(), want_idx)
