@@ -394,6 +394,12 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
     const bool owner = (t & 3) == (t >> 3);      // holds diagonal entries: column 8 J + b0 + e, e = (t / 4) % 2
     const int oe = (t >> 2) & 1;
     const uint32_t tq = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(which * 256 + 32 * q);
+    // Columns 0 .. 63 of a span's first tile are products with whatever the ring holds, keys of another head among it.  They
+    // are dropped and not only weighed with 0, which an infinity or a NaN among them would survive.
+    auto drop = [](float(&v)[2][16]) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i >> 4][i & 15] = 0.f;
+    };
     uint32_t n = 0;
     Span sp;
 #pragma unroll 1
@@ -449,6 +455,7 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
             const float* wy = q >= 1 ? &s->w[slot][32 * q - 32] : before + 32;
             const float* wx = q >= 2 ? &s->w[slot][32 * q - 64] : before + 32 * q;
             tmem_wait_ld(y[0], y[1]);
+            if (tau == 0 && q == 0) drop(y);
             tmem_ld_frag32(tq, z[0]);
             tmem_ld_frag32(tq + (16u << 16), z[1]);
             chunk_sums<kChunkY>(y, wy + b0, wrow, p0, p1, row, cy);
@@ -460,6 +467,7 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
             tc_fence_before();
             __syncwarp();
             if (t == 0) mbar_arrive(&s->tempty[which]);
+            if (tau == 0 && q < 2) drop(z);
             chunk_sums<kChunkX>(z, wx + b0, wrow, p0, p1, row, cx);
 
             // row sums over the four lanes of a row; afterwards lane t holds row 8 (t % 4) + t / 4 of the quarter
@@ -634,7 +642,7 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < kHalo) s->zero[tid] = 0.f;
-    // the rows in front of the first tile weigh nothing, but they have to be numbers
+    // (the rows in front of the first tile, which count for nothing)
     for (int half = 0; half < C::kHalves; ++half)
         for (int i = tid; i < kHaloHalfBytes / 16; i += kThreads)
             reinterpret_cast<uint4*>(ring + half * C::kHalfBytes)[i] = make_uint4(0u, 0u, 0u, 0u);

@@ -655,3 +655,25 @@ def test_a_key_that_is_not_finite_leaves_no_position_unwritten(N, layers, d, r):
         want_b, want_idx = _select_by_key(res.a_star[g].cpu().numpy(), r, nkv.nkv_safeguard_count(N, r))
         assert np.array_equal(res.budgets[g].cpu().numpy(), want_b)
         assert np.array_equal(res.idx[g].cpu().numpy(), want_idx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,d,N", [("bf16", 128, 256), ("bf16", 64, 256), ("fp16", 128, 320), ("fp16", 64, 256)])
+def test_a_key_that_is_not_finite_stays_inside_its_head(dtype, d, N):
+    """Three heads and more per SM in the tensor-core passes: what the last key of one of them is does not reach the others."""
+    K, _ = _cache(N, d, dtype, H=8, layers=56)
+    bad = K.clone()
+    worst = torch.finfo(K.dtype).max if dtype == "bf16" else float("inf")   # bf16: finite, but not its products
+    heads = bad.view(-1, N, d)
+    heads[0::15, -1, 3], heads[5::15, -1, 3], heads[10::15, -1] = float("inf"), float("nan"), worst
+    p = nkv.nkv_default_params()
+    ws = nkv.alloc_workspace(K, p)
+    nkv.nkv_set_key_passes("tensor")
+    try:
+        want, got = nkv.nkv_key_scan(K, p, ws=ws), nkv.nkv_key_scan(bad, p, ws=ws)
+    finally:
+        nkv.nkv_set_key_passes("auto")
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    clean = torch.arange(8 * 56) % 5 != 0
+    for a, b in zip(want, got):
+        assert torch.equal(a.flatten(0, 1)[clean], b.flatten(0, 1)[clean])
