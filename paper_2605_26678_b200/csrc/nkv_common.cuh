@@ -18,7 +18,6 @@ constexpr int kSeg = 8;              // rows per window segment (one 8-lane grou
 constexpr int kStatusWords = 64;     // 256 bytes
 constexpr int kStatusCode = 0;       // 0, NKV_ERR_TIMEOUT or NKV_ERR_DEVICE_CHECK
 constexpr int kStatusDetail = 1;     // where it happened
-constexpr int kStatusFallbacks = 2;  // number of selections that took the radix fallback (informational)
 
 // Internal description of a key/value tensor passed to kernels by value.
 struct TensorView {

@@ -677,3 +677,58 @@ def test_a_key_that_is_not_finite_stays_inside_its_head(dtype, d, N):
     clean = torch.arange(8 * 56) % 5 != 0
     for a, b in zip(want, got):
         assert torch.equal(a.flatten(0, 1)[clean], b.flatten(0, 1)[clean])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,H,N,r", [(1, 8, 16384, 0.5), (2, 16, 9001, 0.75), (1, 64, 3000, 0.9), (5, 1, 20000, 0.5), (1, 2, 40003, 0.95)])
+@pytest.mark.parametrize("kind", ["sliver", "near zero", "above one", "two values", "ties and sliver"])
+def test_bins_that_hold_more_scores_than_a_list(G, H, N, r, kind):
+    """Scores that crowd one bin of the competition and of the heads' thresholds, down to one, two and three levels below it."""
+    rng = np.random.default_rng(N + len(kind))
+    s = rng.random((G, H, N)).astype(np.float32)
+    if kind == "sliver":             # one bin of 2048 holds them all
+        s = (np.float32(0.3) + np.float32(1e-5) * s * rng.uniform(0.3, 1.0, (G, H, 1))).astype(np.float32)
+    elif kind == "near zero":        # the lowest bin: every exponent down to the denormals
+        s = np.exp2(-140.0 * s - 12.0).astype(np.float32)
+    elif kind == "above one":        # and the highest
+        s = np.exp2(120.0 * s + 1.0).astype(np.float32)
+    elif kind == "two values":
+        s = np.where(s < 0.5, np.float32(0.25), np.nextafter(np.float32(0.25), np.float32(1.0))).astype(np.float32)
+    else:
+        s = np.where(s < 0.6, np.float32(0.7), np.float32(0.7) + np.float32(1e-6) * rng.integers(-40, 40, s.shape)).astype(np.float32)
+    s[:, :, :4] = np.inf
+    a_star = torch.from_numpy(s).to(DEV)
+    ws = torch.zeros(1 << 20, dtype=torch.uint8, device=DEV)
+    budgets = nkv.nkv_budget(a_star, r, ws=ws)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    idx, _, _ = nkv.nkv_select(a_star, budgets, H * nkv.nkv_keep_per_head(N, r), ws=ws)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    for g in {0, G - 1}:
+        want_b, want_idx = _select_by_key(s[g], r, nkv.nkv_safeguard_count(N, r))
+        assert np.array_equal(budgets[g].cpu().numpy(), want_b)
+        assert np.array_equal(idx[g].cpu().numpy(), want_idx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("layers,H,N", [(1, 8, 777), (36, 8, 2500), (1, 8, 30011), (20, 8, 9000), (1, 3, 16700)])
+def test_keys_whose_anomalies_crowd_a_few_bins(layers, H, N):
+    """A head's bulk within a hundredth of the range that a few outliers span: crowded tails of the three scales (one CTA per
+    head and several) and a crowded competition."""
+    gen = torch.Generator(device=DEV).manual_seed(N)
+    mu = 2.0 * torch.randn((layers, H, 1, 64), generator=gen, device=DEV)
+    x = mu + 0.05 * torch.randn((layers, H, N, 64), generator=gen, device=DEV)
+    # Outliers in every head: the range of an anomaly is then of order 1 and its error of about 1e-7 stays one.  (The bulk by
+    # itself spans (0.05 / 2)^2, about 6e-4, and would turn the same error into 2e-4 of a normalised score.)
+    outlier = torch.rand((layers, H, N, 1), generator=gen, device=DEV) < 0.002
+    outlier[:, :, 10::250] = True
+    K = torch.where(outlier, 3.0 * torch.randn(x.shape, generator=gen, device=DEV), x).to(torch.bfloat16)
+    p = nkv.nkv_default_params()
+    ws = nkv.alloc_workspace(K, p)
+    res = nkv.nkv_compress(K, K, 0.5, p, ws=ws, want_a_star=True)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    for g in {0, layers - 1}:
+        for h in {0, H - 1}:
+            pr.assert_close(res.a_star[g, h].cpu().numpy(), oracle.score_head(K[g, h].cpu()).a_star, "a_star")
+        own = oracle.budget_select(res.a_star[g].cpu().numpy(), 0.5, pr.oracle_params(p))
+        assert np.array_equal(own.budgets, res.budgets[g].cpu().numpy())
+        assert np.array_equal(own.idx, res.idx[g].cpu().numpy())
