@@ -5,7 +5,10 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <cuda.h>
+
 #include "nkv_common.cuh"
+#include "nkv_hostrange.h"
 
 using namespace nkv;
 
@@ -276,17 +279,31 @@ HostPlan host_plan(int64_t H, int64_t N, int64_t d, int dtype, int64_t keep, con
 
 // The address at which the current device reads [p, p + bytes) of host memory in place; null when it cannot.
 const void* device_address(const void* p, size_t bytes) {
-    cudaPointerAttributes first, last;
-    if (cudaPointerGetAttributes(&first, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, static_cast<const unsigned char*>(p) + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer || !last.devicePointer)
-        return nullptr;
-    if (static_cast<unsigned char*>(last.devicePointer) - static_cast<unsigned char*>(first.devicePointer) != (ptrdiff_t)(bytes - 1))
-        return nullptr;
-    return first.devicePointer;
+    return readable_in_place(p, bytes, [](const void* q, HostRange* r) {
+        using GetAttribute = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+        static const GetAttribute attribute = [] {   // looked up once (the library does not link against the driver)
+            void* f = nullptr;
+            cudaDriverEntryPointQueryResult found;
+            if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &f, cudaEnableDefault, &found) != cudaSuccess ||
+                found != cudaDriverEntryPointSuccess)
+                f = nullptr;
+            return reinterpret_cast<GetAttribute>(f);
+        }();
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (!attribute || a.type != cudaMemoryTypeHost || !a.devicePointer) return false;
+        CUdeviceptr start = 0;
+        size_t size = 0;
+        const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(a.devicePointer);
+        if (attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+            attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS)
+            return false;
+        *r = {static_cast<const unsigned char*>(a.devicePointer), static_cast<uintptr_t>(start), size};
+        return true;
+    });
 }
 
 // ordered min/max keys -> floats (lo_s, hi_s, lo_e, hi_e, lo_c, hi_c per head)
