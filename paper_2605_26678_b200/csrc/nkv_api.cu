@@ -24,12 +24,13 @@ struct nkv_handle {
     int key_pass;     // NKV_KEY_PASS_*: which kernels make the two key passes
     cudaEvent_t ev[NKV_NUM_STAGES + 1];
     cudaStream_t copy_streams[kHostSlots];
-    int* chunk_status;   // pinned host copy of every chunk's status words (nkv_compress_host)
+    int* chunk_status;   // pinned: the status code of every step of nkv_compress_host
+    int64_t chunk_capacity;
     int inject_status;   // tests: status code planted in chunk `inject_chunk` of nkv_compress_host
     int inject_chunk;
 };
 
-constexpr int kMaxHostChunks = 4096;
+constexpr int64_t kHostSteps = 4096;   // steps of nkv_compress_host that the first status buffer holds
 
 namespace {
 
@@ -409,10 +410,11 @@ int nkv_create(nkv_handle** out, int device) {
             delete h;
             return NKV_ERR_CUDA;
         }
-    if (cudaMallocHost(reinterpret_cast<void**>(&h->chunk_status), kMaxHostChunks * 4 * sizeof(int)) != cudaSuccess) {
+    if (cudaMallocHost(reinterpret_cast<void**>(&h->chunk_status), kHostSteps * sizeof(int)) != cudaSuccess) {
         delete h;
         return NKV_ERR_CUDA;
     }
+    h->chunk_capacity = kHostSteps;
     for (int i = 0; i < kHostSlots; ++i) {
         if (cudaStreamCreateWithFlags(&h->copy_streams[i], cudaStreamNonBlocking) != cudaSuccess) {
             delete h;
@@ -658,8 +660,17 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
     // copy is the better way; the two meet at about 0.6 of the rows.
     const void* v_mapped = (double)keep <= kHostRowsShare * (double)N ? device_address(Vh->ptr, (size_t)G * grp_in) : nullptr;
 
+    const int64_t steps = (G + p.groups - 1) / p.groups;
+    if (steps > h->chunk_capacity) {
+        int* more = nullptr;
+        CU(cudaMallocHost(reinterpret_cast<void**>(&more), steps * sizeof(int)));
+        cudaFreeHost(h->chunk_status);
+        h->chunk_status = more;
+        h->chunk_capacity = steps;
+    }
+
     int result = NKV_OK;
-    int step = 0;
+    int64_t step = 0;
     for (int64_t g0 = 0; g0 < G && result == NKV_OK; g0 += p.groups, ++step) {
         cudaStream_t st = h->copy_streams[step % p.slots];
         const int64_t gc = (G - g0 < p.groups) ? (G - g0) : p.groups;
@@ -701,19 +712,17 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
             cudaMemcpyAsync(head_offsets_host + g0 * (H + 1), dOff, gc * (H + 1) * 4, cudaMemcpyDeviceToHost, st) !=
                 cudaSuccess ||
             cudaMemcpyAsync(budgets_host + g0 * H, dBud, gc * H * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            (step < kMaxHostChunks &&
-             cudaMemcpyAsync(h->chunk_status + step * 4, dWs, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess)) {
+            cudaMemcpyAsync(h->chunk_status + step, static_cast<int*>(dWs) + kStatusCode, sizeof(int), cudaMemcpyDeviceToHost, st) !=
+                cudaSuccess) {
             result = NKV_ERR_CUDA;
             break;
         }
     }
-    const int chunk_index = step;
     for (int i = 0; i < kHostSlots; ++i)
         if (cudaStreamSynchronize(h->copy_streams[i]) != cudaSuccess) result = result ? result : NKV_ERR_CUDA;
-    // every chunk's device status words were copied out before its slot was reused: report the first failure
-    for (int c2 = 0; c2 < chunk_index && c2 < kMaxHostChunks && result == NKV_OK; ++c2)
-        if (h->chunk_status[c2 * 4 + kStatusCode] != 0)
-            result = h->chunk_status[c2 * 4 + kStatusCode] == NKV_ERR_TIMEOUT ? NKV_ERR_TIMEOUT : NKV_ERR_DEVICE_CHECK;
+    // the status of every step was copied out before its slot was reused: report the first failure
+    for (int64_t i = 0; i < step && result == NKV_OK; ++i)
+        if (h->chunk_status[i] != 0) result = h->chunk_status[i] == NKV_ERR_TIMEOUT ? NKV_ERR_TIMEOUT : NKV_ERR_DEVICE_CHECK;
     return result;
 }
 

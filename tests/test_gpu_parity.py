@@ -732,3 +732,24 @@ def test_keys_whose_anomalies_crowd_a_few_bins(layers, H, N):
         own = oracle.budget_select(res.a_star[g].cpu().numpy(), 0.5, pr.oracle_params(p))
         assert np.array_equal(own.budgets, res.budgets[g].cpu().numpy())
         assert np.array_equal(own.idx, res.idx[g].cpu().numpy())
+
+
+@pytest.mark.gpu
+def test_host_entry_point_reports_a_device_status_behind_thousands_of_chunks():
+    """The status of the last of 4300 one-group steps (chunks of two groups), of the first, and of none."""
+    G, H, N, d, r = 4300, 1, 8, 64, 0.5
+    K = torch.randn((G, H, N, d), generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).pin_memory()
+    k = nkv.nkv_keep_per_head(N, r)
+    out = nkv.Compressed(*[torch.empty(shape, dtype=dt).pin_memory() for shape, dt in (
+        ((G, H * k, d), K.dtype), ((G, H * k, d), K.dtype), ((G, H * k), torch.int32), ((G, H + 1), torch.int32), ((G, H), torch.int32))], None)
+    staging = torch.empty(nkv.nkv_host_staging_bytes(H, N, d, nkv.NKV_BF16, r, 2), dtype=torch.uint8, device=DEV)
+    for chunk in (G // 2 - 1, 0):
+        nkv.nkv_debug_set("inject_host_status", chunk * 16 + nkv.NKV_ERR_TIMEOUT)
+        try:
+            with pytest.raises(nkv.NkvError) as e:
+                nkv.nkv_compress_host(K, K, r, out, staging, 2)
+            assert e.value.status == nkv.NKV_ERR_TIMEOUT
+        finally:
+            nkv.nkv_debug_set("inject_host_status", 0)
+    nkv.nkv_compress_host(K, K, r, out, staging, 2)
+    assert int(out.budgets.sum()) == G * H * k
