@@ -154,8 +154,10 @@ int check_ws(const void* ws, size_t ws_bytes, size_t need) {
 template <typename T>
 T* at(void* ws, size_t off) { return reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(ws) + off); }
 
-// With NKV_TRACE set in the environment a failing CUDA call is named on stderr.
+// With NKV_TRACE set in the environment a failing CUDA call is named on stderr.  The call's error does not stay behind as the
+// runtime's last one: launches that ask for it would take it for theirs.
 int cuda_failed(cudaError_t e, const char* what, int line) {
+    cudaGetLastError();
     static const bool trace = getenv("NKV_TRACE") != nullptr;
     if (trace) fprintf(stderr, "nkv: %s (nkv_api.cu:%d): %s\n", what, line, cudaGetErrorString(e));
     return NKV_ERR_CUDA;
@@ -723,6 +725,7 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
     // the status of every step was copied out before its slot was reused: report the first failure
     for (int64_t i = 0; i < step && result == NKV_OK; ++i)
         if (h->chunk_status[i] != 0) result = h->chunk_status[i] == NKV_ERR_TIMEOUT ? NKV_ERR_TIMEOUT : NKV_ERR_DEVICE_CHECK;
+    if (result == NKV_ERR_CUDA) cudaGetLastError();
     return result;
 }
 

@@ -58,11 +58,16 @@ extern "C" int nkv_budget_static(const float* a_star, int64_t G, int64_t H, int6
     if (rc != NKV_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     // the scratch keeps the previous call's contents: the status words must start at zero
-    if (cudaMemsetAsync(scratch, 0, kStatusBytes, st) != cudaSuccess) return NKV_ERR_CUDA;
+    if (cudaMemsetAsync(scratch, 0, kStatusBytes, st) != cudaSuccess) {
+        cudaGetLastError();   // (not left behind for the next call)
+        return NKV_ERR_CUDA;
+    }
     int64_t launches = 0;
     unsigned char* base = reinterpret_cast<unsigned char*>(scratch);
     if (nkv::launch_budget((int)G, (int)H, (int)N, (int)keep, (int)n_safe, a_star, budgets,
-                           nullptr, reinterpret_cast<int*>(base), st, &launches) != cudaSuccess)
+                           nullptr, reinterpret_cast<int*>(base), st, &launches) != cudaSuccess) {
+        cudaGetLastError();
         return NKV_ERR_CUDA;
+    }
     return NKV_OK;
 }

@@ -753,3 +753,34 @@ def test_host_entry_point_reports_a_device_status_behind_thousands_of_chunks():
             nkv.nkv_debug_set("inject_host_status", 0)
     nkv.nkv_compress_host(K, K, r, out, staging, 2)
     assert int(out.budgets.sum()) == G * H * k
+
+
+@pytest.mark.gpu
+def test_a_call_that_failed_leaves_no_error_for_the_next():
+    """A launch that the runtime refuses (the stream's capture has been invalidated, on the host): the call says so, and the
+    next one on a stream in order is not blamed for it."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.12")
+    K, V = _cache(200, 64, "bf16", H=2)
+    a_star = torch.rand((1, 2, 200), device=DEV)
+    budgets = nkv.nkv_budget(a_star, 0.5)
+    idx, offs, _ = nkv.nkv_select(a_star, budgets, 200)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    handle = ctypes.c_void_p(side.cuda_stream)
+    graph = ctypes.c_void_p()
+    K_out, V_out, ws = (torch.empty((1, 200, 64), dtype=K.dtype, device=DEV) for _ in range(3))
+    h = nkv.handle()
+    kt, vt = nkv._tensor(K), nkv._tensor(V)
+    assert rt.cudaStreamBeginCapture(handle, 2) == 0          # relaxed: other streams stay as they are
+    try:
+        assert rt.cudaStreamSynchronize(handle) != 0           # not allowed while capturing: ends the capture's validity
+        status = h.lib.nkv_compact(h.h, ctypes.byref(kt), ctypes.byref(vt), nkv._p(idx), nkv._p(offs), 200, nkv._p(K_out),
+                                   nkv._p(V_out), nkv.NKV_OUT_OF_PLACE, nkv._p(ws), ws.numel(), handle)
+    finally:
+        rt.cudaStreamEndCapture(handle, ctypes.byref(graph))
+        rt.cudaGetLastError()
+    assert status == nkv.NKV_ERR_CUDA
+    again, _, _ = nkv.nkv_select(a_star, budgets, 200)
+    torch.cuda.synchronize()
+    assert torch.equal(again, idx)
