@@ -3,9 +3,9 @@
 //
 // The dots of 128 keys with the anchors are one skinny product [128 x d] x [d x 16] per tile.  The fp32
 // anchors enter as three columns of the keys' type each (hi + mid + lo carries all 24 mantissa bits; products of
-// 16-bit numbers are exact in fp32 and tcgen05.mma accumulates in fp32; for fp16 the anchors, means of unit
-// vectors, are scaled by 2^10, which brings lo's quantum to 2^-34 of the anchors' scale), so a tile's right-hand
-// side is
+// 16-bit numbers are exact in fp32 and tcgen05.mma accumulates in fp32; for fp16 every anchor is scaled by the power
+// of two that brings its norm to 2^9 .. 2^10, whatever it was, which puts lo's quantum at 2^-34 of the norm or below), so a
+// tile's right-hand side is
 //     columns 0..2  mu_s        3..5  mu_e of the block the tile starts in        6..8  mu_e of the next block
 // (a tile of 128 keys touches at most two blocks because a block has at least 128 keys).  Key tiles are staged by TMA
 // (128-byte swizzle); the tensor core reads them from shared memory directly.  Warp roles: TMA producer, MMA issuer, four
@@ -49,7 +49,8 @@ struct Cfg {
     static constexpr size_t kRhsAt = (size_t)kSlots * kTileBytes;             // offsets of the parts behind the tiles
     static constexpr size_t kRowsAt = kRhsAt + (size_t)kRhs * kRhsBytes;      // [kAhead][2][kTile] floats
     static constexpr size_t kMuAt = kRowsAt + (size_t)kAhead * 2 * kTile * 4; // [kAhead][D] floats
-    static constexpr size_t kSmemAt = kMuAt + (size_t)kAhead * D * 4;
+    static constexpr size_t kInvAt = kMuAt + (size_t)kAhead * D * 4;          // [kAhead][D] floats (fp16: 1/||mu_e||)
+    static constexpr size_t kSmemAt = kInvAt + (size_t)kAhead * D * 4;
     static_assert(kSlots <= kMaxSlots, "barrier arrays too small");
 };
 
@@ -192,16 +193,25 @@ __device__ void dots_mma(unsigned char* tiles, unsigned char* rhs, Smem* s, uint
 }
 
 // Thread k writes column k of the nine right-hand-side rows of every block (rows 9..15 stay zero).
-template <typename T> constexpr float kAnchorScale = 1.f;
-template <> constexpr float kAnchorScale<__half> = 1024.f;
+// fp16 has five exponent bits: an anchor of norm 1 / inv enters times the power of two below inv, times 2^10, and inv's
+// mantissa is left for the epilogue (both exact).
+template <typename T> constexpr bool kScaled = false;
+template <> constexpr bool kScaled<__half> = true;
+constexpr float kAnchorScale = 1024.f;
+__device__ __forceinline__ float scale_of(float inv) { return __uint_as_float(__float_as_uint(inv) & 0x7f800000u) * kAnchorScale; }
+template <typename T>
+__device__ __forceinline__ float rest_of(float inv) {   // 1 / ||mu|| over the scale that the dots carry
+    return kScaled<T> ? __uint_as_float((__float_as_uint(inv) & 0x007fffffu) | 0x3f800000u) * (1.f / kAnchorScale) : inv;
+}
 template <typename T> __device__ __forceinline__ T narrow(float v);
 template <> __device__ __forceinline__ __nv_bfloat16 narrow<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 template <> __device__ __forceinline__ __half narrow<__half>(float v) { return __float2half_rn(v); }
 template <typename T> __device__ __forceinline__ float widen(T v) { return (float)v; }
 
 template <typename T, int D>
-__device__ void dots_prep(unsigned char* rhs, float* mu, Smem* s, ScoreParams sp, TileRange tr, int units, int N,
-                          const float* __restrict__ mu_s, const float* __restrict__ mu_e, int* status) {
+__device__ void dots_prep(unsigned char* rhs, float* mu, float* inv, Smem* s, ScoreParams sp, TileRange tr, int units, int N,
+                          const float* __restrict__ mu_s, const float* __restrict__ mu_e, const float* __restrict__ inv_s,
+                          const float* __restrict__ inv_e, int* status) {
     using C = Cfg<D>;
     const int k = threadIdx.x - kPrepWarp0 * 32, lane = k & 31;
     if (k >= D) return;   // d = 64 needs two of the four warps
@@ -214,11 +224,13 @@ __device__ void dots_prep(unsigned char* rhs, float* mu, Smem* s, ScoreParams sp
     auto fetch_to = [&](int64_t end) {
         for (; fetched < end; ++fetched) {
             if (fetched < rows) copy4(mu + (int)(fetched % kAhead) * D + k, mu_e + fetched * D + k);
+            if (kScaled<T> && fetched < rows) copy4(inv + (int)(fetched % kAhead) * D + k, inv_e + fetched);
             copies_commit();
         }
     };
     int cur_u = -1;
     float v[3] = {0.f, 0.f, 0.f}, s_next = mu_s[(int64_t)at.u * D + k];
+    float i_next = kScaled<T> ? inv_s[at.u] : 0.f;
     Ring<kRhs> r;
     bool fresh = true, wrapped = false;
     for (int n = 0; n < tr.count; ++n, fresh = at.next(N, sp.block)) {
@@ -228,18 +240,25 @@ __device__ void dots_prep(unsigned char* rhs, float* mu, Smem* s, ScoreParams sp
         copies_wait<kAhead - 2>();   // rows `row` and `row` + 1 are here
         if (at.u != cur_u) {
             cur_u = at.u;
-            v[0] = s_next;
-            if (cur_u + 1 < units) s_next = mu_s[(int64_t)(cur_u + 1) * D + k];
+            v[0] = kScaled<T> ? s_next * scale_of(i_next) : s_next;
+            if (cur_u + 1 < units) {
+                s_next = mu_s[(int64_t)(cur_u + 1) * D + k];
+                if (kScaled<T>) i_next = inv_s[cur_u + 1];
+            }
         }
-        v[1] = mu[(int)(row % kAhead) * D + k];
-        v[2] = at.blk + 1 < sp.nblocks ? mu[(int)((row + 1) % kAhead) * D + k] : 0.f;
+        const int here = (int)(row % kAhead) * D + k, after = (int)((row + 1) % kAhead) * D + k;
+        v[1] = mu[here];
+        v[2] = at.blk + 1 < sp.nblocks ? mu[after] : 0.f;
+        if (kScaled<T>) {
+            v[1] *= scale_of(inv[here]);
+            if (at.blk + 1 < sp.nblocks) v[2] *= scale_of(inv[after]);
+        }
         if (wrapped && !mbar_wait(&s->rfree[r.at], r.round ^ 1u, status, 715)) break;
         unsigned char* base = rhs + (size_t)r.at * C::kRhsBytes + (size_t)half * kRhsHalfBytes + (kk & 7) * 2;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float x = v[a] * kAnchorScale<T>;
-            const T hi = narrow<T>(x);
-            const float r1 = x - widen(hi);
+            const T hi = narrow<T>(v[a]);
+            const float r1 = v[a] - widen(hi);
             const T mid = narrow<T>(r1);
             const T lo = narrow<T>(r1 - widen(mid));
             const T part[3] = {hi, mid, lo};
@@ -303,11 +322,11 @@ __device__ void dots_epilogue(Smem* s, float* rows, uint32_t tmem_base, ScorePar
         if (at.u != cur_u) {
             flush();
             cur_u = at.u;
-            rs = rs_next;
+            rs = rest_of<T>(rs_next);
             if (cur_u + 1 < units) rs_next = inv_s[cur_u + 1];
         }
         copies_wait<kAhead - 1>();
-        const float inv_i = rows[(n % kAhead) * 2 * kTile + r], re = rows[((n % kAhead) * 2 + 1) * kTile + r];
+        const float inv_i = rows[(n % kAhead) * 2 * kTile + r], re = rest_of<T>(rows[((n % kAhead) * 2 + 1) * kTile + r]);
         fetch(n + kAhead);
         const int i = at.i0 + r;
         const bool second = i >= at.blk_end;   // the key lies in the block after the tile's first
@@ -321,9 +340,8 @@ __device__ void dots_epilogue(Smem* s, float* rows, uint32_t tmem_base, ScorePar
         if (lane == 0) mbar_arrive(&s->tempty[stage.at]);
         const float ds = d[0] + d[1] + d[2];
         const float de = second ? d[6] + d[7] + d[8] : d[3] + d[4] + d[5];
-        const float scaled = inv_i * (1.f / kAnchorScale<T>);
-        const float a_s = -(ds * scaled) * rs + 0.f;
-        const float a_e = -(de * scaled) * re + 0.f;
+        const float a_s = -(ds * inv_i) * rs + 0.f;
+        const float a_e = -(de * inv_i) * re + 0.f;
         if (i < N) {
             float* out = a_raw + (int64_t)cur_u * 3 * sp.raw_row + i;
             out[0] = a_s;
@@ -350,6 +368,7 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
     unsigned char* rhs = tiles + C::kRhsAt;
     float* rows = reinterpret_cast<float*>(tiles + C::kRowsAt);
     float* mu = reinterpret_cast<float*>(tiles + C::kMuAt);
+    float* inv = reinterpret_cast<float*>(tiles + C::kInvAt);
     Smem* s = reinterpret_cast<Smem*>(tiles + C::kSmemAt);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const TileRange tr = my_tiles(units, N);
@@ -388,7 +407,7 @@ anchor_dots_kernel(const __grid_constant__ CUtensorMap tmap, ScoreParams sp, int
     } else if (warp >= kEpiWarp0) {
         dots_epilogue<T>(s, rows, tmem_base, sp, tr, units, N, inv_norm, inv_s, inv_e, a_raw, mm, status);
     } else {
-        dots_prep<T, D>(rhs, mu, s, sp, tr, units, N, mu_s, mu_e, status);
+        dots_prep<T, D>(rhs, mu, inv, s, sp, tr, units, N, mu_s, mu_e, inv_s, inv_e, status);
     }
 
     tc_fence_before();

@@ -784,3 +784,23 @@ def test_a_call_that_failed_leaves_no_error_for_the_next():
     again, _, _ = nkv.nkv_select(a_star, budgets, 200)
     torch.cuda.synchronize()
     assert torch.equal(again, idx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,d", [("fp16", 64), ("fp16", 128), ("bf16", 128)])
+def test_anomalies_do_not_depend_on_the_length_of_the_anchors(dtype, d):
+    """nkv_score takes cosines: anchors that a caller brings longer (sums instead of means) or shorter give the same anomalies,
+    bit for bit where the factor is a power of two."""
+    K, _ = _cache(3000, d, dtype, H=4, layers=10)
+    p = nkv.nkv_default_params()
+    mu_s, mu_e, inv_norm, _ = nkv.nkv_anchors(K, p)
+    nkv.nkv_set_key_passes("tensor")
+    try:
+        raw = lambda f, g: nkv.nkv_score(K, mu_s * f, mu_e * g, inv_norm, p, want_raw=True)[1]
+        want = raw(1.0, 1.0)
+        for factor in (4096.0, 2.0 ** -20, 2.0 ** 40):
+            assert torch.equal(raw(factor, factor), want), factor
+        # the anchors' own rounding, 2^-24 each, and the same again in their norms
+        assert float((raw(3000.0, 0.3) - want).abs().max()) <= 1e-6
+    finally:
+        nkv.nkv_set_key_passes("auto")
