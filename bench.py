@@ -548,8 +548,8 @@ def run_e2e(args, cfg, r, K, V, h, params, dist, dev, world):
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
     dt = float(t.item())
     keys = groups * H * N * world
-    h2d = Kh.numel() * Kh.element_size() + Vh.numel() * Vh.element_size()
-    d2h = sum(x.numel() * x.element_size() for x in (out.k_out, out.v_out, out.idx, out.head_offsets, out.budgets))
+    # as the library moved them: K, and of a pinned V only the retained rows where they are fetched in place
+    h2d, d2h = nkv.nkv_host_bytes(h)
     return {"value": keys * steps / dt, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
             "steps": steps, "ms_per_step": 1e3 * dt / steps,
             "workload": "%d of %d layer groups per GPU, pinned host buffers, %d groups per staged chunk" % (

@@ -33,7 +33,8 @@
  *     with nkv_last_device_status after synchronising the stream.
  *   - Every function returns an nkv_status.  Argument errors are detected on
  *     the host before anything is launched; nothing throws or aborts.
- *   - Keys are assumed finite.  Non-finite keys are not detected.
+ *   - Keys are assumed finite, with a squared norm that fp32 holds.  Others are not detected: the scores of their head may be
+ *     NaN, which is ordered by its bits (above +inf), and no other head is touched.
  *   - r is the fraction of entries REMOVED (Section 3.1), 0 <= r < 1, and
  *     k = floor((1-r)*N) >= 1 must hold (evaluated in double).
  */
@@ -241,6 +242,10 @@ NKV_API int nkv_compress_host(nkv_handle* h, const nkv_tensor* K_host, const nkv
                       const nkv_params* params, void* K_out_host, void* V_out_host, int32_t* idx_host,
                       int32_t* head_offsets_host, int32_t* budgets_host, int64_t groups_per_chunk, void* dev,
                       size_t dev_bytes);
+
+/* Bytes that the handle's last nkv_compress_host moved: K and V (or V's retained rows, where they were fetched in place) to
+ * the device, and the outputs back (host pointers). */
+NKV_API int nkv_host_bytes(const nkv_handle* h, int64_t* in, int64_t* out);
 
 /* Reads the device status word of `ws` (synchronises `stream` first).
  * Returns NKV_OK, NKV_ERR_TIMEOUT, NKV_ERR_DEVICE_CHECK or NKV_ERR_CUDA. */

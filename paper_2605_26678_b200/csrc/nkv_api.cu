@@ -26,6 +26,7 @@ struct nkv_handle {
     cudaStream_t copy_streams[kHostSlots];
     int* chunk_status;   // pinned: the status code of every step of nkv_compress_host
     int64_t chunk_capacity;
+    int64_t host_in, host_out;   // bytes that the last nkv_compress_host moved to the device and back
     int inject_status;   // tests: status code planted in chunk `inject_chunk` of nkv_compress_host
     int inject_chunk;
 };
@@ -671,6 +672,8 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
         h->chunk_capacity = steps;
     }
 
+    h->host_in = G * (int64_t)(grp_in + (v_mapped ? grp_out : grp_in));
+    h->host_out = G * (int64_t)(2 * grp_out + (H * keep + 2 * H + 1) * 4);
     int result = NKV_OK;
     int64_t step = 0;
     for (int64_t g0 = 0; g0 < G && result == NKV_OK; g0 += p.groups, ++step) {
@@ -751,6 +754,13 @@ int nkv_get_stage_ms(nkv_handle* h, float* ms_out) {
     if (cudaEventSynchronize(h->ev[NKV_NUM_STAGES]) != cudaSuccess) return NKV_ERR_CUDA;
     for (int i = 0; i < NKV_NUM_STAGES; ++i)
         if (cudaEventElapsedTime(&ms_out[i], h->ev[i], h->ev[i + 1]) != cudaSuccess) return NKV_ERR_CUDA;
+    return NKV_OK;
+}
+
+int nkv_host_bytes(const nkv_handle* h, int64_t* in, int64_t* out) {
+    if (!h || !in || !out) return NKV_ERR_INVALID_ARG;
+    *in = h->host_in;
+    *out = h->host_out;
     return NKV_OK;
 }
 

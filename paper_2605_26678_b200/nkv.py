@@ -37,7 +37,7 @@ EXPORTS = (
     "nkv_workspace_bytes", "nkv_anchors", "nkv_score", "nkv_budget", "nkv_select", "nkv_compact",
     "nkv_compress", "nkv_host_staging_bytes", "nkv_compress_host", "nkv_last_device_status",
     "nkv_set_timing", "nkv_get_stage_ms", "nkv_launch_count", "nkv_budget_static", "nkv_set_key_passes",
-    "nkv_key_scan", "nkv_debug_set", "nkv_debug_wait_probe",
+    "nkv_key_scan", "nkv_debug_set", "nkv_debug_wait_probe", "nkv_host_bytes",
 )
 
 
@@ -108,6 +108,7 @@ def load_library():
     L.nkv_host_staging_bytes.argtypes = [vp, i64, i64, i64, i32, dbl, pp, i64, ctypes.POINTER(sz)]
     L.nkv_compress_host.argtypes = [vp, tp, tp, dbl, pp, vp, vp, vp, vp, vp, i64, vp, sz]
     L.nkv_last_device_status.argtypes = [vp, vp, vp]
+    L.nkv_host_bytes.argtypes = [vp, ctypes.POINTER(i64), ctypes.POINTER(i64)]
     L.nkv_set_timing.argtypes = [vp, ctypes.c_int]
     L.nkv_get_stage_ms.argtypes = [vp, ctypes.POINTER(ctypes.c_float)]
     L.nkv_launch_count.argtypes = [vp]
@@ -287,9 +288,7 @@ def nkv_budget(a_star: torch.Tensor, r: float, params: Optional[Params] = None,
     a_star = a_star.contiguous()
     G, H, N = a_star.shape
     budgets = torch.empty((G, H), dtype=torch.int32, device=a_star.device)
-    # status words, thresholds and the scratch of the parallel form of the group competition
-    ws = ws if ws is not None else torch.empty(8192 + 16 * G * H + G * H * 8192 + G * (256 + 5 * 8192), dtype=torch.uint8,
-                                               device=a_star.device)
+    ws = ws if ws is not None else torch.empty(512 + (8 * G * H + 255) // 256 * 256, dtype=torch.uint8, device=a_star.device)
     thresholds = torch.empty((G, H), dtype=torch.float32, device=a_star.device) if want_thresholds else None
     _check(h.lib.nkv_budget(h.h, _p(a_star), G, H, N, float(r), ctypes.byref(params), _p(budgets), _p(thresholds), _p(ws),
                             ws.numel(), _stream()), "nkv_budget")
@@ -407,6 +406,14 @@ def nkv_compress_host(K: torch.Tensor, V: torch.Tensor, r: float, out: Compresse
     return out
 
 
+def nkv_host_bytes(h: Optional[Handle] = None) -> Tuple[int, int]:
+    """Bytes that the last nkv_compress_host moved to the device and back."""
+    h = h or handle()
+    a, b = ctypes.c_int64(), ctypes.c_int64()
+    _check(h.lib.nkv_host_bytes(h.h, ctypes.byref(a), ctypes.byref(b)), "nkv_host_bytes")
+    return int(a.value), int(b.value)
+
+
 def nkv_last_device_status(ws: torch.Tensor, h: Optional[Handle] = None) -> int:
     h = h or handle()
     return int(h.lib.nkv_last_device_status(h.h, _p(ws), _stream()))
@@ -433,7 +440,7 @@ KEY_PASS = {"auto": 0, "fma": 1, "tensor": 2}
 
 
 def nkv_set_key_passes(mode: str = "auto", h: Optional[Handle] = None) -> None:
-    """Kernels of the two key passes: "auto", "fma" or "tensor" (bf16, d = 128 only); see nkv.h."""
+    """Kernels of the two key passes: "auto", "fma" or "tensor" (16-bit keys, W = 64, blocks of 128 or more); see nkv.h."""
     h = h or handle()
     _check(h.lib.nkv_set_key_passes(h.h, KEY_PASS[mode]), "nkv_set_key_passes")
 

@@ -590,6 +590,10 @@ def test_host_entry_point_with_rows_fetched_in_place_and_copied(layers, chunk, r
                            (dev.k_out, dev.v_out, dev.idx, dev.head_offsets, dev.budgets)], None)
     staging = torch.empty(nkv.nkv_host_staging_bytes(3, 700, 64, nkv.NKV_BF16, r, chunk), dtype=torch.uint8, device=DEV)
     nkv.nkv_compress_host(Kh, Vh, r, out, staging, chunk)
+    size = lambda t: t.numel() * t.element_size()
+    in_place = pinned and r >= 0.4
+    assert nkv.nkv_host_bytes() == (size(K) + size(out.v_out if in_place else V),
+                                    sum(size(t) for t in (out.k_out, out.v_out, out.idx, out.head_offsets, out.budgets)))
     for a, b in ((out.k_out, dev.k_out), (out.v_out, dev.v_out), (out.idx, dev.idx), (out.head_offsets, dev.head_offsets),
                  (out.budgets, dev.budgets)):
         assert torch.equal(a, b.cpu())
