@@ -17,7 +17,6 @@ constexpr int kHostSlots = 4;   // staging slots of nkv_compress_host, a stream 
 struct nkv_handle {
     int device;
     int sm_count;
-    int l2_bytes;
     int64_t launches;
     int timing;
     int timing_valid;
@@ -113,7 +112,7 @@ int check_tensor(const nkv_tensor* t) {
     return NKV_OK;
 }
 
-// Some score-side kernels put the heads on gridDim.y.
+// The bound that calls on keys have always had (heads once lay on gridDim.y).
 int check_units(int64_t units) { return units > 65535 ? NKV_ERR_UNSUPPORTED : NKV_OK; }
 
 TensorView view_of(const nkv_tensor* t) {
@@ -193,6 +192,8 @@ Bufs bufs_at(void* ws, const Layout& L) {
 //     d = 64    17 MB of keys 52 / 54 / 56   33 MB 69 / 70 / 69   67 MB 106 / 100 / 99 (64 x 8192), 99 / 102 / 102 (128 x 4096)
 //     d = 128   17 MB 53 / 54 / 54           33 MB 66 / 62 / 62   67 MB 98 / 84 / 84
 // With keys that are not in L2, 41 MB of 16 x 8 x 2500 x 64 at r = 0.5: 84.7 with the second pass in FMA form, 85.5 with none.
+// (For d = 64 the two forms of the second pass are within a percent or two of each other from 33 to 67 MB: where its line lies
+// between them matters little.)
 constexpr int kFirstPassKb = 192, kSecondPassKb64 = 320, kSecondPassKb128 = 192;   // of keys per SM
 bool tensor_pays(const nkv_handle* h, const TensorView& kv, int G, const ScoreParams& sp, int kb) {
     const int64_t bytes = (int64_t)G * kv.H * kv.N * kv.d * 2;
@@ -400,7 +401,6 @@ int nkv_create(nkv_handle** out, int device) {
         return NKV_ERR_CUDA;
     }
     h->sm_count = prop.multiProcessorCount;
-    h->l2_bytes = prop.l2CacheSize;
     h->key_pass = NKV_KEY_PASS_AUTO;
     if (configure_scan_kernels() != cudaSuccess || configure_stream_kernels() != cudaSuccess ||
         configure_gram_kernels() != cudaSuccess ||

@@ -68,33 +68,22 @@ __device__ __forceinline__ bool bar_or(int id, int count, bool pred) {
         : "memory");
     return r != 0;
 }
-__device__ __forceinline__ void bar_sync(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
 
 // ---------------------------------------------------------------------------- TMA
-// One box of a 4-d tiled tensor map into shared memory; c0 is the innermost coordinate (c0 * element
-// size must be a multiple of 16 bytes).  Rows outside the tensor arrive as zeros.
-__device__ __forceinline__ void tma_load_4d(void* dst_smem, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-        "[%6];" ::"r"(smem_addr(dst_smem)),
-        "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_addr(bar))
-        : "memory");
-}
 __device__ __forceinline__ uint64_t l2_evict_normal_policy() {
     uint64_t policy;
     asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
     return policy;
 }
-// The same with an L2 cache policy.  Keys are read once per pass and are far larger than L2: marking their lines
-// "evict first" leaves L2 to what is read again (anchors, weights, the scores written for the next kernel).
+// Keys are read once per pass and are far larger than L2: marking their lines "evict first" leaves L2 to what is read again
+// (anchors, weights, the scores written for the next kernel).
 __device__ __forceinline__ uint64_t l2_evict_first_policy() {
     uint64_t policy;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
     return policy;
 }
+// One box of a 4-d tiled tensor map into shared memory, with an L2 cache policy; c0 is the innermost coordinate (c0 * element
+// size must be a multiple of 16 bytes).  Rows outside the tensor arrive as zeros.
 __device__ __forceinline__ void tma_load_4d(void* dst_smem, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             uint64_t* bar, uint64_t policy) {
     asm volatile(
@@ -115,24 +104,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {   
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// 32 consecutive fp32 columns of this warp's 32 lanes (lane i of the warp reads row lane_base + i).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // 16 consecutive fp32 columns of this warp's 32 lanes.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
@@ -181,8 +152,8 @@ __device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, float* v) {
 }
 
 // ---------------------------------------------------------------------------- UMMA (tcgen05.mma)
-// Shared-memory operand descriptor for a K-major bf16 tile stored as 8-row x 128-byte swizzle atoms
-// (the layout a 128B-swizzled TMA box of 64 bf16 columns produces): consecutive 8-row groups are
+// Shared-memory operand descriptor for a K-major tile of 16-bit numbers stored as 8-row x 128-byte swizzle atoms
+// (the layout a 128B-swizzled TMA box of 64 such columns produces): consecutive 8-row groups are
 // 1024 bytes apart.  `addr` is the shared address of the first row at the wanted K offset (a
 // multiple of 32 bytes inside the 128-byte atom row); the tile base must be 1024-byte aligned.
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t addr) {

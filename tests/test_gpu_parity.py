@@ -808,3 +808,45 @@ def test_anomalies_do_not_depend_on_the_length_of_the_anchors(dtype, d):
         assert float((raw(3000.0, 0.3) - want).abs().max()) <= 1e-6
     finally:
         nkv.nkv_set_key_passes("auto")
+
+
+@pytest.mark.gpu
+def test_own_roots_and_quotients_against_64_bits():
+    """The Newton steps behind the approximate reciprocal root, over their range and at its floor: 1/||k|| of keys with one
+    component (its square is exact), a_c of unit keys along two axes (integers over the root of an integer), and the
+    surprise's extremes."""
+    rng = np.random.default_rng(5)
+    N, H = 256, 40
+    p = nkv.nkv_default_params()
+    K = np.zeros((1, H, N, 64), np.float32)
+    K[..., 3] = np.exp2(rng.uniform(-60.0, 60.0, (1, H, N)))
+    K = torch.from_numpy(K).to(torch.bfloat16).to(DEV)
+    nkv.nkv_set_key_passes("tensor")
+    try:
+        inv = nkv.nkv_key_scan(K, p)[0].cpu().numpy().astype(np.float64)
+        axis = torch.from_numpy((rng.random((1, H, N)) < rng.uniform(0.05, 0.95, (1, H, 1))).astype(np.int64)).to(DEV)
+        E = torch.nn.functional.one_hot(axis, 64).to(torch.bfloat16)
+        a_c = nkv.nkv_key_scan(E, p)[3][0, :, 2].cpu().numpy().astype(np.float64)
+    finally:
+        nkv.nkv_set_key_passes("auto")
+    norm = K[..., 3].double().cpu().numpy()
+    # 2^-24 for each of the two roundings behind the last Newton step, and as much again for the floor (1e-24 in fp32)
+    assert np.abs(inv * np.maximum(norm, 1e-12) - 1.0).max() <= 2.0 ** -22
+    ax = axis[0].cpu().numpy()
+    for h in range(H):
+        ones = np.concatenate([[0], np.cumsum(ax[h])])
+        end = np.arange(1, N + 1)
+        beg = np.maximum(0, end - 64)
+        n1 = ones[end] - ones[beg]
+        n0 = (end - beg) - n1
+        want = -np.where(ax[h] == 1, n1, n0) / np.sqrt(n0.astype(np.float64) ** 2 + n1.astype(np.float64) ** 2)
+        assert np.abs(a_c[h] / want - 1.0).max() <= 2.0 ** -21   # root and quotient, each corrected once
+    C, _ = _cache(2000, 64, "bf16", H=4, layers=10)
+    mu_s, mu_e, inv_norm, _ = nkv.nkv_anchors(C, p)
+    _, raw, stats = nkv.nkv_score(C, mu_s, mu_e, inv_norm, p, want_raw=True, want_stats=True)
+    raw, stats = raw.double().cpu().numpy(), stats.double().cpu().numpy()
+    lo, hi = raw.min(-1, keepdims=True), raw.max(-1, keepdims=True)
+    s = ((raw - lo) / (hi - lo)).std(2)
+    # three normalised values, each within 2^-22 of its own (difference, reciprocal of the range, product); a deviation moves
+    # by no more than they do, and the arithmetic behind adds 2^-23
+    assert np.abs(stats[..., 12] - s.min(-1)).max() <= 2.0 ** -21 and np.abs(stats[..., 13] - s.max(-1)).max() <= 2.0 ** -21
