@@ -660,7 +660,9 @@ int nkv_compress_host(nkv_handle* h, const nkv_tensor* Kh, const nkv_tensor* Vh,
     // Only the retained rows of V are needed on the device.  Where the device can read V in place (pinned memory) the
     // gather kernel fetches them from there, which spares the bus the others.  16 x 8 heads of 8192 x 64 bf16 keys: with
     // a quarter of the rows kept 5.34 -> 3.52 ms, with half 5.67 -> 4.92, with three quarters 6.06 -> 6.60, where one
-    // copy is the better way; the two meet at about 0.6 of the rows.
+    // copy is the better way; the two meet between 0.6 and 0.7 of the rows.  The same with rows of 256 and
+    // 512 bytes: half of the rows kept 9.79 / 11.35 and 18.9 / 22.3 ms, 0.6 of them 11.05 / 11.58 and 21.5 / 22.8, 0.7 12.29 / 11.78
+    // and 23.9 / 23.2 (in place / copied).
     const void* v_mapped = (double)keep <= kHostRowsShare * (double)N ? device_address(Vh->ptr, (size_t)G * grp_in) : nullptr;
 
     const int64_t steps = (G + p.groups - 1) / p.groups;
