@@ -26,23 +26,27 @@
 // and ||S_i||^2 follows from T_i = T_{i-1} + (2 c_i - g_ii) - (2 f_{i-W} - g_{i-W,i-W}), a prefix sum over
 // the tile that restarts every tile from an exact value (the sum of the 64 x 64 Gram block that ends at
 // the previous tile's last row, which is in that tile's D).  f is read with a lag of 64 rows, when every row of its
-// column has been seen.  Only the block sums of normalised keys need the key values themselves and stay on the FMA
-// pipes.  (As a second product, K[tile]^T x (1/||k|| split three ways into bf16), it was slower: 280 cycles per K step
-// with the tile as the transposed A operand, 290 to 400 with it as the MN-major B operand, all issued by one thread.)
+// column has been seen.  The block sums of normalised keys are a second product, K[tile]^T x (1/||k|| split three ways into
+// bf16), with the tile as the transposed A operand; fp16 keys form them on the FMA pipes (kFmaSums).
 //
 // The CTA is a pipeline of warp groups:
 //     producer (1 thread)    TMA loads of the stages
-//     mma      (1 warp)      the Gram rectangle of the tile
+//     mma      (1 warp)      issues the Gram rectangle of the tile
 //     band     (2 x 4 warps) the two groups take alternate tiles: norms from the diagonal, then row and column
 //                            sums of the band and the row's part of the next exact restart value
-//     sums     (8 warps)     block sums of normalised keys, kept in registers over the block
+//     sums     (4 warps)     issue the product behind the block sums, add it up over the block (fp16: 8 warps, on FMA pipes)
 //     scan     (2 warps)     alternate tiles: prefix sum, a_c, outputs, min/max
 // Groups hand work to each other through mbarriers; every wait is bounded and a group that gives up
 // records where and leaves, which makes the others give up in turn.
 //
-// Bound: instruction issue (60 % of the slots) and the hand-over chain of a tile; DRAM is the floor.  Measured at
-// 144 x 8 heads of 32768 x 128 bf16 keys (9.66 GB): 3.07 ms for the form before (one CTA per head, a product of N = 256
-// with the forward band read from its own columns), 2.23 ms for this one.
+// Bound: the hand-over chain of a tile (accumulator freed, product issued, product done, norms, band loaded: two tiles in
+// flight) and the issue of the Gram products by one warp; DRAM is the floor.  What moved it last: with the block sums on
+// the FMA pipes a tile of 128 x 128 took 4981 warp instructions, a third of them for these; on the tensor cores it takes
+// 3290, and the 16 warps left have 128 registers each, with which a band warp takes the whole band out of tensor memory
+// before it works on it.  36 x 8 heads of 8192 x 128 bf16 keys: 155 -> 132 us (93 at the copy rate); 16 x 8 x 32768 x 64: 222
+// -> 187.
+#include <type_traits>
+
 #include "nkv_sm100.cuh"
 
 namespace nkv {
@@ -55,14 +59,23 @@ constexpr int kTile = 128;                    // keys per tile (rows of D)
 constexpr int kHalo = 64;                     // keys in front of a tile (W = 64)
 constexpr int kStageHalfBytes = kTile * 128;  // one 64-column half of a stage
 constexpr int kHaloHalfBytes = kHalo * 128;
-constexpr int kBandGroup = 128, kSumsThreads = 256;
-constexpr int kSumsWarp0 = 8, kScanWarp0 = 16, kProducerWarp = 18, kMmaWarp = 19;
-constexpr int kThreads = 20 * 32;
+constexpr int kBandGroup = 128;
+constexpr int kSumsWarp0 = 8;
 constexpr int kWRing = 8;                     // tiles whose per-row scalars (1/||k||, g_ii) are kept
 constexpr int kCfRing = 4;                    // band -> scan hand-over buffers
-constexpr uint32_t kTmemCols = 512;           // two accumulators of 192 columns, 256 apart
+constexpr int kRhsRing = 4;                   // tiles whose split norms are kept
+constexpr uint32_t kTmemCols = 512;           // two Gram accumulators of 192 columns, two of block sums of 64
+constexpr uint32_t kGramCols = kTile + kHalo, kSumsAt = 2 * kGramCols, kSumsCols = 64;
 constexpr int kBarSums = 1;                   // named barrier
 constexpr int kBandCols = 96;                 // columns a quarter of the tile's rows can reach
+
+// The warps of a CTA.  kFma: block sums on the FMA pipes (eight warps) instead of the tensor cores (four).
+template <bool kFma>
+struct Warps {
+    static constexpr int kSums = kFma ? 8 : 4, kSumsThreads = kSums * 32;
+    static constexpr int kScan0 = kSumsWarp0 + kSums, kProducer = kScan0 + 2, kMma = kScan0 + 3;
+    static constexpr int kThreads = (kMma + 1) * 32;
+};
 
 template <int D>
 struct Cfg {
@@ -70,15 +83,18 @@ struct Cfg {
     static constexpr int kStages = D == 128 ? 5 : 7;
     static constexpr int kHalfBytes = kHaloHalfBytes + kStages * kStageHalfBytes;   // halo copy, then all stages of one half
     static constexpr int kRingBytes = kHalves * kHalfBytes;
-    static constexpr int kLanes = D / 8;                   // lanes per row in the sums group (8 columns each)
-    static constexpr int kGroups = kSumsThreads / kLanes;  // row groups of the sums group
+    static constexpr int kLanes = D / 8;                   // lanes per row in the FMA sums group (8 columns each)
+    static constexpr int kGroups = Warps<true>::kSumsThreads / kLanes;   // row groups of that group
     static constexpr int kRowsPerGroup = kTile / kGroups;
+    // Norms as the right-hand side of the block sums' product: 16 rows of kRhsKeys keys.  With d = 64 the upper half of the
+    // product's rows takes the upper half of the tile's keys, for which rows 8 .. 15 hold the norms.
+    static constexpr int kRhsKeys = D, kRhsBytes = 16 * kRhsKeys * 2;
 };
 constexpr int kMaxStages = 7;
 
-template <int D>
+template <int D, bool kFma>
 struct Smem {
-    float red[2][kSumsThreads / 32][D];   // block sums by warp, at the end of a block
+    float red[2][kFma ? 8 : 1][kFma ? D : 64];   // block sums by warp (d = 64: of the upper rows), at the end of a block
     float w[kWRing][kTile];      // 1/||k|| by row (0 outside the head)
     float g[kWRing][kTile];      // g_ii by row
     float zero[kHalo];           // the weights of the rows before a span
@@ -86,20 +102,23 @@ struct Smem {
     float f[kCfRing][4][kBandCols];   // column sums of the tile's band by row quarter (columns 32 q .. 32 q + 95 of D)
     float bp[kCfRing][kTile];    // row's share of the Gram block of the tile's last 64 rows
     uint64_t full[kMaxStages];   // stage landed
-    uint64_t sfree[kMaxStages];  // stage no longer needed (the sums warps, and the product of the next tile)
+    uint64_t sfree[kMaxStages];  // stage no longer needed (the tile's block sums, and the product of the next tile)
     uint64_t tfull[2];           // accumulator written
     uint64_t tempty[2];          // accumulator read (one arrival per warp of the band group)
     uint64_t wready[kWRing];     // 1/||k|| of a tile written (one arrival per warp)
     uint64_t cready[kCfRing];    // band sums of a tile written (one arrival per warp)
     uint64_t cfree[kCfRing];     // band sums of a tile consumed (by the scans of the tile and of the next)
-    uint64_t drain;              // products issued before a give-up have completed
+    uint64_t sdone[kRhsRing];    // block sums of a tile formed: accumulator written, split norms no longer needed
+    uint64_t sempty[2];          // accumulator of block sums read (one arrival per warp)
+    uint64_t drain[5];           // products issued before a give-up have completed, by issuing warp
     uint32_t tmem_base;
 };
 static_assert(kMaxStages < kWRing, "a tile's 1/||k|| has to outlive its stage");
-static_assert(1024 + Cfg<128>::kRingBytes + sizeof(Smem<128>) <= 232448 && 1024 + Cfg<64>::kRingBytes + sizeof(Smem<64>) <= 232448,
+template <int D, bool kFma>
+constexpr size_t smem_bytes() { return 1024 + (size_t)Cfg<D>::kRingBytes + (kFma ? 0 : kRhsRing * Cfg<D>::kRhsBytes) + sizeof(Smem<D, kFma>); }
+static_assert(smem_bytes<128, false>() <= 232448 && smem_bytes<64, false>() <= 232448 && smem_bytes<128, true>() <= 232448 &&
+                  smem_bytes<64, true>() <= 232448,
               "more shared memory than an SM has");
-template <int D>
-constexpr size_t smem_bytes() { return 1024 + (size_t)Cfg<D>::kRingBytes + sizeof(Smem<D>); }
 
 // The spans of a CTA: blocks [first, last) of the call (head-major), cut at head boundaries.
 struct Walk {
@@ -175,8 +194,8 @@ __device__ __forceinline__ void treduce(float* v, int l) {
 
 // ---------------------------------------------------------------------------- producer and MMA
 // TMA producer (one thread): the tiles of every span, in order.  Rows behind the head arrive as zeros.
-template <int D>
-__device__ void producer_role(const CUtensorMap* tmap, unsigned char* ring, Smem<D>* s, Walk walk, int block, int N, int H,
+template <int D, bool kFma>
+__device__ void producer_role(const CUtensorMap* tmap, unsigned char* ring, Smem<D, kFma>* s, Walk walk, int block, int N, int H,
                               bool keep_in_l2, int* status) {
     using C = Cfg<D>;
     uint32_t n = 0;
@@ -216,31 +235,40 @@ __device__ void producer_role(const CUtensorMap* tmap, unsigned char* ring, Smem
 }
 
 // MMA issuer (one warp).  A = the tile's 128 rows, B = those rows and the 64 in front of them.
-template <typename T, int D>
-__device__ void mma_role(unsigned char* ring, Smem<D>* s, uint32_t tmem_base, Walk walk, int block, int N, int* status) {
-    using C = Cfg<D>;
-    constexpr uint32_t idesc = umma_idesc<T>(kTile, kTile + kHalo);
-    const uint32_t ring_addr = smem_addr(ring);
-    uint32_t n = 0;
+__device__ __forceinline__ uint32_t count_tiles(Walk walk, int block, int N) {
+    uint32_t tiles = 0;
     Span sp;
 #pragma unroll 1
-    while (next_span(walk, block, N, sp)) {
+    while (next_span(walk, block, N, sp)) tiles += (uint32_t)sp.tiles;
+    return tiles;
+}
+template <typename T, int D, bool kFma>
+__device__ void mma_role(unsigned char* ring, Smem<D, kFma>* s, uint32_t tmem_base, Walk walk, int block, int N, int* status) {
+    using C = Cfg<D>;
+    constexpr uint32_t idesc = umma_idesc<T>(kTile, kTile + kHalo);
+    const uint32_t ring_addr = smem_addr(ring), tiles = count_tiles(walk, block, N);
+    int st = 0, before = 0;
+    uint32_t round = 0;
 #pragma unroll 1
-        for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
-            const int st = (int)(n % C::kStages), acc = (int)(n & 1);
-            if (!warp_wait(&s->full[st], (n / C::kStages) & 1u, status, 702)) return umma_drain(&s->drain);
-            if (!warp_wait(&s->tempty[acc], ((n >> 1) & 1u) ^ 1u, status, 703)) return umma_drain(&s->drain);
-            tc_fence_after();
-            // the address field of a descriptor counts 16-byte units: a K step moves it by a constant
-            const uint64_t bdesc = umma_desc_sw128(ring_addr + (uint32_t)st * kStageHalfBytes);
-            const uint64_t adesc = umma_desc_sw128(ring_addr + (uint32_t)st * kStageHalfBytes + kHaloHalfBytes);
+    for (uint32_t n = 0; n < tiles; ++n) {
+        const uint32_t acc = n & 1u;
+        if (!warp_wait(&s->full[st], round, status, 702)) return umma_drain(&s->drain[0]);
+        if (!warp_wait(&s->tempty[acc], ((n >> 1) & 1u) ^ 1u, status, 703)) return umma_drain(&s->drain[0]);
+        tc_fence_after();
+        // the address field of a descriptor counts 16-byte units: a K step moves it by a constant
+        const uint64_t bdesc = umma_desc_sw128(ring_addr + (uint32_t)st * kStageHalfBytes);
+        const uint64_t adesc = umma_desc_sw128(ring_addr + (uint32_t)st * kStageHalfBytes + kHaloHalfBytes);
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                const uint64_t koff = (uint64_t)((uint32_t)(kk >> 2) * (uint32_t)(C::kHalfBytes >> 4) + (uint32_t)(kk & 3) * 2u);
-                umma_f16(tmem_base + (uint32_t)acc * 256u, adesc + koff, bdesc + koff, idesc, kk > 0);
-            }
-            umma_commit(&s->tfull[acc]);
-            if (n > 0) umma_commit(&s->sfree[(n - 1) % C::kStages]);   // the tile before has been read as the rows in front
+        for (int kk = 0; kk < D / 16; ++kk) {
+            const uint64_t koff = (uint64_t)((uint32_t)(kk >> 2) * (uint32_t)(C::kHalfBytes >> 4) + (uint32_t)(kk & 3) * 2u);
+            umma_f16(tmem_base + acc * kGramCols, adesc + koff, bdesc + koff, idesc, kk > 0);
+        }
+        umma_commit(&s->tfull[acc]);
+        if (n > 0) umma_commit(&s->sfree[before]);   // the tile before has been read as the rows in front
+        before = st;
+        if (++st == C::kStages) {
+            st = 0;
+            round ^= 1u;
         }
     }
 }
@@ -249,10 +277,11 @@ __device__ void mma_role(unsigned char* ring, Smem<D>* s, uint32_t tmem_base, Wa
 // Sums of normalised keys per episodic block.  Lane group grp (8 columns per lane) takes rows
 // [grp * R, grp * R + R) of every tile and keeps its running sum in registers until the block ends; then the groups'
 // parts are added up over the warp and in shared memory.
-template <typename T, int D, bool kGiven>
-__device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int block, int N, float* __restrict__ block_sums,
+template <typename T, int D>
+__device__ void sums_role(const unsigned char* ring, Smem<D, true>* s, Walk walk, int block, int N, float* __restrict__ block_sums,
                           int* status) {
     using C = Cfg<D>;
+    constexpr int kSumsThreads = Warps<true>::kSumsThreads;
     constexpr int R = C::kRowsPerGroup;
     const int t = threadIdx.x - kSumsWarp0 * 32, lane = t & 31;
     const int grp = t / C::kLanes, l = t % C::kLanes, r0 = grp * R;
@@ -288,7 +317,7 @@ __device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int 
             while (true) {
                 const int cut = min(end - R0, hi);
                 const int a = lo - r0, b = cut - r0;        // the same in rows of this group
-                if (!kGiven && a < R && b > 0) {
+                if (a < R && b > 0) {
                     float v[R];
 #pragma unroll
                     for (int i = 0; i < R; ++i) v[i] = w[i];
@@ -324,7 +353,7 @@ __device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int 
                     *reinterpret_cast<float4*>(dst + 4) = make_float4(o[4], o[5], o[6], o[7]);
                 }
                 if (bar_or(kBarSums, kSumsThreads, false)) return;
-                if (!kGiven && t < D) {
+                if (t < D) {
                     float sum = 0.f;
 #pragma unroll
                     for (int q = 0; q < kSumsThreads / 32; ++q) sum += s->red[flushes & 1][q][t];
@@ -338,6 +367,90 @@ __device__ void sums_role(const unsigned char* ring, Smem<D>* s, Walk walk, int 
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&s->sfree[st]);
+        }
+    }
+}
+
+// The same from the tensor cores: row c of a tile's accumulator is channel c (d = 64: rows c and 64 + c, of the lower and of
+// the upper 64 keys), its columns are the products with the three parts of the norms of the block that is open where the
+// tile starts and of the next one, in sums over 32 keys each.  These are added up in fp32.  Relative error of a sum of 256
+// keys, root mean square against 64 bits: 4.0e-8, as in the FMA form (4.1e-8); with all keys of a tile added in tensor
+// memory, which truncates, 1.1e-7.
+// The four warps read the accumulator and take turns at issuing the products, a tile ahead: one warp for these and the Gram
+// products needed 1900 cycles per tile, each step of it being a wait or an issue of 150 to 550.
+template <typename T, int D>
+__device__ void tensor_sums_role(unsigned char* ring, const unsigned char* rhs, Smem<D, false>* s, uint32_t tmem_base, Walk walk, int block,
+                                 int N, float* __restrict__ block_sums, int* status) {
+    using C = Cfg<D>;
+    constexpr int kSumsThreads = Warps<false>::kSumsThreads, kParts = C::kRhsKeys / 32;
+    const int t = threadIdx.x - kSumsWarp0 * 32, lane = t & 31, q = t >> 5;
+    const bool upper = D == 64 && q >= 2;
+    const uint32_t at = tmem_base + ((uint32_t)(32 * q) << 16) + kSumsAt + (upper ? 8u : 0u);
+    const uint32_t ring_addr = smem_addr(ring), rhs_addr = smem_addr(rhs), tiles = count_tiles(walk, block, N);
+    auto issue = [&](uint32_t m) {   // A = the tile's keys with the channels as rows, B = its split norms
+        constexpr uint32_t idesc = umma_idesc<T>(kTile, 16) | kTransposeA;
+        const uint32_t st = m % C::kStages, buf = m & 1u, rs = m & (kRhsRing - 1);
+        if (!warp_wait(&s->wready[m & (kWRing - 1)], (m / kWRing) & 1u, status, 717)) return false;
+        if (!warp_wait(&s->sempty[buf], ((m >> 1) & 1u) ^ 1u, status, 718)) return false;
+        tc_fence_after();
+        // the channels' second 64 rows: the other half of the stage (d = 128), or the upper 64 keys (d = 64)
+        const uint64_t adesc = umma_desc_sw128_mn(ring_addr + st * kStageHalfBytes + kHaloHalfBytes,
+                                                  D == 128 ? (uint32_t)C::kHalfBytes : (uint32_t)kHaloHalfBytes);
+        const uint64_t bdesc = umma_desc_sw128(rhs_addr + rs * C::kRhsBytes);
+#pragma unroll
+        for (int kk = 0; kk < C::kRhsKeys / 16; ++kk)   // 32 keys per sum in tensor memory
+            umma_f16(tmem_base + kSumsAt + buf * kSumsCols + (uint32_t)(kk >> 1) * 16u, adesc + (uint64_t)(kk * 2048 >> 4),
+                     bdesc + (uint64_t)((kk >> 2) * 2048 + (kk & 3) * 32 >> 4), idesc, kk & 1);
+        umma_commit(&s->sdone[rs]);
+        umma_commit(&s->sfree[st]);
+        return true;
+    };
+    auto give_up = [&] {
+        umma_drain(&s->drain[1 + q]);
+        if (D == 64) bar_or(kBarSums, kSumsThreads, true);
+    };
+    uint32_t n = 0, flushes = 0;
+    Span sp;
+    if (q == 0 && tiles > 0 && !issue(0)) return give_up();
+#pragma unroll 1
+    while (next_span(walk, block, N, sp)) {
+        int blk = sp.blk, end = min(sp.row0 + block, N);   // the open block and the row it ends before
+        float acc = 0.f;
+#pragma unroll 1
+        for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
+            const int rs = (int)(n & (kRhsRing - 1)), buf = (int)(n & 1);
+            if (((n + 1) & 3u) == (uint32_t)q && n + 1 < tiles && !issue(n + 1)) return give_up();
+            if (!warp_wait(&s->sdone[rs], (n / kRhsRing) & 1u, status, 719)) return give_up();
+            tc_fence_after();
+            float v[kParts][8];
+            tmem_ld8<kParts, 16>(at + (uint32_t)buf * kSumsCols, v);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s->sempty[buf]);
+            float part[6];
+#pragma unroll
+            for (int p = 0; p < 6; ++p) {
+                if constexpr (kParts == 4) part[p] = (v[0][p] + v[1][p]) + (v[2][p] + v[3][p]);
+                else part[p] = v[0][p] + v[1][p];
+            }
+            acc += part[0] + (part[1] + part[2]);
+            const int stop = min(sp.base + kTile * (tau + 1), sp.row1);
+            float next = part[3] + (part[4] + part[5]);
+#pragma unroll 1
+            while (end <= stop) {   // the block ends in this tile
+                if constexpr (D == 64) {
+                    if (upper) s->red[flushes & 1][0][t - 64] = acc;
+                    if (bar_or(kBarSums, kSumsThreads, false)) return umma_drain(&s->drain[1 + q]);
+                    if (!upper) acc += s->red[flushes & 1][0][t];
+                    ++flushes;   // the other buffer next: the barrier of its use orders these reads before the next writes here
+                }
+                if (!upper) block_sums[((int64_t)sp.u * walk.nb + blk) * D + t] = acc;
+                if (end >= sp.row1) break;
+                acc = next;
+                next = 0.f;
+                ++blk;
+                end = min(end + block, N);
+            }
         }
     }
 }
@@ -384,16 +497,45 @@ __device__ __forceinline__ void chunk_sums(const float (*v)[16], const float* wc
     }
 }
 
-template <int D, bool kGiven>
-__device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, int N, const float* __restrict__ given, int64_t inv_row,
-                          int* status) {
+// Norms of the quarter's rows, one per lane: lane t has row lr = 8 (t % 4) + t / 4.  The diagonal entries of rows t / 4 + 8 J,
+// in columns 8 J + b0 + e with e = (t / 4) % 2, are held by lane t / 8 of the four lanes that share these rows.
+__device__ __forceinline__ float own_diagonal(const float (*z)[16], int t) {
+    float G = 0.f;
+#pragma unroll
+    for (int J = 0; J < 4; ++J) {
+        const float* c = z[J >> 1] + 4 * J + 2 * (J & 1);
+        const float d = __shfl_sync(0xffffffffu, (t & 4) ? c[1] : c[0], (t & 28) | (t >> 3));
+        if ((t & 3) == J) G = d;
+    }
+    return G;
+}
+// A row's norm in three bf16 parts (24 mantissa bits), as column `row` of the right-hand side of the block sums' product: in
+// rows 0 .. 2 for a key of the block that is open where the tile starts, 3 .. 5 for one of the next; zeros otherwise.
+template <int D>
+__device__ __forceinline__ void split_norm(unsigned char* rhs, int row, float w, bool first, bool second) {
+    const int kk = row & 63;
+    unsigned char* at = rhs + (row >> 6) * (D == 128 ? 2048 : 1024) + (kk & 7) * 2;
+    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+    const float r1 = w - __bfloat162float(hi);
+    const __nv_bfloat16 mid = __float2bfloat16_rn(r1), lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+    const uint16_t part[3] = {__bfloat16_as_ushort(hi), __bfloat16_as_ushort(mid), __bfloat16_as_ushort(lo)};
+#pragma unroll
+    for (int line = 0; line < 6; ++line)
+        *reinterpret_cast<uint16_t*>(at + line * 128 + (((kk >> 3) ^ line) << 4)) = (line < 3 ? first : second) ? part[line % 3] : (uint16_t)0;
+}
+
+// kSums: the norms go to the tensor cores as well.  kEarly (128 registers per thread): the whole band is loaded at once, and
+// the next product into this accumulator is not held up by the arithmetic.
+template <int D, bool kFma, bool kGiven, bool kSums>
+__device__ void band_role(unsigned char* rhs, Smem<D, kFma>* s, uint32_t tmem_base, Walk walk, int block, int N,
+                          const float* __restrict__ given, int64_t inv_row, int* status) {
+    constexpr bool kEarly = !kFma;
     const int warp = threadIdx.x >> 5, t = threadIdx.x & 31;
     const int q = warp & 3, which = warp >> 2;   // lane quarter; the group takes tiles n with n % 2 == which
     const int b0 = 2 * (t & 3), r0 = (t >> 2) + 1;
     const bool p0 = b0 >= r0, p1 = b0 + 1 >= r0;
-    const bool owner = (t & 3) == (t >> 3);      // holds diagonal entries: column 8 J + b0 + e, e = (t / 4) % 2
-    const int oe = (t >> 2) & 1;
-    const uint32_t tq = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(which * 256 + 32 * q);
+    const int own = 32 * q + 8 * (t & 3) + (t >> 2);   // the lane's own row where every lane has one
+    const uint32_t tq = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)which * kGramCols + (uint32_t)(32 * q);
     // Columns 0 .. 63 of a span's first tile are products with whatever the ring holds, keys of another head among it.  They
     // are dropped and not only weighed with 0, which an infinity or a NaN among them would survive.
     auto drop = [](float(&v)[2][16]) {
@@ -404,41 +546,47 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
     Span sp;
 #pragma unroll 1
     while (next_span(walk, block, N, sp)) {
+        int end = sp.row0 + block;   // of the block that is open where the tile starts
 #pragma unroll 1
         for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
+            const int R0 = sp.base + kTile * tau;
+            if (kSums && end <= R0) end += block;   // (a block has at least a tile's keys)
             if ((int)(n & 1) != which) continue;
             const int slot = (int)(n & (kWRing - 1)), prev = (int)((n - 1) & (kWRing - 1)), cb = (int)(n & (kCfRing - 1));
-            float have[4];   // the norms of the quarter's rows, where the caller brings them
-            if constexpr (kGiven) {
-#pragma unroll
-                for (int J = 0; J < 4; ++J) {
-                    const int i = sp.base + kTile * tau + 32 * q + 8 * J + (t >> 2);
-                    have[J] = i < N ? given[sp.u * inv_row + i] : 0.f;
-                }
-            }
+            const int i = R0 + own;
+            const float have = kGiven && i < N ? given[sp.u * inv_row + i] : 0.f;
             if (!warp_wait(&s->tfull[which], (n >> 1) & 1u, status, 706)) return;
             tc_fence_after();
-            float z[2][16], y[2][16];
+            float z[2][16], y[2][16], x_early[2][16];
+            float(&x)[2][16] = *(kEarly ? &x_early : &z);
             tmem_ld_frag32(tq + 64, z[0]);
             tmem_ld_frag32(tq + 64 + (16u << 16), z[1]);
             tmem_wait_ld(z[0], z[1]);
-            if (owner) {   // 1/||k|| and g_ii of the quarter's rows
-                const int R0 = sp.base + kTile * tau;
-#pragma unroll
-                for (int J = 0; J < 4; ++J) {
-                    const float* c = z[J >> 1];
-                    const float G = oe ? c[4 * J + 2 * (J & 1) + 1] : c[4 * J + 2 * (J & 1)];
-                    const int row = 32 * q + 8 * J + (t >> 2);
-                    // 1 / max(||k||, eps)
-                    const float inv = kGiven ? have[J] : R0 + row < N ? inv_sqrt(fmaxf(G, kEps * kEps)) : 0.f;
-                    s->w[slot][row] = inv;
-                    s->g[slot][row] = inv * inv * G;
-                }
+            tmem_ld_frag32(tq + 32, y[0]);
+            tmem_ld_frag32(tq + 32 + (16u << 16), y[1]);
+            if constexpr (kEarly) {
+                tmem_ld_frag32(tq, x[0]);
+                tmem_ld_frag32(tq + (16u << 16), x[1]);
+            }
+            const float G = own_diagonal(z, t);
+            const float wi = kGiven ? have : i < N ? inv_sqrt(fmaxf(G, kEps * kEps)) : 0.f;   // 1 / max(||k||, eps)
+            s->w[slot][own] = wi;
+            s->g[slot][own] = wi * wi * G;
+            if constexpr (kSums) {
+                const int rs = (int)(n & (kRhsRing - 1));
+                if (!warp_wait(&s->sdone[rs], ((n / kRhsRing) & 1u) ^ 1u, status, 720)) return;
+                split_norm<D>(rhs + rs * Cfg<D>::kRhsBytes, own, wi, i >= sp.row0 && i < end && i < sp.row1, i >= end && i < sp.row1);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads these writes
             }
             __syncwarp();
             if (t == 0) mbar_arrive(&s->wready[slot]);
-            tmem_ld_frag32(tq + 32, y[0]);
-            tmem_ld_frag32(tq + 32 + (16u << 16), y[1]);
+            if constexpr (kEarly) {
+                tmem_wait_ld(y[0], y[1]);
+                tmem_wait_ld(x[0], x[1]);
+                tc_fence_before();
+                __syncwarp();
+                if (t == 0) mbar_arrive(&s->tempty[which]);
+            }
             float wrow[4];
 #pragma unroll
             for (int J = 0; J < 4; ++J) wrow[J] = s->w[slot][32 * q + 8 * J + (t >> 2)];
@@ -454,21 +602,25 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
             const float* before = tau > 0 ? &s->w[prev][kTile - kHalo] : s->zero;   // columns 0 .. 63
             const float* wy = q >= 1 ? &s->w[slot][32 * q - 32] : before + 32;
             const float* wx = q >= 2 ? &s->w[slot][32 * q - 64] : before + 32 * q;
-            tmem_wait_ld(y[0], y[1]);
+            if constexpr (!kEarly) {
+                tmem_wait_ld(y[0], y[1]);
+                tmem_ld_frag32(tq, x[0]);
+                tmem_ld_frag32(tq + (16u << 16), x[1]);
+            }
             if (tau == 0 && q == 0) drop(y);
-            tmem_ld_frag32(tq, z[0]);
-            tmem_ld_frag32(tq + (16u << 16), z[1]);
             chunk_sums<kChunkY>(y, wy + b0, wrow, p0, p1, row, cy);
             if (q == 3) {
 #pragma unroll
                 for (int J = 0; J < 4; ++J) part[J] = row[J];
             }
-            tmem_wait_ld(z[0], z[1]);
-            tc_fence_before();
-            __syncwarp();
-            if (t == 0) mbar_arrive(&s->tempty[which]);
-            if (tau == 0 && q < 2) drop(z);
-            chunk_sums<kChunkX>(z, wx + b0, wrow, p0, p1, row, cx);
+            if constexpr (!kEarly) {
+                tmem_wait_ld(x[0], x[1]);
+                tc_fence_before();
+                __syncwarp();
+                if (t == 0) mbar_arrive(&s->tempty[which]);
+            }
+            if (tau == 0 && q < 2) drop(x);
+            chunk_sums<kChunkX>(x, wx + b0, wrow, p0, p1, row, cx);
 
             // row sums over the four lanes of a row; afterwards lane t holds row 8 (t % 4) + t / 4 of the quarter
             float tot[4];
@@ -496,16 +648,14 @@ __device__ void band_role(Smem<D>* s, uint32_t tmem_base, Walk walk, int block, 
                     }
             }
             if (!warp_wait(&s->cfree[cb], ((n / kCfRing) & 1u) ^ 1u, status, 709)) return;
-            const int lr = 8 * (t & 3) + (t >> 2);
-            const float wi = s->w[slot][32 * q + lr];
-            s->c[cb][32 * q + lr] = wi * tot[0];
+            s->c[cb][own] = wi * tot[0];
             // Gram block of the tile's last 64 rows: columns 128 .. diagonal of rows 64 .. 127
             if (q >= 2) {
                 float pt[4];
 #pragma unroll
                 for (int J = 0; J < 4; ++J) pt[J] = hsum2(part[J]);
                 treduce<4, 4>(pt, t & 3);
-                s->bp[cb][32 * q + lr] = wi * pt[0];
+                s->bp[cb][own] = wi * pt[0];
             }
             const int m = t >> 2, lc = 8 * (m >> 1) + b0 + (m & 1);
 #pragma unroll
@@ -527,10 +677,10 @@ __device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x, a
 
 // (Out of line: five roles share the instruction caches, and with this one inlined the pass took 158 instead of 154 us at
 // 36 x 8 heads of 8192 x 128 keys.)
-template <int D, bool kGiven>
-__device__ __noinline__ void scan_role(Smem<D>* s, Walk walk, int block, int N, float* __restrict__ inv_norm, int64_t inv_row,
+template <int D, bool kFma, bool kGiven>
+__device__ __noinline__ void scan_role(Smem<D, kFma>* s, Walk walk, int block, int N, float* __restrict__ inv_norm, int64_t inv_row,
                           float* __restrict__ a_raw, int64_t raw_row, uint32_t* __restrict__ mm, int* status) {
-    const int which = (threadIdx.x >> 5) - kScanWarp0, l = threadIdx.x & 31;
+    const int which = (threadIdx.x >> 5) - Warps<kFma>::kScan0, l = threadIdx.x & 31;
     const int r = 4 * l, q = l >> 3, c = r - 32 * q;
     uint32_t n = 0;
     Span sp;
@@ -612,42 +762,53 @@ __device__ __noinline__ void scan_role(Smem<D>* s, Walk walk, int block, int N, 
     }
 }
 
+// Block sums of bf16 keys come from the tensor cores.  fp16 keys would need their norms as fp16 numbers, whose range is short
+// of what norms span, so theirs stay on the FMA pipes.
+template <typename T, bool kGiven> constexpr bool kFmaSums = !kGiven && std::is_same<T, __half>::value;
+
 template <typename T, int D, bool kGiven>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Warps<kFmaSums<T, kGiven>>::kThreads, 1)
 gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblocks, int units, int H, int N, bool keep_in_l2,
                  const float* __restrict__ given, float* __restrict__ block_sums, float* __restrict__ inv_norm, int64_t inv_row, float* __restrict__ a_raw,
                  int64_t raw_row, uint32_t* __restrict__ mm, int* status) {
     using C = Cfg<D>;
+    constexpr bool kFma = kFmaSums<T, kGiven>, kSums = !kFma && !kGiven;
+    using W = Warps<kFma>;
     extern __shared__ unsigned char smem_raw[];
     // the swizzle atoms (8 rows x 128 bytes) must start on 1024-byte boundaries
     unsigned char* ring = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-    Smem<D>* s = reinterpret_cast<Smem<D>*>(ring + C::kRingBytes);
+    unsigned char* rhs = ring + C::kRingBytes;
+    Smem<D, kFma>* s = reinterpret_cast<Smem<D, kFma>*>(rhs + (kFma ? 0 : kRhsRing * C::kRhsBytes));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
         for (int i = 0; i < C::kStages; ++i) {
             mbar_init(&s->full[i], 1);
-            mbar_init(&s->sfree[i], kSumsThreads / 32 + 1);
+            mbar_init(&s->sfree[i], kFma ? W::kSums + 1 : kSums ? 2 : 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&s->tfull[i], 1);
             mbar_init(&s->tempty[i], kBandGroup / 32);
         }
-        mbar_init(&s->drain, 1);
+        for (int i = 0; i < 5; ++i) mbar_init(&s->drain[i], 1);
         for (int i = 0; i < kWRing; ++i) mbar_init(&s->wready[i], kBandGroup / 32);
         for (int i = 0; i < kCfRing; ++i) {
             mbar_init(&s->cready[i], kBandGroup / 32);
             mbar_init(&s->cfree[i], 2);
         }
+        for (int i = 0; i < kRhsRing; ++i) mbar_init(&s->sdone[i], 1);
+        for (int i = 0; i < 2; ++i) mbar_init(&s->sempty[i], W::kSums);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < kHalo) s->zero[tid] = 0.f;
     // (the rows in front of the first tile, which count for nothing)
     for (int half = 0; half < C::kHalves; ++half)
-        for (int i = tid; i < kHaloHalfBytes / 16; i += kThreads)
+        for (int i = tid; i < kHaloHalfBytes / 16; i += W::kThreads)
             reinterpret_cast<uint4*>(ring + half * C::kHalfBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (kSums)
+        for (int i = tid; i < kRhsRing * C::kRhsBytes / 16; i += W::kThreads) reinterpret_cast<uint4*>(rhs)[i] = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (warp == kMmaWarp) tmem_alloc(&s->tmem_base, kTmemCols);
+    if (warp == W::kMma) tmem_alloc(&s->tmem_base, kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -655,23 +816,24 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
     pdl_wait();
     const Walk walk = my_walk(units, nblocks);
 
-    if (warp == kProducerWarp) {
-        if (lane == 0) producer_role<D>(&tmap, ring, s, walk, block, N, H, keep_in_l2, status);
+    if (warp == W::kProducer) {
+        if (lane == 0) producer_role<D, kFma>(&tmap, ring, s, walk, block, N, H, keep_in_l2, status);
         __syncwarp();
-    } else if (warp == kMmaWarp) {
-        mma_role<T, D>(ring, s, tmem_base, walk, block, N, status);
+    } else if (warp == W::kMma) {
+        mma_role<T, D, kFma>(ring, s, tmem_base, walk, block, N, status);
         __syncwarp();
-    } else if (warp >= kScanWarp0) {
-        scan_role<D, kGiven>(s, walk, block, N, inv_norm, inv_row, a_raw, raw_row, mm, status);
+    } else if (warp >= W::kScan0) {
+        scan_role<D, kFma, kGiven>(s, walk, block, N, inv_norm, inv_row, a_raw, raw_row, mm, status);
     } else if (warp >= kSumsWarp0) {
-        sums_role<T, D, kGiven>(ring, s, walk, block, N, block_sums, status);
+        if constexpr (kFma) sums_role<T, D>(ring, s, walk, block, N, block_sums, status);
+        else if constexpr (kSums) tensor_sums_role<T, D>(ring, rhs, s, tmem_base, walk, block, N, block_sums, status);
     } else {
-        band_role<D, kGiven>(s, tmem_base, walk, block, N, given, inv_row, status);
+        band_role<D, kFma, kGiven, kSums>(rhs, s, tmem_base, walk, block, N, given, inv_row, status);
     }
 
     tc_fence_before();
     __syncthreads();
-    if (warp == kMmaWarp) tmem_dealloc(tmem_base, kTmemCols);
+    if (warp == W::kMma) tmem_dealloc(tmem_base, kTmemCols);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -697,9 +859,13 @@ cudaError_t launch_typed(const CUtensorMap& tmap, const TensorView& K, int units
                          cudaStream_t stream) {
     const long long total = (long long)units * sp.nblocks;
     const unsigned grid = (unsigned)(total < sm_count ? total : sm_count);
-    auto kernel = given ? gram_pass_kernel<T, D, true> : gram_pass_kernel<T, D, false>;
-    return launch_chained(kernel, grid, kThreads, smem_bytes<D>(), stream, 1, tmap, sp.block, sp.nblocks, units, K.H, K.N, keep_in_l2, given,
-                          block_sums, inv_norm, sp.inv_row, a_raw, sp.raw_row, mm, status);
+    auto launch = [&](auto kernel, int threads, size_t smem) {
+        return launch_chained(kernel, grid, (unsigned)threads, smem, stream, 1, tmap, sp.block, sp.nblocks, units, K.H, K.N, keep_in_l2, given,
+                              block_sums, inv_norm, sp.inv_row, a_raw, sp.raw_row, mm, status);
+    };
+    if (given) return launch(gram_pass_kernel<T, D, true>, Warps<false>::kThreads, smem_bytes<D, false>());
+    constexpr bool kFma = kFmaSums<T, false>;
+    return launch(gram_pass_kernel<T, D, false>, Warps<kFma>::kThreads, smem_bytes<D, kFma>());
 }
 
 }  // namespace
@@ -723,9 +889,9 @@ cudaError_t configure_gram_kernels() {
     cudaError_t e;
 #define NKV_SET(T, D)                                                                                                    \
     if ((e = cudaFuncSetAttribute(gram_pass_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,            \
-                                  (int)smem_bytes<D>())) != cudaSuccess ||                                               \
+                                  (int)smem_bytes<D, kFmaSums<T, false>>())) != cudaSuccess ||                           \
         (e = cudaFuncSetAttribute(gram_pass_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,             \
-                                  (int)smem_bytes<D>())) != cudaSuccess)                                                  \
+                                  (int)smem_bytes<D, false>())) != cudaSuccess)                                          \
         return e
     NKV_SET(__nv_bfloat16, 64);
     NKV_SET(__nv_bfloat16, 128);

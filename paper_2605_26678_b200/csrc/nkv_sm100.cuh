@@ -119,6 +119,26 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// kCount groups of 8 consecutive fp32 columns of this warp's 32 lanes, kApart columns apart, and the wait for them.
+template <int kCount, int kApart>
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (*v)[8]) {
+    static_assert(kCount == 2 || kCount == 4, "two or four groups");
+    uint32_t r[4][8];
+#pragma unroll
+    for (int k = 0; k < kCount; ++k)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[k][0]), "=r"(r[k][1]), "=r"(r[k][2]), "=r"(r[k][3]), "=r"(r[k][4]), "=r"(r[k][5]), "=r"(r[k][6]), "=r"(r[k][7])
+                     : "r"(taddr + (uint32_t)(k * kApart))
+                     : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int k = 0; k < kCount; ++k) {   // no use is scheduled above the wait
+        asm volatile("" : "+r"(r[k][0]), "+r"(r[k][1]), "+r"(r[k][2]), "+r"(r[k][3]), "+r"(r[k][4]), "+r"(r[k][5]), "+r"(r[k][6]), "+r"(r[k][7]));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[k][i] = __uint_as_float(r[k][i]);
+    }
+}
+
 // Wait for the tensor-memory loads issued so far; a and b (16 values each) are the registers the loads
 // fill, named here so that no use of them is scheduled above the wait.
 __device__ __forceinline__ void tmem_wait_ld(float* a, float* b) {
@@ -165,6 +185,18 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t addr) {
     d |= (uint64_t)2 << 61;                     // 128-byte swizzle
     return d;
 }
+// The same for an operand that lies in memory with its rows along K, 64 columns (M or N) per atom: `addr` is the first atom
+// of the wanted K offset (16 rows per K step, so a multiple of 2048 bytes), the next 64 columns are `next64` bytes on.
+__device__ __forceinline__ uint64_t umma_desc_sw128_mn(uint32_t addr, uint32_t next64) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3ffffu) >> 4);    // start address
+    d |= (uint64_t)(next64 >> 4) << 16;         // leading byte offset: between atoms along M or N
+    d |= (uint64_t)(1024 >> 4) << 32;           // stride byte offset: between 8-row groups along K
+    d |= (uint64_t)1 << 46;                     // descriptor version of sm_100
+    d |= (uint64_t)2 << 61;                     // 128-byte swizzle
+    return d;
+}
+constexpr uint32_t kTransposeA = 1u << 15;      // instruction descriptor: A lies that way
 // Instruction descriptor: bf16 x bf16 or fp16 x fp16 -> fp32, both operands K-major, tile M x N.
 template <typename T> constexpr uint32_t kOperandType = 1u;            // bf16
 template <> inline constexpr uint32_t kOperandType<__half> = 0u;

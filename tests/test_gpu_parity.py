@@ -850,3 +850,32 @@ def test_own_roots_and_quotients_against_64_bits():
     # three normalised values, each within 2^-22 of its own (difference, reciprocal of the range, product); a deviation moves
     # by no more than they do, and the arithmetic behind adds 2^-23
     assert np.abs(stats[..., 12] - s.min(-1)).max() <= 2.0 ** -21 and np.abs(stats[..., 13] - s.max(-1)).max() <= 2.0 ** -21
+
+
+@pytest.mark.parametrize("N,d,layers", [(128, 128, 1), (129, 64, 1), (1000, 64, 2), (4133, 128, 2), (6000, 64, 1), (6000, 128, 1),
+                                        (8193, 128, 1), (8320, 64, 1)])
+def test_block_sums_of_the_tensor_pass(N, d, layers):
+    """Means of normalised keys whose norms span many powers of two (zero keys among them), against 64 bits.  Blocks that
+    end inside a tile, on its edge and after one key.  A sum of 32 terms in tensor memory may lose 2**-24 of its largest
+    term per addition and the few additions behind it as much of the sum, so a mean is off by less than 44 * 2**-24 of
+    the largest component (the root mean square, as of the FMA form, is 4e-8 of a component's)."""
+    g = torch.Generator().manual_seed(N + d)
+    K = torch.randn((layers, 3, N, d), generator=g) + 2.0 * torch.randn((layers, 3, 1, d), generator=g)
+    K *= torch.exp(3.0 * torch.randn((layers, 3, N, 1), generator=g))
+    K[:, :, ::37] = 0
+    K = K.to(torch.bfloat16).to(DEV)
+    p = nkv.nkv_default_params()
+    nkv.nkv_set_key_passes("tensor")
+    try:
+        _, mu_s, mu_e, _, _ = nkv.nkv_key_scan(K, p)
+        torch.cuda.synchronize()
+    finally:
+        nkv.nkv_set_key_passes("auto")
+    k = K.double()
+    k = k / k.norm(dim=3, keepdim=True).clamp(min=1e-12)
+    b = nkv.nkv_block_size(N, p)
+    want = torch.stack([k[:, :, i:i + b].mean(2) for i in range(0, N, b)], 2)
+    err = mu_e.double() - want
+    assert err.abs().max() <= 44 * 2.0 ** -24 * k.abs().max()
+    assert err.square().mean().sqrt() <= 2e-7 * want.square().mean().sqrt()
+    assert (mu_s.double() - k.mean(2)).abs().max() <= 44 * 2.0 ** -24 * k.abs().max()
