@@ -44,7 +44,7 @@
 // the FMA pipes a tile of 128 x 128 took 4981 warp instructions, a third of them for these; on the tensor cores it takes
 // 3290, and the 16 warps left have 128 registers each, with which a band warp takes the whole band out of tensor memory
 // before it works on it.  36 x 8 heads of 8192 x 128 bf16 keys: 155 -> 132 us (93 at the copy rate); 16 x 8 x 32768 x 64: 222
-// -> 187.
+// -> 183.
 #include <type_traits>
 
 #include "nkv_sm100.cuh"
@@ -63,7 +63,7 @@ constexpr int kBandGroup = 128;
 constexpr int kSumsWarp0 = 8;
 constexpr int kWRing = 8;                     // tiles whose per-row scalars (1/||k||, g_ii) are kept
 constexpr int kCfRing = 4;                    // band -> scan hand-over buffers
-constexpr int kRhsRing = 4;                   // tiles whose split norms are kept
+constexpr int kSumsRing = 4;                  // tiles whose block sums may be under way
 constexpr uint32_t kTmemCols = 512;           // two Gram accumulators of 192 columns, two of block sums of 64
 constexpr uint32_t kGramCols = kTile + kHalo, kSumsAt = 2 * kGramCols, kSumsCols = 64;
 constexpr int kBarSums = 1;                   // named barrier
@@ -88,6 +88,7 @@ struct Cfg {
     static constexpr int kRowsPerGroup = kTile / kGroups;
     // Norms as the right-hand side of the block sums' product: 16 rows of kRhsKeys keys.  With d = 64 the upper half of the
     // product's rows takes the upper half of the tile's keys, for which rows 8 .. 15 hold the norms.
+    // One right-hand side goes with every stage.
     static constexpr int kRhsKeys = D, kRhsBytes = 16 * kRhsKeys * 2;
 };
 constexpr int kMaxStages = 7;
@@ -108,14 +109,15 @@ struct Smem {
     uint64_t wready[kWRing];     // 1/||k|| of a tile written (one arrival per warp)
     uint64_t cready[kCfRing];    // band sums of a tile written (one arrival per warp)
     uint64_t cfree[kCfRing];     // band sums of a tile consumed (by the scans of the tile and of the next)
-    uint64_t sdone[kRhsRing];    // block sums of a tile formed: accumulator written, split norms no longer needed
+    uint64_t rready[kMaxStages]; // split norms of a tile written (one arrival per warp)
+    uint64_t sdone[kSumsRing];   // block sums of a tile formed
     uint64_t sempty[2];          // accumulator of block sums read (one arrival per warp)
     uint64_t drain[5];           // products issued before a give-up have completed, by issuing warp
     uint32_t tmem_base;
 };
 static_assert(kMaxStages < kWRing, "a tile's 1/||k|| has to outlive its stage");
 template <int D, bool kFma>
-constexpr size_t smem_bytes() { return 1024 + (size_t)Cfg<D>::kRingBytes + (kFma ? 0 : kRhsRing * Cfg<D>::kRhsBytes) + sizeof(Smem<D, kFma>); }
+constexpr size_t smem_bytes() { return 1024 + (size_t)Cfg<D>::kRingBytes + (kFma ? 0 : Cfg<D>::kStages * Cfg<D>::kRhsBytes) + sizeof(Smem<D, kFma>); }
 static_assert(smem_bytes<128, false>() <= 232448 && smem_bytes<64, false>() <= 232448 && smem_bytes<128, true>() <= 232448 &&
                   smem_bytes<64, true>() <= 232448,
               "more shared memory than an SM has");
@@ -247,13 +249,12 @@ __device__ void mma_role(unsigned char* ring, Smem<D, kFma>* s, uint32_t tmem_ba
     using C = Cfg<D>;
     constexpr uint32_t idesc = umma_idesc<T>(kTile, kTile + kHalo);
     const uint32_t ring_addr = smem_addr(ring), tiles = count_tiles(walk, block, N);
-    int st = 0, before = 0;
+    int st = 0;
     uint32_t round = 0;
 #pragma unroll 1
     for (uint32_t n = 0; n < tiles; ++n) {
         const uint32_t acc = n & 1u;
-        if (!warp_wait(&s->full[st], round, status, 702)) return umma_drain(&s->drain[0]);
-        if (!warp_wait(&s->tempty[acc], ((n >> 1) & 1u) ^ 1u, status, 703)) return umma_drain(&s->drain[0]);
+        if (!warp_wait2(&s->full[st], round, &s->tempty[acc], ((n >> 1) & 1u) ^ 1u, status, 702)) return umma_drain(&s->drain[0]);
         tc_fence_after();
         // the address field of a descriptor counts 16-byte units: a K step moves it by a constant
         const uint64_t bdesc = umma_desc_sw128(ring_addr + (uint32_t)st * kStageHalfBytes);
@@ -263,9 +264,7 @@ __device__ void mma_role(unsigned char* ring, Smem<D, kFma>* s, uint32_t tmem_ba
             const uint64_t koff = (uint64_t)((uint32_t)(kk >> 2) * (uint32_t)(C::kHalfBytes >> 4) + (uint32_t)(kk & 3) * 2u);
             umma_f16(tmem_base + acc * kGramCols, adesc + koff, bdesc + koff, idesc, kk > 0);
         }
-        umma_commit(&s->tfull[acc]);
-        if (n > 0) umma_commit(&s->sfree[before]);   // the tile before has been read as the rows in front
-        before = st;
+        umma_commit(&s->tfull[acc]);   // (a commit takes 170 cycles to issue: whoever waits for this one frees the stage, too)
         if (++st == C::kStages) {
             st = 0;
             round ^= 1u;
@@ -389,20 +388,18 @@ __device__ void tensor_sums_role(unsigned char* ring, const unsigned char* rhs, 
     const uint32_t ring_addr = smem_addr(ring), rhs_addr = smem_addr(rhs), tiles = count_tiles(walk, block, N);
     auto issue = [&](uint32_t m) {   // A = the tile's keys with the channels as rows, B = its split norms
         constexpr uint32_t idesc = umma_idesc<T>(kTile, 16) | kTransposeA;
-        const uint32_t st = m % C::kStages, buf = m & 1u, rs = m & (kRhsRing - 1);
-        if (!warp_wait(&s->wready[m & (kWRing - 1)], (m / kWRing) & 1u, status, 717)) return false;
-        if (!warp_wait(&s->sempty[buf], ((m >> 1) & 1u) ^ 1u, status, 718)) return false;
+        const uint32_t st = m % C::kStages, buf = m & 1u;
+        if (!warp_wait2(&s->rready[st], (m / C::kStages) & 1u, &s->sempty[buf], ((m >> 1) & 1u) ^ 1u, status, 717)) return false;
         tc_fence_after();
         // the channels' second 64 rows: the other half of the stage (d = 128), or the upper 64 keys (d = 64)
         const uint64_t adesc = umma_desc_sw128_mn(ring_addr + st * kStageHalfBytes + kHaloHalfBytes,
                                                   D == 128 ? (uint32_t)C::kHalfBytes : (uint32_t)kHaloHalfBytes);
-        const uint64_t bdesc = umma_desc_sw128(rhs_addr + rs * C::kRhsBytes);
+        const uint64_t bdesc = umma_desc_sw128(rhs_addr + st * C::kRhsBytes);
 #pragma unroll
         for (int kk = 0; kk < C::kRhsKeys / 16; ++kk)   // 32 keys per sum in tensor memory
             umma_f16(tmem_base + kSumsAt + buf * kSumsCols + (uint32_t)(kk >> 1) * 16u, adesc + (uint64_t)(kk * 2048 >> 4),
                      bdesc + (uint64_t)((kk >> 2) * 2048 + (kk & 3) * 32 >> 4), idesc, kk & 1);
-        umma_commit(&s->sdone[rs]);
-        umma_commit(&s->sfree[st]);
+        umma_commit(&s->sdone[m & (kSumsRing - 1)]);
         return true;
     };
     auto give_up = [&] {
@@ -418,9 +415,10 @@ __device__ void tensor_sums_role(unsigned char* ring, const unsigned char* rhs, 
         float acc = 0.f;
 #pragma unroll 1
         for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
-            const int rs = (int)(n & (kRhsRing - 1)), buf = (int)(n & 1);
+            const int rs = (int)(n & (kSumsRing - 1)), buf = (int)(n & 1);
             if (((n + 1) & 3u) == (uint32_t)q && n + 1 < tiles && !issue(n + 1)) return give_up();
-            if (!warp_wait(&s->sdone[rs], (n / kRhsRing) & 1u, status, 719)) return give_up();
+            if (!warp_wait(&s->sdone[rs], (n / kSumsRing) & 1u, status, 719)) return give_up();
+            if (t == 0) mbar_arrive(&s->sfree[n % C::kStages]);
             tc_fence_after();
             float v[kParts][8];
             tmem_ld8<kParts, 16>(at + (uint32_t)buf * kSumsCols, v);
@@ -543,12 +541,18 @@ __device__ void band_role(unsigned char* rhs, Smem<D, kFma>* s, uint32_t tmem_ba
         for (int i = 0; i < 32; ++i) v[i >> 4][i & 15] = 0.f;
     };
     uint32_t n = 0;
+    int st = 0, last = 0;   // stages of the tile and of the one before
+    auto step = [&] {
+        ++n;
+        last = st;
+        st = st + 1 == Cfg<D>::kStages ? 0 : st + 1;
+    };
     Span sp;
 #pragma unroll 1
     while (next_span(walk, block, N, sp)) {
         int end = sp.row0 + block;   // of the block that is open where the tile starts
 #pragma unroll 1
-        for (int tau = 0; tau < sp.tiles; ++tau, ++n) {
+        for (int tau = 0; tau < sp.tiles; ++tau, step()) {
             const int R0 = sp.base + kTile * tau;
             if (kSums && end <= R0) end += block;   // (a block has at least a tile's keys)
             if ((int)(n & 1) != which) continue;
@@ -556,6 +560,7 @@ __device__ void band_role(unsigned char* rhs, Smem<D, kFma>* s, uint32_t tmem_ba
             const int i = R0 + own;
             const float have = kGiven && i < N ? given[sp.u * inv_row + i] : 0.f;
             if (!warp_wait(&s->tfull[which], (n >> 1) & 1u, status, 706)) return;
+            if (q == 0 && t == 0 && n > 0) mbar_arrive(&s->sfree[last]);   // read as the rows in front of this tile
             tc_fence_after();
             float z[2][16], y[2][16], x_early[2][16];
             float(&x)[2][16] = *(kEarly ? &x_early : &z);
@@ -572,12 +577,6 @@ __device__ void band_role(unsigned char* rhs, Smem<D, kFma>* s, uint32_t tmem_ba
             const float wi = kGiven ? have : i < N ? inv_sqrt(fmaxf(G, kEps * kEps)) : 0.f;   // 1 / max(||k||, eps)
             s->w[slot][own] = wi;
             s->g[slot][own] = wi * wi * G;
-            if constexpr (kSums) {
-                const int rs = (int)(n & (kRhsRing - 1));
-                if (!warp_wait(&s->sdone[rs], ((n / kRhsRing) & 1u) ^ 1u, status, 720)) return;
-                split_norm<D>(rhs + rs * Cfg<D>::kRhsBytes, own, wi, i >= sp.row0 && i < end && i < sp.row1, i >= end && i < sp.row1);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads these writes
-            }
             __syncwarp();
             if (t == 0) mbar_arrive(&s->wready[slot]);
             if constexpr (kEarly) {
@@ -586,6 +585,12 @@ __device__ void band_role(unsigned char* rhs, Smem<D, kFma>* s, uint32_t tmem_ba
                 tc_fence_before();
                 __syncwarp();
                 if (t == 0) mbar_arrive(&s->tempty[which]);
+            }
+            if constexpr (kSums) {   // (the stage's earlier right-hand side was used up before the stage was filled again)
+                split_norm<D>(rhs + st * Cfg<D>::kRhsBytes, own, wi, i >= sp.row0 && i < end && i < sp.row1, i >= end && i < sp.row1);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads these writes
+                __syncwarp();
+                if (t == 0) mbar_arrive(&s->rready[st]);
             }
             float wrow[4];
 #pragma unroll
@@ -597,8 +602,12 @@ __device__ void band_role(unsigned char* rhs, Smem<D, kFma>* s, uint32_t tmem_ba
 #pragma unroll
             for (int J = 0; J < 4; ++J) part[J] = row[J];
             // the other columns belong to rows of the other warps and of the tile before
-            if (!warp_wait(&s->wready[slot], (n / kWRing) & 1u, status, 707)) return;
-            if (q < 2 && tau > 0 && !warp_wait(&s->wready[prev], ((n - 1) / kWRing) & 1u, status, 708)) return;
+            {
+                const bool both = q < 2 && tau > 0;
+                if (!warp_wait2(&s->wready[slot], (n / kWRing) & 1u, &s->wready[both ? prev : slot], ((both ? n - 1 : n) / kWRing) & 1u,
+                                status, 707))
+                    return;
+            }
             const float* before = tau > 0 ? &s->w[prev][kTile - kHalo] : s->zero;   // columns 0 .. 63
             const float* wy = q >= 1 ? &s->w[slot][32 * q - 32] : before + 32;
             const float* wx = q >= 2 ? &s->w[slot][32 * q - 64] : before + 32 * q;
@@ -692,8 +701,8 @@ __device__ __noinline__ void scan_role(Smem<D, kFma>* s, Walk walk, int block, i
             if ((int)(n & 1) != which) continue;
             const int cb = (int)(n & (kCfRing - 1)), pb = (int)((n - 1) & (kCfRing - 1));
             const int slot = (int)(n & (kWRing - 1)), prev = (int)((n - 1) & (kWRing - 1));
-            if (!warp_wait(&s->cready[cb], (n / kCfRing) & 1u, status, 710)) return;
-            if (tau > 0 && !warp_wait(&s->cready[pb], ((n - 1) / kCfRing) & 1u, status, 714)) return;
+            if (!warp_wait2(&s->cready[cb], (n / kCfRing) & 1u, &s->cready[tau > 0 ? pb : cb], ((tau > 0 ? n - 1 : n) / kCfRing) & 1u, status, 710))
+                return;
             const float4 ci = ld4(&s->c[cb][r]), gi = ld4(&s->g[slot][r]), wi = ld4(&s->w[slot][r]);
             float4 F = ld4(&s->f[cb][q][c]);
             if (q >= 1) add4(F, ld4(&s->f[cb][q - 1][c + 32]));
@@ -778,13 +787,14 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
     // the swizzle atoms (8 rows x 128 bytes) must start on 1024-byte boundaries
     unsigned char* ring = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     unsigned char* rhs = ring + C::kRingBytes;
-    Smem<D, kFma>* s = reinterpret_cast<Smem<D, kFma>*>(rhs + (kFma ? 0 : kRhsRing * C::kRhsBytes));
+    Smem<D, kFma>* s = reinterpret_cast<Smem<D, kFma>*>(rhs + (kFma ? 0 : C::kStages * C::kRhsBytes));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
         for (int i = 0; i < C::kStages; ++i) {
             mbar_init(&s->full[i], 1);
             mbar_init(&s->sfree[i], kFma ? W::kSums + 1 : kSums ? 2 : 1);
+            mbar_init(&s->rready[i], kBandGroup / 32);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&s->tfull[i], 1);
@@ -796,7 +806,7 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
             mbar_init(&s->cready[i], kBandGroup / 32);
             mbar_init(&s->cfree[i], 2);
         }
-        for (int i = 0; i < kRhsRing; ++i) mbar_init(&s->sdone[i], 1);
+        for (int i = 0; i < kSumsRing; ++i) mbar_init(&s->sdone[i], 1);
         for (int i = 0; i < 2; ++i) mbar_init(&s->sempty[i], W::kSums);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -806,7 +816,7 @@ gram_pass_kernel(const __grid_constant__ CUtensorMap tmap, int block, int nblock
         for (int i = tid; i < kHaloHalfBytes / 16; i += W::kThreads)
             reinterpret_cast<uint4*>(ring + half * C::kHalfBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (kSums)
-        for (int i = tid; i < kRhsRing * C::kRhsBytes / 16; i += W::kThreads) reinterpret_cast<uint4*>(rhs)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < C::kStages * C::kRhsBytes / 16; i += W::kThreads) reinterpret_cast<uint4*>(rhs)[i] = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (warp == W::kMma) tmem_alloc(&s->tmem_base, kTmemCols);
     tc_fence_before();

@@ -58,6 +58,13 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, int* s
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, where));
 }
 
+// The same for two barriers, whose first looks overlap (a wait that finds its phase complete takes 150 cycles beside busy warps).
+__device__ __forceinline__ bool warp_wait2(uint64_t* a, uint32_t parity_a, uint64_t* b, uint32_t parity_b, int* status, int where) {
+    const bool oa = mbar_try_wait(a, parity_a), ob = mbar_try_wait(b, parity_b);
+    if (__all_sync(0xffffffffu, oa && ob)) return true;
+    return warp_wait(a, parity_a, status, where) && warp_wait(b, parity_b, status, where + 1);
+}
+
 // Named barrier over `count` threads that also ORs a predicate over them.
 __device__ __forceinline__ bool bar_or(int id, int count, bool pred) {
     uint32_t r;
