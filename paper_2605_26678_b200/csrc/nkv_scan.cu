@@ -1,7 +1,5 @@
 // Anchor and anomaly kernels: the two passes over the keys.
 //
-//   anchor_sums   (Section 2.1, 2.2)  1/||k_i|| per token and the sum of normalised
-//                                     keys of every episodic block
 //   anchor_means  (Section 2.2)       block means and the stable mean, their reciprocal norms
 //   anchor_norms                      the reciprocal norms of anchors that a caller brings
 //   scan_scores   (Section 2.3)       a_s, a_e, a_c of every token from one staged
@@ -65,59 +63,6 @@ __device__ __forceinline__ void store_cols(float* vec, int l, const float* v) {
                                    v[j * M::kPerChunk + e + 2], v[j * M::kPerChunk + e + 3]);
             *reinterpret_cast<float4*>(vec + M::col(l, j, e)) = f;
         }
-}
-
-// ------------------------------------------------------------------------------------------
-// anchor_sums: one CTA per (episodic block, head).
-// ------------------------------------------------------------------------------------------
-template <typename T, int D>
-__global__ void __launch_bounds__(256) anchor_sums_kernel(TensorView K, ScoreParams sp, float* __restrict__ block_sums,
-                                                          float* __restrict__ inv_norm) {
-    using M = RowMap<T, D>;
-    __shared__ float red[32][D];
-    const int u = blockIdx.x / sp.nblocks, t = blockIdx.x - u * sp.nblocks;
-    const int g = u / K.H, h = u % K.H;
-    const unsigned char* base =
-        reinterpret_cast<const unsigned char*>(K.ptr) + ((int64_t)g * K.stride_g + (int64_t)h * K.stride_h) * sizeof(T);
-    const int row0 = t * sp.block;
-    const int row1 = min(K.N, row0 + sp.block);
-    const int grp = threadIdx.x >> 3, l = threadIdx.x & 7;
-
-    float acc[M::kCols];
-#pragma unroll
-    for (int c = 0; c < M::kCols; ++c) acc[c] = 0.f;
-
-    const int iters = (sp.block + 31) / 32;
-#pragma unroll 2
-    for (int it = 0; it < iters; ++it) {
-        const int r = row0 + grp + 32 * it;
-        const bool ok = r < row1;
-        float v[M::kCols];
-        if (ok) {
-            load_row_chunks<T, D>(base + (int64_t)r * M::kRowBytes, l, v);
-        } else {
-#pragma unroll
-            for (int c = 0; c < M::kCols; ++c) v[c] = 0.f;
-        }
-        float ss = 0.f;
-#pragma unroll
-        for (int c = 0; c < M::kCols; ++c) ss = fmaf(v[c], v[c], ss);
-        ss = group8_sum(ss);
-        const float inv = 1.0f / fmaxf(sqrtf(ss), kEps);
-        if (ok) {
-#pragma unroll
-            for (int c = 0; c < M::kCols; ++c) acc[c] = fmaf(v[c], inv, acc[c]);
-            if (l == 0) inv_norm[u * sp.inv_row + r] = inv;
-        }
-    }
-    store_cols<T, D>(&red[grp][0], l, acc);
-    __syncthreads();
-    if (threadIdx.x < D) {
-        float s = 0.f;
-#pragma unroll 8
-        for (int q = 0; q < 32; ++q) s += red[q][threadIdx.x];
-        block_sums[((int64_t)u * sp.nblocks + t) * D + threadIdx.x] = s;
-    }
 }
 
 // anchor_means: block sums -> block means (in place), the stable mean (compensated sum over blocks) and the reciprocal
@@ -417,16 +362,6 @@ cudaError_t configure_scan_kernels() {
         else if ((dtype) == NKV_F32 && (d) == 128) { CALL(float, 128); } \
         else return cudaErrorInvalidValue;                             \
     } while (0)
-
-cudaError_t launch_anchor_sums(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
-                               float* inv_norm, cudaStream_t stream, int64_t* launches) {
-    const unsigned grid = (unsigned)sp.nblocks * (unsigned)(G * K.H);
-#define CALL(T, D) anchor_sums_kernel<T, D><<<grid, 256, 0, stream>>>(K, sp, block_sums, inv_norm)
-    NKV_DISPATCH(dtype, K.d, CALL);
-#undef CALL
-    ++*launches;
-    return cudaGetLastError();
-}
 
 cudaError_t launch_anchor_means(int units, int N, int d, const ScoreParams& sp, float* mu_e_inout, float* mu_s,
                                 float* inv_mu_e_norm_or_null, float* inv_mu_s_norm_or_null, cudaStream_t stream,

@@ -13,6 +13,8 @@
 // The sliding-window sum is a running sum over the 8 tokens of a group, seeded from exact sums of
 // 8-row segments, so no long prefix sum is ever differenced.  FP32 arithmetic uses the packed
 // two-wide fma/add forms of sm_100.
+#include <type_traits>
+
 #include "nkv_common.cuh"
 
 namespace nkv {
@@ -445,6 +447,77 @@ stream_a_kernel(TensorView K, ScoreParams sp, int units, float* __restrict__ blo
 }
 
 // ============================================================================================
+// anchor_sums: 1/||k_i|| and the sums of normalised keys of every episodic block, by themselves (staged calls, and block
+// sizes that the passes above do not take).  One CTA per (episodic block, head); a lane group takes four rows at a time, so
+// that a root and a division serve four rows (one at a time behind the last full round: blocks of 129 keys are common), and
+// keeps its running sum in registers.
+// Bound: DRAM and issue.  28 x 8 heads of 4133 x 128 bf16 keys (237 MB): 66 us with eight lanes per row, each of which worked
+// out every norm; 56 like this (36 at the copy rate).
+// ============================================================================================
+template <typename T, int D>
+__global__ void __launch_bounds__(256) anchor_sums_kernel(TensorView K, ScoreParams sp, float* __restrict__ block_sums,
+                                                          float* __restrict__ inv_norm) {
+    using G = Geo<T, D>;
+    constexpr int L = G::kLanes, kGroups = 256 / L;
+    __shared__ __align__(16) float red[kGroups][D];
+    pdl_wait();
+    const int u = blockIdx.x / sp.nblocks, t = blockIdx.x - u * sp.nblocks;
+    const int g = u / K.H, h = u % K.H;
+    const unsigned char* base =
+        reinterpret_cast<const unsigned char*>(K.ptr) + ((int64_t)g * K.stride_g + (int64_t)h * K.stride_h) * sizeof(T);
+    const int row0 = t * sp.block, row1 = min(K.N, row0 + sp.block);
+    const int grp = threadIdx.x / L, l = threadIdx.x % L;
+    F2 acc[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) acc[p] = pack2(0.f, 0.f);
+    auto rows = [&](auto count, int r) {   // `count` rows from r on
+        constexpr int C = decltype(count)::value, kApart = L / C;
+        F2 x[C][4];
+        float n2[C];
+#pragma unroll
+        for (int k = 0; k < C; ++k) {
+            if (r + k < row1) {
+                G::load_row(base + (int64_t)(r + k) * G::kRowBytes, l, x[k]);
+            } else {
+#pragma unroll
+                for (int p = 0; p < 4; ++p) x[k][p] = pack2(0.f, 0.f);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < C; ++k) {
+            F2 s = pack2(0.f, 0.f);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) s = fma2(x[k][p], x[k][p], s);
+            n2[k] = hsum2(s);
+        }
+        treduce<C, L>(n2, l);   // lane l has the squared norm of row l / kApart
+        const float inv = 1.0f / fmaxf(sqrtf(n2[0]), kEps);
+        const int mine = r + l / kApart;
+        if ((l & (kApart - 1)) == 0 && mine < row1) inv_norm[u * sp.inv_row + mine] = inv;
+#pragma unroll
+        for (int k = 0; k < C; ++k) {
+            const float ir = __shfl_sync(0xffffffffu, inv, k * kApart, L);
+            const F2 ir2 = pack2(ir, ir);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) acc[p] = fma2(x[k][p], ir2, acc[p]);
+        }
+    };
+    int first = row0;
+#pragma unroll 1
+    for (; row1 - first > 2 * kGroups; first += 4 * kGroups) rows(std::integral_constant<int, 4>{}, first + 4 * grp);
+#pragma unroll 1
+    for (; first < row1; first += kGroups) rows(std::integral_constant<int, 1>{}, first + grp);
+    G::store_vec(&red[grp][0], l, acc);
+    __syncthreads();
+    if (threadIdx.x < D) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q) s += red[q][threadIdx.x];
+        block_sums[((int64_t)u * sp.nblocks + t) * D + threadIdx.x] = s;
+    }
+}
+
+// ============================================================================================
 // stream_b
 // ============================================================================================
 template <typename T, int D, int TILE>
@@ -624,6 +697,24 @@ bool stream_path_supported(const ScoreParams& sp) { return sp.block % kSeg == 0;
         else if ((dtype) == NKV_F32 && (d) == 128) { CALL(float, 128); }     \
         else return cudaErrorInvalidValue;                                   \
     } while (0)
+
+cudaError_t launch_anchor_sums(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
+                               float* inv_norm, cudaStream_t stream, int64_t* launches) {
+    const unsigned grid = (unsigned)(G * K.H) * (unsigned)sp.nblocks;
+    ++*launches;
+#define NKV_SUMS(T, D) return launch_chained(anchor_sums_kernel<T, D>, grid, 256u, 0, stream, 1, K, sp, block_sums, inv_norm)
+    if (dtype == NKV_BF16) {
+        if (K.d == 128) NKV_SUMS(__nv_bfloat16, 128);
+        NKV_SUMS(__nv_bfloat16, 64);
+    }
+    if (dtype == NKV_F16) {
+        if (K.d == 128) NKV_SUMS(__half, 128);
+        NKV_SUMS(__half, 64);
+    }
+    if (K.d == 128) NKV_SUMS(float, 128);
+    NKV_SUMS(float, 64);
+#undef NKV_SUMS
+}
 
 cudaError_t launch_stream_a(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
                             float* inv_norm, float* a_raw, uint32_t* mm, int* status, int sm_count,
