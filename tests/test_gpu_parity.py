@@ -879,3 +879,28 @@ def test_block_sums_of_the_tensor_pass(N, d, layers):
     assert err.abs().max() <= 44 * 2.0 ** -24 * k.abs().max()
     assert err.square().mean().sqrt() <= 2e-7 * want.square().mean().sqrt()
     assert (mu_s.double() - k.mean(2)).abs().max() <= 44 * 2.0 ** -24 * k.abs().max()
+
+
+@pytest.mark.parametrize("layers,H,N,r,kind", [(1, 1, 130, 0.5, "plain"), (2, 3, 777, 0.5, "plain"), (1, 5, 2049, 0.75, "plain"),
+                                               (1, 33, 515, 0.85, "plain"), (1, 64, 300, 0.25, "plain"), (3, 8, 4097, 0.95, "plain"),
+                                               (1, 8, 6000, 0.75, "crowded"), (2, 7, 1030, 0.5, "equal"), (1, 4, 2500, 0.75, "short")])
+def test_fused_competition_matches_the_budget_call(layers, H, N, r, kind):
+    """The fused call takes the pool's bin from the histograms that the scores left; nkv_budget and nkv_select work on the
+    scores alone.  Same scores, same integers: heads in any number, bins that hold most scores, scores all equal, and a
+    head that only its safeguard keeps."""
+    K, V = _cache(N, 64, "bf16", H=H, layers=layers, seed=5 + N)
+    if kind == "crowded":
+        K = (K[:, :, :1] + 0.02 * K).contiguous()
+    elif kind == "equal":
+        K = K[:, :, :1].expand_as(K).contiguous()
+    elif kind == "short":
+        K[:, 1] = (K[:, 1, :1] + 0.001 * K[:, 1].float()).to(K.dtype)
+    p = nkv.nkv_default_params()
+    ws = nkv.alloc_workspace(K, p)
+    res = nkv.nkv_compress(K, V, r, p, ws=ws, want_a_star=True)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    budgets = nkv.nkv_budget(res.a_star, r, p)
+    idx, offs, _ = nkv.nkv_select(res.a_star, budgets, res.idx.shape[1])
+    assert torch.equal(res.budgets, budgets)
+    assert torch.equal(res.head_offsets, offs)
+    assert torch.equal(res.idx, idx)
