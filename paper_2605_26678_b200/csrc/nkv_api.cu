@@ -203,8 +203,8 @@ bool tensor_pays(const nkv_handle* h, const TensorView& kv, int G, const ScorePa
 // The second pass over the keys: a_s and a_e of every token from the anchors.
 int anchor_scores(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreParams& sp, const float* mu_s, const float* mu_e,
                   const float* inv_norm, const Bufs& B, float* a_raw, int* status, cudaStream_t st) {
-    const bool tensor = h->key_pass != NKV_KEY_PASS_FMA && anchor_dots_supported(kv, dtype, sp) &&
-                        tensor_pays(h, kv, G, sp, kv.d == 64 ? kSecondPassKb64 : kSecondPassKb128);
+    const bool tensor = h->key_pass != NKV_KEY_PASS_FMA && tensor_pays(h, kv, G, sp, kv.d == 64 ? kSecondPassKb64 : kSecondPassKb128) &&
+                        anchor_dots_supported(kv, dtype, sp);
     if (tensor)
         CU(launch_anchor_dots(kv, dtype, G, sp, mu_s, mu_e, inv_norm, B.inv_s, B.inv_e, a_raw, B.mm, status, h->sm_count, st,
                               &h->launches));
@@ -221,8 +221,9 @@ template <typename Mark>
 int key_scan(nkv_handle* h, const TensorView& kv, int dtype, int G, const ScoreParams& sp, const Bufs& B, int* status,
              cudaStream_t st, Mark&& mark) {
     const int units = G * kv.H, N = kv.N, d = kv.d;
-    const bool tensor_a = h->key_pass != NKV_KEY_PASS_FMA && gram_pass_supported(kv, dtype, sp) &&
-                          anchor_dots_supported(kv, dtype, sp) && tensor_pays(h, kv, G, sp, kFirstPassKb);
+    // (sizes first: the other two encode a tensor map to ask the driver, which a call that small does not need)
+    const bool tensor_a = h->key_pass != NKV_KEY_PASS_FMA && tensor_pays(h, kv, G, sp, kFirstPassKb) &&
+                          gram_pass_supported(kv, dtype, sp) && anchor_dots_supported(kv, dtype, sp);
     if (!tensor_a && !stream_path_supported(sp)) {
         CU(launch_anchor_sums(kv, dtype, G, sp, B.mu_e, B.inv_norm, st, &h->launches));
         CU(launch_anchor_means(units, N, d, sp, B.mu_e, B.mu_s, B.inv_e, B.inv_s, st, &h->launches));
