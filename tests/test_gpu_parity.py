@@ -940,3 +940,28 @@ def test_crowded_competition_again_and_again(layers, H, N):
                 own = oracle.budget_select(res.a_star[g].cpu().numpy(), r, pr.oracle_params(p))
                 assert np.array_equal(own.budgets, res.budgets[g].cpu().numpy()) and np.array_equal(own.idx, res.idx[g].cpu().numpy())
             assert 2 * int((res.budgets.min(1).values > nkv.nkv_safeguard_count(N, r, p)).sum()) > layers
+
+
+@pytest.mark.parametrize("G,H,N", [(1, 1, 700), (2, 2, 900), (1, 3, 700), (1, 5, 5000), (3, 8, 2049), (1, 8, 32768), (2, 12, 3001), (1, 64, 400)])
+def test_budget_of_heads_short_of_their_safeguard(G, H, N):
+    """Heads that come out short for certain (none of their scores reaches the bin of the last slot), that fall short by the
+    scores inside that bin, and that have just enough: budgets bit for bit."""
+    r = 0.75
+    rng = np.random.default_rng(N + H)
+    s = rng.random((G, H, N)).astype(np.float32)
+    n_safe = nkv.nkv_safeguard_count(N, r)
+    if H > 1:
+        s[:, 0] *= np.float32(0.25)               # nothing near the others' best
+        for h in range(1, H, 3):                  # its n_safe best, one more and one less, around the others' quarter
+            top = n_safe - 5 + (h // 3) % 3       # (and four sinks)
+            s[:, h] = np.float32(0.3) * rng.random((G, N)).astype(np.float32)
+            s[:, h, 5:5 + top] = np.float32(0.999)
+    s[:, :, :4] = np.inf
+    a_star = torch.from_numpy(s).to(DEV)
+    ws = torch.zeros(1 << 16, dtype=torch.uint8, device=DEV)
+    budgets = nkv.nkv_budget(a_star, r, ws=ws)
+    assert nkv.nkv_last_device_status(ws) == nkv.NKV_OK
+    for g in range(G):
+        assert np.array_equal(budgets[g].cpu().numpy(), _select_by_key(s[g], r, n_safe)[0])
+    if H > 3:   # (of fewer heads too many are low)
+        assert int(budgets[:, 0].max()) == n_safe
