@@ -701,19 +701,12 @@ bool stream_path_supported(const ScoreParams& sp) { return sp.block % kSeg == 0;
 cudaError_t launch_anchor_sums(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
                                float* inv_norm, cudaStream_t stream, int64_t* launches) {
     const unsigned grid = (unsigned)(G * K.H) * (unsigned)sp.nblocks;
+#define CALL(T, D) e = launch_chained(anchor_sums_kernel<T, D>, grid, 256u, 0, stream, 1, K, sp, block_sums, inv_norm)
+    cudaError_t e;
+    NKV_DISPATCH(dtype, K.d, CALL);
+#undef CALL
     ++*launches;
-#define NKV_SUMS(T, D) return launch_chained(anchor_sums_kernel<T, D>, grid, 256u, 0, stream, 1, K, sp, block_sums, inv_norm)
-    if (dtype == NKV_BF16) {
-        if (K.d == 128) NKV_SUMS(__nv_bfloat16, 128);
-        NKV_SUMS(__nv_bfloat16, 64);
-    }
-    if (dtype == NKV_F16) {
-        if (K.d == 128) NKV_SUMS(__half, 128);
-        NKV_SUMS(__half, 64);
-    }
-    if (K.d == 128) NKV_SUMS(float, 128);
-    NKV_SUMS(float, 64);
-#undef NKV_SUMS
+    return e;
 }
 
 cudaError_t launch_stream_a(const TensorView& K, int dtype, int G, const ScoreParams& sp, float* block_sums,
