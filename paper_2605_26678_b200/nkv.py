@@ -163,7 +163,7 @@ def _check(status: int, where: str) -> None:
 
 # Marshalling is most of what a small call costs the host (8 x 777 keys, nothing kept between calls: 60 us, 15 of them in the
 # library, beside 38 us on the device), so it goes by the cheaper of equal ways: strides in one tuple, addresses as
-# integers, the stream's address without a Stream object, outputs by new_empty.
+# integers, the stream's address without a Stream object, outputs by new_empty (where that is torch.empty: _maker).
 _DTYPE_CODES = {torch.bfloat16: NKV_BF16, torch.float32: NKV_F32, torch.float16: NKV_F16}
 
 
@@ -182,6 +182,14 @@ def _tensor(t: torch.Tensor) -> Tensor:
         raise NkvError(NKV_ERR_UNSUPPORTED, "d must be contiguous")
     G, H, N, d = t.shape
     return Tensor(t.data_ptr(), _dtype_code(t), 0, G, H, N, d, stride[0], stride[1], stride[2])
+
+
+def _maker(t: torch.Tensor):
+    """shape -> an empty tensor on t's device, of t's type if none is given.  A subclass's new_empty makes another of its
+    kind, and tensors with named dimensions refuse theirs."""
+    if type(t) is torch.Tensor and not t.has_names():
+        return t.new_empty
+    return lambda shape, dtype=t.dtype: torch.empty(shape, dtype=dtype, device=t.device)
 
 
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
@@ -244,7 +252,7 @@ def nkv_workspace_bytes(G: int, H: int, N: int, d: int, dtype: int, params: Opti
 def alloc_workspace(K: torch.Tensor, params: Optional[Params] = None, h: Optional[Handle] = None) -> torch.Tensor:
     G, H, N, d = K.shape
     n = nkv_workspace_bytes(G, H, N, d, _dtype_code(K), params, h)
-    return K.new_empty((n,), dtype=torch.uint8)
+    return _maker(K)((n,), dtype=torch.uint8)
 
 
 def nkv_anchors(K: torch.Tensor, params: Optional[Params] = None, want_mu_c: bool = False,
@@ -372,10 +380,10 @@ def alloc_outputs(K: torch.Tensor, V: torch.Tensor, r: float, want_a_star: bool 
     k = nkv_keep_per_head(N, r)
     if k < 1:
         raise NkvError(NKV_ERR_INVALID_ARG, "r leaves no token")
-    i32 = torch.int32
-    return Compressed(K.new_empty((G, H * k, d)), V.new_empty((G, H * k, V.shape[3])), K.new_empty((G, H * k), dtype=i32),
-                      K.new_empty((G, H + 1), dtype=i32), K.new_empty((G, H), dtype=i32),
-                      K.new_empty((G, H, N), dtype=torch.float32) if want_a_star else None)
+    i32, new = torch.int32, _maker(K)
+    return Compressed(new((G, H * k, d)), _maker(V)((G, H * k, V.shape[3])), new((G, H * k), dtype=i32),
+                      new((G, H + 1), dtype=i32), new((G, H), dtype=i32),
+                      new((G, H, N), dtype=torch.float32) if want_a_star else None)
 
 
 def nkv_compress(K: torch.Tensor, V: torch.Tensor, r: float, params: Optional[Params] = None,

@@ -965,3 +965,19 @@ def test_budget_of_heads_short_of_their_safeguard(G, H, N):
         assert np.array_equal(budgets[g].cpu().numpy(), _select_by_key(s[g], r, n_safe)[0])
     if H > 3:   # (of fewer heads too many are low)
         assert int(budgets[:, 0].max()) == n_safe
+
+
+class _Kind(torch.Tensor):
+    pass
+
+
+@pytest.mark.filterwarnings("ignore:Named tensors")
+def test_caches_of_a_subclass_and_with_named_dimensions():
+    K, V = _cache(300, 64, "bf16", H=3)
+    want = nkv.nkv_compress(K, V, 0.5)
+    names = ("g", "h", "n", "d")
+    for k, v in ((K.as_subclass(_Kind), V.as_subclass(_Kind)), (K.refine_names(*names), V.refine_names(*names))):
+        got = nkv.nkv_compress(k, v, 0.5)
+        for name in ("k_out", "v_out", "idx", "head_offsets", "budgets"):
+            t = getattr(got, name)
+            assert type(t) is torch.Tensor and torch.equal(t, getattr(want, name))

@@ -4,6 +4,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2605_26678_b200 import build as nkv_build
 from paper_2605_26678_b200 import nkv
@@ -58,8 +59,30 @@ def test_defaults_and_derived_sizes(lib):
 
 
 def test_no_cpu_fallback():
-    import torch
     if torch.cuda.is_available():
         pytest.skip("a GPU is present")
     with pytest.raises(nkv.NkvUnavailable):
         nkv.Handle(0)
+
+
+class _Kind(torch.Tensor):
+    pass
+
+
+@pytest.mark.filterwarnings("ignore:Named tensors")
+@pytest.mark.parametrize("kind", ["plain", "subclass", "named", "parameter"])
+def test_outputs_are_plain_tensors_whatever_the_cache_is(lib, kind):
+    K, V = torch.zeros((2, 3, 40, 64), dtype=torch.bfloat16), torch.zeros((2, 3, 40, 64), dtype=torch.float32)
+    if kind == "subclass":
+        K, V = K.as_subclass(_Kind), V.as_subclass(_Kind)
+    elif kind == "named":
+        K, V = K.refine_names("g", "h", "n", "d"), V.refine_names("g", "h", "n", "d")
+    elif kind == "parameter":
+        K, V = torch.nn.Parameter(K), torch.nn.Parameter(V)
+    o = nkv.alloc_outputs(K, V, 0.5, want_a_star=True)
+    want = {"k_out": ((2, 60, 64), torch.bfloat16), "v_out": ((2, 60, 64), torch.float32), "idx": ((2, 60), torch.int32),
+            "head_offsets": ((2, 4), torch.int32), "budgets": ((2, 3), torch.int32), "a_star": ((2, 3, 40), torch.float32)}
+    for name, (shape, dtype) in want.items():
+        t = getattr(o, name)
+        assert type(t) is torch.Tensor and not t.has_names() and not t.requires_grad
+        assert tuple(t.shape) == shape and t.dtype == dtype and t.device == K.device
