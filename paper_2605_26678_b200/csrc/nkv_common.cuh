@@ -183,7 +183,7 @@ cudaError_t launch_budget(int G, int H, int N, int keep, int n_safe, const float
                           float* thresholds_opt, int* status, cudaStream_t stream, int64_t* launches);
 cudaError_t launch_select(int G, int H, int N, int64_t idx_capacity, const float* a_star, const int32_t* budgets,
                           int32_t* idx, int32_t* head_offsets, int* status, cudaStream_t stream, int64_t* launches);
-// the three in one or two launches; rows of a_star are star_row floats apart; hist: scratch of score_hist_bytes
+// the three in two launches; rows of a_star are star_row floats apart; hist: scratch of score_hist_bytes
 size_t score_hist_bytes(int64_t units);
 cudaError_t launch_score_to_select(int G, int H, int N, const ScoreParams& sp, int keep, int n_safe, const float* a_raw,
                                    const uint32_t* minmax_keys, float* a_star, int64_t star_row, int* hist, int32_t* budgets, int32_t* idx,

@@ -16,7 +16,7 @@
 //
 // Keys are staged by TMA (128-byte swizzle, 64-column halves) in a ring of 128-row stages; the 64 rows in front of
 // stage 0 hold a second copy of the last stage's second half, so the 64 rows before a tile always lie in front of
-// it.  For tile n the MMA thread forms D = K[tile] x K[64 rows before the tile .. tile]^T (128 x 192, fp32 in tensor
+// it.  For tile n the MMA warp forms D = K[tile] x K[64 rows before the tile .. tile]^T (128 x 192, fp32 in tensor
 // memory, double buffered, one N = 192 product per 16-wide K step).  The diagonal of D holds ||k||^2 of the
 // tile's rows, so the norms cost no pass over the key values.  Row r of D holds the 64 entries of the backward band
 // ending at its diagonal.  Their row sums give

@@ -519,7 +519,7 @@ def test_budget_and_select_in_every_layout(G, H, N, r, ties):
 @pytest.mark.gpu
 @pytest.mark.parametrize("layers,H,N,d", [(40, 8, 701, 64), (20, 12, 1100, 64), (2, 8, 30011, 64), (37, 4, 5000, 64)])
 def test_score_to_select_in_every_layout(layers, H, N, d):
-    """The score side of the fused call in one launch and in two, one head per CTA and several."""
+    """The score side of the fused call, one head per CTA and several."""
     K, V = _cache(N, d, "bf16", H=H, layers=layers)
     p = nkv.nkv_default_params()
     ws = nkv.alloc_workspace(K, p)
@@ -538,7 +538,7 @@ def test_score_to_select_in_every_layout(layers, H, N, d):
 @pytest.mark.parametrize("safeguard", [0.0, 0.9, 1.0])
 @pytest.mark.parametrize("layers,H,N", [(3, 8, 701), (2, 3, 30011), (30, 12, 900)])
 def test_safeguard_that_no_head_and_some_head_needs(layers, H, N, safeguard):
-    """Heads that compete once, and twice because one came out short of its safeguard; scores of one launch and of two."""
+    """Heads that compete once, and twice because one came out short of its safeguard."""
     K, V = _cache(N, 64, "bf16", H=H, layers=layers)
     p = nkv.nkv_default_params()
     p.safeguard = safeguard
