@@ -39,12 +39,16 @@
 // Groups hand work to each other through mbarriers; every wait is bounded and a group that gives up
 // records where and leaves, which makes the others give up in turn.
 //
-// Bound: the hand-over chain of a tile (accumulator freed, product issued, product done, norms, band loaded: two tiles in
-// flight) and the issue of the Gram products by one warp; DRAM is the floor.  What moved it last: with the block sums on
-// the FMA pipes a tile of 128 x 128 took 4981 warp instructions, a third of them for these; on the tensor cores it takes
-// 3290, and the 16 warps left have 128 registers each, with which a band warp takes the whole band out of tensor memory
-// before it works on it.  36 x 8 heads of 8192 x 128 bf16 keys: 155 -> 132 us (93 at the copy rate); 16 x 8 x 32768 x 64: 222
-// -> 183.
+// Bound, by clocks read in the roles.  d = 128: the warp that issues the Gram products, 1340 to 1490 cycles a tile.  It is hardly ever
+// idle: 550 for the products, 180 for the commit, 300 to 500 for looks at barriers whose phase is complete (keys were there at every
+// look, so memory is not waited for); the band groups are busy for 2550 of the 2900 cycles that each has for a tile.
+// At 1965 MHz that would be the copy rate, but the SMs do not keep that clock under the load of this pass: clock and time
+// counters over the same tiles give 1650 to 1710 MHz in a call of 110 us and 1460 to 1480 in one of 2 ms.  36 x 8 heads of 8192 x
+// 128 bf16 keys with the anchors' means 130 us (93 at the copy rate), 144 x 8 x 32768 x 128 2.04 ms (1.48).  d = 64: the band
+// groups, 2400 of 2530 cycles; 16 x 8 x 32768 x 64 179 us (82), at 1735 to 1785 MHz.
+// What moved it last: with the block sums on the FMA pipes a tile of 128 x 128 took 4981 warp instructions, a third of
+// them for these; on the tensor cores it takes 3290, and the 16 warps left have 128 registers each, with which a band warp
+// takes the whole band out of tensor memory before it works on it: 155 -> 132 us and 222 -> 183.
 #include <type_traits>
 
 #include "nkv_sm100.cuh"
