@@ -46,8 +46,8 @@
 // counters over the same tiles give 1650 to 1710 MHz in a call of 110 us and 1460 to 1480 in one of 2 ms.  36 x 8 heads of 8192 x
 // 128 bf16 keys with the anchors' means 130 us (93 at the copy rate), 144 x 8 x 32768 x 128 2.04 ms (1.48).  d = 64: the band
 // groups, 2400 of 2530 cycles; 16 x 8 x 32768 x 64 179 us (82), at 1735 to 1785 MHz.
-// What moved it last: with the block sums on the FMA pipes a tile of 128 x 128 took 4981 warp instructions, a third of
-// them for these; on the tensor cores it takes 3290, and the 16 warps left have 128 registers each, with which a band warp
+// What moved it last: with the block sums on the FMA pipes 128 keys took 4960 warp instructions, a third of
+// them for these; on the tensor cores 3265, and the 16 warps left have 128 registers each, with which a band warp
 // takes the whole band out of tensor memory before it works on it: 155 -> 132 us and 222 -> 183.
 #include <type_traits>
 
